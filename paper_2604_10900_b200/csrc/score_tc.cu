@@ -153,12 +153,6 @@ __device__ __forceinline__ float4 lds_f4(uint32_t a) {
     return r;
 }
 
-__device__ __forceinline__ uint64_t lds_u64(uint32_t a) {
-    uint64_t r;
-    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(r) : "r"(a));
-    return r;
-}
-
 // Sum of the n <= 4 partial key sums of one key (one per epilogue group and column half, 128 floats apart), added in
 // that order; the four reads are independent shared-space loads, so the fold costs one latency and not four.
 __device__ __forceinline__ float fold_partials(const float* p, int n) {
@@ -174,69 +168,48 @@ __device__ __forceinline__ float fold_partials(const float* p, int n) {
     return acc;
 }
 
-// ---- the masked form of a tile: chunks of 16 accumulator columns, bit x of `vis` = this thread's row sees column x ----------------
+// ---- the masked form of a tile: bit x of `vis` = this thread's row sees column x of the block -------------------------------------
 // One small rolled body for every tile that is not streamed (the causal diagonal, the ends of a unit, ragged columns): written out
 // per block and per case it is 11 KB of instructions that each of sixteen warps fetches once a segment, and a causal tile
 // took longer than a full one; leaving out blocks nobody sees in that form made it slower still, by the second case's code.
-// (3,072 units of 640 rows, one tile of five causal: normaliser pass 370 to 337 us, score pass 350 to 344.)
-__device__ __forceinline__ unsigned low_bits(int n) { return n >= 16 ? 0xFFFFu : n <= 0 ? 0u : (1u << n) - 1u; }
+// The order of the additions is that of 32-column blocks (four sums over every fourth column, added up per block; the normaliser's
+// block moves its reference to its own greatest column first and adds column by column).  It is kept because rows whose scores
+// agree to 1e-7 at a selection boundary are told apart by it.  (3,072 units of 640 rows, one tile of five causal: 339 and 337 us
+// a pass; with the sums of 16-column chunks, in another order, 316 and 318.)
+__device__ __forceinline__ unsigned low_bits(int n) { return n >= 32 ? ~0u : n <= 0 ? 0u : (1u << n) - 1u; }
 
-// Pass S: adds sum_r 2^(y_r*scale2 + nc[r]) over the visible rows (columns) r of the chunk to the packed partial sums.
-template <int PAIRS>
-__device__ __forceinline__ void mass_chunk(const float (&v)[16], uint32_t nc32, unsigned vis, float scale2, uint64_t& a01, uint64_t& a23) {
+// Pass S: adds sum_r 2^(y_r*scale2 + nc[r]) over the visible rows (columns) r of a 32-column block to the packed partial sums.
+__device__ __forceinline__ void mass_block(const float (&v)[32], uint32_t nc32, unsigned vis, float scale2, uint64_t& a01) {
     const uint64_t s2 = pack2(scale2, scale2);
     float b[4] = {0.f, 0.f, 0.f, 0.f};
-    if (PAIRS == 8) {
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const float4 c4 = lds_f4(nc32 + 16u * x);
-            float t0, t1, t2, t3;
-            unpack2(fma2(pack2(v[4 * x], v[4 * x + 1]), s2, pack2(c4.x, c4.y)), t0, t1);
-            unpack2(fma2(pack2(v[4 * x + 2], v[4 * x + 3]), s2, pack2(c4.z, c4.w)), t2, t3);
-            if (vis & (1u << (4 * x))) b[0] += ex2(t0);
-            if (vis & (2u << (4 * x))) b[1] += ex2(t1);
-            if (vis & (4u << (4 * x))) b[2] += ex2(t2);
-            if (vis & (8u << (4 * x))) b[3] += ex2(t3);
-        }
-    } else
-#pragma unroll
-    for (int x = 0; x < PAIRS; ++x) {
-        float t0, t1;
-        unpack2(fma2(pack2(v[2 * x], v[2 * x + 1]), s2, lds_u64(nc32 + 8u * x)), t0, t1);
-        if (vis & (1u << (2 * x))) b[2 * (x & 1)] += ex2(t0);
-        if (vis & (2u << (2 * x))) b[2 * (x & 1) + 1] += ex2(t1);
+    for (int x = 0; x < 8; ++x) {
+        const float4 c4 = lds_f4(nc32 + 16u * x);
+        float t0, t1, t2, t3;
+        unpack2(fma2(pack2(v[4 * x], v[4 * x + 1]), s2, pack2(c4.x, c4.y)), t0, t1);
+        unpack2(fma2(pack2(v[4 * x + 2], v[4 * x + 3]), s2, pack2(c4.z, c4.w)), t2, t3);
+        if (vis & (1u << (4 * x))) b[0] += ex2(t0);
+        if (vis & (2u << (4 * x))) b[1] += ex2(t1);
+        if (vis & (4u << (4 * x))) b[2] += ex2(t2);
+        if (vis & (8u << (4 * x))) b[3] += ex2(t3);
     }
-    a01 = add2(a01, pack2(b[0], b[1]));
-    a23 = add2(a23, pack2(b[2], b[3]));
+    a01 = add2(a01, pack2((b[0] + b[1]) + (b[2] + b[3]), 0.f));
 }
 
-// Pass N: folds the visible columns of the chunk into the running (reference, sum of 2^(y*scale2 - reference)).
-__device__ __forceinline__ void norm_chunk(const float (&v)[16], unsigned vis, float scale2, float& mref, float& lr) {
-    auto sum = [&]() {
-        float b[4] = {0.f, 0.f, 0.f, 0.f};
+// Pass N: folds the visible columns of a 32-column block into the running (reference, sum of 2^(y*scale2 - reference)).
+__device__ __forceinline__ void norm_block(const float (&v)[32], unsigned vis, float scale2, float& mref, float& lr) {
+    float cm = kNegBig;
 #pragma unroll
-        for (int x = 0; x < 16; ++x)
-            if (vis & (1u << x)) b[x & 3] += ex2(fmaf(v[x], scale2, -mref));
-        return (b[0] + b[1]) + (b[2] + b[3]);
-    };
-    float lb = sum();
-    if (__any_sync(0xffffffffu, !(lb <= 65536.f))) {
-        // some column exceeds its row's reference by more than 16, or the reference is still unset: those rows move it to the
-        // greatest visible column and sum again
-        const bool redo = !(lb <= 65536.f);
-        float cm = kNegBig;
-#pragma unroll
-        for (int x = 0; x < 16; ++x)
-            if (vis & (1u << x)) cm = fmaxf(cm, v[x]);
-        cm *= scale2;
-        if (redo && cm > mref) {
-            lr *= ex2(mref - cm);
-            mref = cm;
-        }
-        const float l2 = sum();
-        if (redo) lb = l2;
+    for (int x = 0; x < 32; ++x)
+        if (vis & (1u << x)) cm = fmaxf(cm, v[x]);
+    cm *= scale2;
+    if (vis && cm > mref) {
+        lr *= ex2(mref - cm);
+        mref = cm;
     }
-    lr += lb;
+#pragma unroll
+    for (int x = 0; x < 32; ++x)
+        if (vis & (1u << x)) lr += ex2(fmaf(v[x], scale2, -mref));
 }
 
 // Walks this CTA's contiguous range of key tiles, segment by segment (a segment: tiles of one row group of one unit).  The
@@ -344,7 +317,7 @@ __device__ __forceinline__ void make_row_table(int u, int rg, int lo, int cnt, b
         for (int r = idx; r < limit; r += n) {
             if (r >= rows) { rc[r] = -1.0e30f; continue; }
             const float lse = lse_in[ou + r];
-            rc[r] = log2f(inv_rows) - lse * kLog2e;
+            rc[r] = log2f(inv_rows) - __fmul_rn(lse, kLog2e);      // (rounded twice, as a stored rowm is)
             if (lse_out && first) lse_out[ou + r] = lse;
         }
         return;
@@ -500,12 +473,7 @@ __device__ __noinline__ void produce_paged_call(const CUtensorMap* tmK, const CU
 // that the compiler knows the numbers of 64-channel halves, contraction steps and row groups.  (The general form of the
 // code costs those shapes 1 to 3 %: branches between the issuer's instructions, registers spilled in the epilogue.)
 // SPLIT: fp32 caches; PLAIN is then about the head_dim only.
-// PAIRS (score pass, NB = 4): pairs of query columns per chunk of the epilogue, 16 * PAIRS query rows per slot.  257 to 448 rows are
-// spread evenly over the four slots (80, 96 or 112 each), so that every warp does the same and no exponential is evaluated for
-// a row that is not there: with whole blocks, 448 rows left one slot of four half empty (112 units of 13,312 rows, score pass
-// 208 to 198 us; of 8,448 rows 133 to 127).  The normaliser pass
-// holds rows in lanes, where a partly filled block saves nothing.
-template <int PASS, int NB, bool PLAIN, bool SPLIT, int PAIRS>
+template <int PASS, int NB, bool PLAIN, bool SPLIT>
 __global__ void __launch_bounds__(kThreadsTc, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ,
                 const UnitDesc* __restrict__ desc, Shape sh, RowGroups rgs, float scale2, int total_tiles, int sub_rows,
@@ -514,8 +482,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 const __grid_constant__ RowDefaults fill, int32_t* __restrict__ err) {
     using C = Cfg<NB, SPLIT>;
     constexpr int kStages = C::kStages, kTps = C::kTps;
-    static_assert(PAIRS == 8 || (PASS == 1 && NB == 4 && !SPLIT), "uneven chunks: score pass only");
-    constexpr int kRows = 16 * PAIRS, kCols = 2 * PAIRS;     // query rows per slot, columns per chunk
+    constexpr int kRows = 128;                               // query rows per slot
     constexpr uint32_t kQRegionBytes = C::kQRegionBytes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -730,8 +697,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                         ++use[p];
                         tc_fence_after();
                         const uint32_t qblk_lo = q_lo + (((b >> 1) * 2 * kQRegionBytes + (b & 1) * (128 * 128)) >> 4);
-                        // (a row past the group's own is one of the next group or a zero, and has no weight)
-                        const uint32_t idesc = umma_idesc(kRows);
+                        // (a row past the group's own is one of the next group or a zero, and has no weight; pass S reads no
+                        // more than the first half of a block with 64 rows or fewer)
+                        const uint32_t idesc = umma_idesc(PASS == 1 && rgs.per - kRows * b <= 64 ? 64 : 128);
                         if (PASS == 1) tc_mma_lo<false>(tmem_base + 128 * j, kst_lo, qblk_lo, idesc);
                         else tc_mma_lo<false>(tmem_base + 128 * j, qblk_lo, kst_lo, idesc);
 #pragma unroll
@@ -792,7 +760,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         const int ch = (ew >> 2) & 1;            // which 64 columns of a slot
         const int g = ew >> 3;                   // group: drains slots g and g + 2 in turn
         const int etid = ew * 32 + lane;
-        const uint32_t taddr = tmem_base + ((uint32_t)(32 * qd) << 16) + (kRows / 2) * ch;
+        const uint32_t taddr = tmem_base + ((uint32_t)(32 * qd) << 16) + 64 * ch;
         constexpr int kStates = NB == 4 ? 2 : 1;
         const int j0 = g, j1 = g + 2;            // this group's slots
         const int b0 = j0 % NB, b1 = j1 % NB;    // the query blocks in them
@@ -845,11 +813,15 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             }
             const int key_begin = wk.key_begin();
             const int nt = wk.seg_tiles();
-            // The columns of its two slots this warp reads: half of each.  (NB < 4, pass S: a ragged last block has fewer; a
+            // The columns of its two slots this warp reads: half of each.  (Pass S: a ragged last block has fewer; a
             // half-filled 64 goes the streamed way whole, its spare columns hold other rows or zeros, without weight.)
-            const int cend0 = PASS == 1 && NB < 4 ? min(64, rgs.per - 128 * b0 - 64 * ch) : 8 * PAIRS;
-            const int cend1 = PASS == 1 && NB < 4 ? min(64, rgs.per - 128 * b1 - 64 * ch) : 8 * PAIRS;
-            const bool full_cols = NB == 4 ? kRows * b1 < rgs.per : 128 * b0 < rgs.per && (PASS == 0 || cend0 > 32);
+            const int cend0 = PASS == 1 ? min(64, rgs.per - 128 * b0 - 64 * ch) : 64;
+            const int cend1 = PASS == 1 ? min(64, rgs.per - 128 * b1 - 64 * ch) : 64;
+            const bool full_cols = NB == 4 || (128 * b0 < rgs.per && (PASS == 0 || cend0 > 32));
+            // NB = 4: does this warp read the group's second slot?  Up to 384 rows leave the fourth slot unused, up to 448 its second
+            // half, and pass S then evaluates no exponential of it.  (448 rows spread over the four slots, 112 in each, keep the
+            // two groups equally busy, 112 units of 13,312 rows 194 against 197 us, but add a key's terms in another order.)
+            const bool slot1 = NB < 4 || 128 * b1 < rgs.per, second = slot1 && (NB < 4 || cend1 > 0);
             const int row0 = 128 * b0 + ((32 * qd + block_turn<PASS, NB>(b0)) & 127) + lane;   // pass N, in the row group
             const int row1 = 128 * b1 + ((32 * qd + block_turn<PASS, NB>(b1)) & 127) + lane;
             const int lastvis0 = (row0 < rows_g) ? (sh.causal ? T - sh.W + ((rg0 + row0) % sh.W) : T - 1) : -1;
@@ -862,6 +834,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
                 for (int p = 0; p < kStates; ++p) {
                     const int j = p ? j1 : j0;
+                    if (p == 1 && !second) break;
                     ok = mbar_wait<true>(&bar.d_full[j], uses(p) & 1u, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
@@ -897,22 +870,17 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     tc_wait_ld_regs(v);
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        const int p = c >> 2, j = p ? j1 : j0, col = kCols * (c & 3);
+                        const int p = c >> 2, j = p ? j1 : j0, col = 16 * (c & 3);
                         const int ps = NB == 4 ? p : 0;          // pass N: the row state of the slot
                         const int pa = NB == 4 ? 0 : p;          // pass S: the key sums of the slot
                         uint64_t t2[8];
                         if (PASS == 1) {
-                            const uint32_t nc32 = smem_u32(&rc[kRows * (p ? b1 : b0) + 8 * PAIRS * ch + col]);
+                            const uint32_t nc32 = smem_u32(&rc[kRows * (p ? b1 : b0) + 64 * ch + col]);
 #pragma unroll
-                            for (int x = 0; x < PAIRS; ++x) {
-                                if (PAIRS == 8) {
-                                    if (x & 1) continue;
-                                    const float4 c4 = lds_f4(nc32 + 8u * x);
-                                    t2[x] = fma2(pack2(v[2 * x], v[2 * x + 1]), s2, pack2(c4.x, c4.y));
-                                    t2[x + 1] = fma2(pack2(v[2 * x + 2], v[2 * x + 3]), s2, pack2(c4.z, c4.w));
-                                } else {
-                                    t2[x] = fma2(pack2(v[2 * x], v[2 * x + 1]), s2, lds_u64(nc32 + 8u * x));
-                                }
+                            for (int x = 0; x < 4; ++x) {
+                                const float4 c4 = lds_f4(nc32 + 16u * x);
+                                t2[2 * x] = fma2(pack2(v[4 * x], v[4 * x + 1]), s2, pack2(c4.x, c4.y));
+                                t2[2 * x + 1] = fma2(pack2(v[4 * x + 2], v[4 * x + 3]), s2, pack2(c4.z, c4.w));
                             }
                         } else {
                             const uint64_t nm2 = pack2(-mm[ps], -mm[ps]);
@@ -924,18 +892,18 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                             __syncwarp();
                             if (lane == 0) mbar_arrive(&bar.d_empty[j]);
                         }
-                        if (c == 3) {
+                        if (c == 3 && second) {
                             ok = mbar_wait<true>(&bar.d_full[j1], uses(1) & 1u, abort_flag);
                             if (!ok) break;
                             tc_fence_after();
                         }
-                        if (c < 7) tc_ld16(taddr + 128 * (((c + 1) >> 2) ? j1 : j0) + kCols * ((c + 1) & 3), v);
+                        if (c < 7 && (c != 3 || second)) tc_ld16(taddr + 128 * (((c + 1) >> 2) ? j1 : j0) + 16 * ((c + 1) & 3), v);
                         if (PASS == 1) {
 #pragma unroll
-                            for (int x = 0; x < PAIRS; ++x) {
+                            for (int x = 0; x < 8; ++x) {
                                 float t0_, t1_;
                                 unpack2(t2[x], t0_, t1_);
-                                const uint64_t e2 = x == PAIRS - 1
+                                const uint64_t e2 = x == 7
                                                         ? ex2_poly2(pack2(fmaxf(t0_, -125.f), fmaxf(t1_, -125.f)))
                                                         : pack2(ex2(t0_), ex2(t1_));
                                 if (x & 1) a23[pa] = add2(a23[pa], e2); else a01[pa] = add2(a01[pa], e2);
@@ -999,9 +967,15 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                                 if (lane == 0) mbar_arrive(&bar.d_empty[j]);
                             }
                         }
+                        if (c == 3 && !second) break;
                         if (c < 7) tc_wait_ld_regs(v);
                     }
                     if (!ok) break;
+                    if (PASS == 1 && NB == 4 && slot1 && !second) {       // the slot is the other column half's alone
+                        ok = mbar_wait<true>(&bar.d_full[j1], uses(1) & 1u, abort_flag);
+                        if (!ok) break;
+                        if (lane == 0) mbar_arrive(&bar.d_empty[j1]);
+                    }
                     ++use[0];
                     ++use[1];
                 } else {
@@ -1019,42 +993,40 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                         const int jmin = ktile + 32 * qd + lane - (T - sh.W);     // pass S: first window position that sees the thread's key
                         const int nvis = (p ? lastvis1 : lastvis0) - (ktile + 64 * ch) + 1;   // pass N: columns of this warp the row sees
                         float mref = NB == 4 && p ? mm[kStates - 1] : mm[0], lr = NB == 4 && p ? l_run[kStates - 1] : l_run[0];
-                        uint64_t s01 = 0ull, s23 = 0ull;
+                        uint64_t s01 = NB == 4 ? a01[0] : 0ull;
 #pragma unroll 1
-                        for (int cc = 0; cc < cend; cc += kCols) {
-                            const int r0 = kRows * (p ? b1 : b0) + 8 * PAIRS * ch + cc;       // pass S: first query row of the chunk
-                            unsigned vis = (1u << kCols) - 1u;
+                        for (int cc = 0; cc < cend; cc += 32) {           // (cend is a multiple of 32)
+                            const int r0 = kRows * (p ? b1 : b0) + 64 * ch + cc;              // pass S: first query row of the block
+                            unsigned vis = ~0u;
                             if (PASS == 0) {
                                 vis = low_bits(nvis - cc);
                             } else if (!tfast && sh.causal) {
                                 // window position of the first column, and columns up to the next head's first
                                 int pos = (rg0 + r0) % sh.W;
-                                const int wrap = sh.W - pos;
-                                if (PAIRS == 8 && (sh.W & 15) == 0) {
-                                    vis &= ~low_bits(jmin - pos);            // the chunk lies inside one head
-                                } else if (PAIRS < 8 && sh.W >= kCols) {
-                                    vis &= (low_bits(wrap) & ~low_bits(jmin - pos)) | (~low_bits(wrap) & ~low_bits(jmin + wrap));
+                                if ((sh.W & 15) == 0) {                   // each half of the block lies inside one head
+                                    const int pos1 = pos + 16 == sh.W ? 0 : pos + 16;
+                                    vis = (~low_bits(jmin - pos) & 0xFFFFu) | (~low_bits(jmin - pos1) << 16);
                                 } else {
                                     vis = 0u;
-                                    for (int x = 0; x < kCols; ++x) {
+                                    for (int x = 0; x < 32; ++x) {
                                         vis |= (pos >= jmin ? 1u : 0u) << x;
                                         if (++pos == sh.W) pos = 0;
                                     }
                                 }
                             }
-                            if (!__any_sync(0xffffffffu, vis)) continue;                      // nothing in the warp sees the chunk
-                            float v[16];
-                            tc_ld16(taddr + 128 * j + cc, v);
+                            if (!__any_sync(0xffffffffu, vis)) continue;                      // nothing in the warp sees the block
+                            float v[32];
+                            tc_ld32(taddr + 128 * j + cc, v);
                             tc_wait_ld_regs(v);
-                            if (PASS == 1) mass_chunk<PAIRS>(v, smem_u32(&rc[r0]), vis, scale2, s01, s23);
-                            else norm_chunk(v, vis, scale2, mref, lr);
+                            if (PASS == 1) mass_block(v, smem_u32(&rc[r0]), vis, scale2, s01);
+                            else norm_block(v, vis, scale2, mref, lr);
                         }
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&bar.d_empty[j]);
                         if (PASS == 1) {
-                            if (NB == 4 || p == 0) { a01[0] = add2(a01[0], s01); a23[0] = add2(a23[0], s23); }
-                            else { a01[2 - kStates] = s01; a23[2 - kStates] = s23; }
+                            if (NB == 4 || p == 0) a01[0] = s01;
+                            else a01[2 - kStates] = s01;
                         } else if (NB == 4 && p) {
                             mm[kStates - 1] = mref; l_run[kStates - 1] = lr;
                         } else {
@@ -1230,7 +1202,7 @@ bool score_tc_supported(const Launch& L) {
 }
 
 namespace {
-template <int NB, bool PLAIN, bool SPLIT, int PAIRS>
+template <int NB, bool PLAIN, bool SPLIT>
 cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMap& tmK, const CUtensorMap& tmQ, int sub_rows,
                           const float* lse_in, float* s, float* lse_out, Workspace& ws) {
     const Shape& sh = L.sh;
@@ -1238,7 +1210,7 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     const int grid = std::max(1, std::min(std::min(L.sms > 0 ? L.sms : 128, kMaxSms), total));
     constexpr size_t smem = smem_bytes<NB, SPLIT>();
     const float scale2 = kLog2e * (float)(1.0 / std::sqrt((double)sh.d));      // logits in log2 units
-    const auto norm = score_tc_kernel<0, NB, PLAIN, SPLIT, 8>, mass = score_tc_kernel<1, NB, PLAIN, SPLIT, PAIRS>;
+    const auto norm = score_tc_kernel<0, NB, PLAIN, SPLIT>, mass = score_tc_kernel<1, NB, PLAIN, SPLIT>;
     // Whether a pass may start while the kernel before it still runs (launch_dependent).  Its warps then take the slots that kernel's
     // leave, and where those are not the first ones of the SM the CTA runs up to 8 % slower, tile for tile, from the first to the
     // last: with the score pass of 288 units of 33,280 rows, a third of the CTAs (pass 1,260 to 1,360 us).  So a pass starts early
@@ -1248,7 +1220,7 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     // its way, below 256 (288 units of 33,280 rows 3,603 and 3,574; 112 of 8,448 399.5 and 403.5).
     const int bit = kSmemBitScore + 2 * (NB >> 1) + 6 * PLAIN + 12 * SPLIT;
     cudaError_t e = lse_in ? cudaSuccess : allow_smem(L, bit, norm, smem);
-    if (e == cudaSuccess) e = allow_smem(L, PAIRS == 8 ? bit + 1 : kSmemBitScore + 20 + PAIRS - 5 + 3 * PLAIN, mass, smem);
+    if (e == cudaSuccess) e = allow_smem(L, bit + 1, mass, smem);
     if (e == cudaSuccess && !lse_in) {
         Timed t(L, KID_SCORE_NORM);
         e = launch_kernel(total < 256 * grid, L.stream, norm, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
@@ -1306,22 +1278,13 @@ cudaError_t launch_score_tc(const Launch& L, const float* lse_in, float* s, floa
             return cudaErrorInvalidValue;
     }
     if (split)
-        return sh.d > 112 ? launch_passes<1, true, true, 8>(L, pl.rg, tmK, tmQ, sub_rows, lse_in, s, lse_out, ws)
-                          : launch_passes<1, false, true, 8>(L, pl.rg, tmK, tmQ, sub_rows, lse_in, s, lse_out, ws);
-    auto go = [&](auto nb, auto pairs, auto plain) {
-        return launch_passes<decltype(nb)::value, decltype(plain)::value, false, decltype(pairs)::value>(L, pl.rg, tmK, tmQ, sub_rows,
-                                                                                                         lse_in, s, lse_out, ws);
-    };
-    using std::integral_constant;
+        return sh.d > 112 ? launch_passes<1, true, true>(L, pl.rg, tmK, tmQ, sub_rows, lse_in, s, lse_out, ws)
+                          : launch_passes<1, false, true>(L, pl.rg, tmK, tmQ, sub_rows, lse_in, s, lse_out, ws);
     auto go_nb = [&](auto plain) {
-        if (pl.nb == 2) return go(integral_constant<int, 2>{}, integral_constant<int, 8>{}, plain);
-        if (pl.nb == 1) return go(integral_constant<int, 1>{}, integral_constant<int, 8>{}, plain);
-        switch ((pl.rg.per + 63) / 64) {
-            case 5: return go(integral_constant<int, 4>{}, integral_constant<int, 5>{}, plain);
-            case 6: return go(integral_constant<int, 4>{}, integral_constant<int, 6>{}, plain);
-            case 7: return go(integral_constant<int, 4>{}, integral_constant<int, 7>{}, plain);
-            default: return go(integral_constant<int, 4>{}, integral_constant<int, 8>{}, plain);
-        }
+        constexpr bool kPlain = decltype(plain)::value;
+        if (pl.nb == 2) return launch_passes<2, kPlain, false>(L, pl.rg, tmK, tmQ, sub_rows, lse_in, s, lse_out, ws);
+        if (pl.nb == 1) return launch_passes<1, kPlain, false>(L, pl.rg, tmK, tmQ, sub_rows, lse_in, s, lse_out, ws);
+        return launch_passes<4, kPlain, false>(L, pl.rg, tmK, tmQ, sub_rows, lse_in, s, lse_out, ws);
     };
     return sh.d > 112 && pl.rg.groups == 1 ? go_nb(std::true_type{}) : go_nb(std::false_type{});
 }
