@@ -494,8 +494,12 @@ __device__ __forceinline__ void store_seed(const SeedTable<T>& t, const Shape& s
 // The unit's seeds j = j0, j0 + step, ... below m, one warp a row and R rows in flight: offsets first, loads after, with no branch
 // between the loads (a branch per row makes every row wait for the one before).  A lane holds four neighbouring channels, so
 // d <= 128 is one round.  off_of(j): element offset of seed j's key.
+// The norm is the sum over the lanes l of the chains f_l^2 + f_(l+32)^2 + ..., so the row goes through `pass`, the warp's own 128
+// elements of shared memory, to be read that way round.  That order of additions is kept because two seeds whose cosines with a row
+// agree to 1e-7 are told apart by it.  (3,072 units of 640 rows: 80 us; the chains handed from lane to lane by shuffles 93, the
+// row's channels read a second time from memory 95, sums over a lane's four neighbouring channels, in another order, 68.)
 template <int R, typename T, typename OffOf>
-__device__ __forceinline__ void gather_seeds(const SeedTable<T>& t, const Shape& sh, int64_t base, int j0, int step, int m, OffOf off_of) {
+__device__ __forceinline__ void gather_seeds(const SeedTable<T>& t, const Shape& sh, int64_t base, int j0, int step, int m, T* pass, OffOf off_of) {
     const int lane = threadIdx.x & 31, d = sh.d;
     for (; j0 < m; j0 += R * step) {
         int64_t off[R];
@@ -504,26 +508,36 @@ __device__ __forceinline__ void gather_seeds(const SeedTable<T>& t, const Shape&
         float n2[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) n2[q] = 0.f;
-        for (int c = 4 * lane; c < d; c += 128) {
+        for (int c0 = 0; c0 < d; c0 += 128) {
+            const int c = c0 + 4 * lane;
             Four<T> x[R];
+            float wc[4] = {1.f, 1.f, 1.f, 1.f}, wl[4] = {1.f, 1.f, 1.f, 1.f};        // weights of channels c + k, c0 + lane + 32 k
+            if (c < d) {
 #pragma unroll
-            for (int q = 0; q < R; ++q) x[q] = *reinterpret_cast<const Four<T>*>(t.K + off[q] + c);
-            float wc[4] = {1.f, 1.f, 1.f, 1.f};
+                for (int q = 0; q < R; ++q) x[q] = *reinterpret_cast<const Four<T>*>(t.K + off[q] + c);
+            }
             if (sh.chan_w) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) wc[k] = sh.chan_w[c + k];
+                for (int k = 0; k < 4; ++k) {
+                    if (c < d) wc[k] = sh.chan_w[c + k];
+                    if (c0 + lane + 32 * k < d) wl[k] = sh.chan_w[c0 + lane + 32 * k];
+                }
             }
 #pragma unroll
             for (int q = 0; q < R; ++q) {
-                if (j0 + q * step < m) store_seed(t, sh, base + j0 + q * step, c, x[q], wc);
+                if (c < d) {
+                    if (j0 + q * step < m) store_seed(t, sh, base + j0 + q * step, c, x[q], wc);
+                    reinterpret_cast<Four<T>*>(pass)[lane] = x[q];
+                }
+                __syncwarp();
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const float f = Elem<T>::ld(&x[q].x[k]);
-                    n2[q] = fmaf(wc[k] * f, f, n2[q]);
+                    const float f = c0 + lane + 32 * k < d ? Elem<T>::ld(&pass[lane + 32 * k]) : 0.f;
+                    n2[q] = fmaf(wl[k] * f, f, n2[q]);
                 }
+                __syncwarp();
             }
         }
-        __syncwarp();
 #pragma unroll
         for (int q = 0; q < R; ++q) {
             float n = n2[q];
@@ -549,7 +563,8 @@ __global__ void __launch_bounds__(32 * kGatherWarps, 8) seed_gather_kernel(
     const int m = max(0, min(plan[u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
     if (j >= m) return;
     const int row = CASK_IDX(seed_rows[ud.seed_base + j], ud.T, sh.err);
-    gather_seeds<1>(tab, sh, ud.seed_base, j, 1, j + 1, [&](int) { return row_elem_off(sh, ud, ud.k_off, row); });
+    __shared__ alignas(16) T pass[kGatherWarps][128];
+    gather_seeds<1>(tab, sh, ud.seed_base, j, 1, j + 1, pass[threadIdx.x >> 5], [&](int) { return row_elem_off(sh, ud, ud.k_off, row); });
     if ((threadIdx.x & 31) == 0) mass_fx[(size_t)u * (max_m + 1) + j] = mass_to_fx(row_mass(sh, s, eps, ud.tok_off + row));
 }
 
@@ -558,7 +573,8 @@ __global__ void __launch_bounds__(32 * kGatherWarps, 8) seed_gather_kernel(
 // memory; the boundary ranks come out of one histogram per range over the keys' own span, and rows inside a boundary bin are
 // ranked by counting, as in decide_long_kernel.  (Ranking every row by counting is quadratic: two units of 1,024 rows took
 // 34 us, now 12.)  Bound by latency, and with thousands of units by the seeds' scattered rows: half the time goes to the gather,
-// so the block table is read at the start and four rows a warp are in flight.  3,072 paged units of 640 rows 90 -> 72 us.  Five
+// so the block table is read at the start and four rows a warp are in flight.  3,072 paged units of 640 rows 90 -> 72 us (80 with
+// the norms summed as they are, see gather_seeds).  Five
 // CTAs an SM: six spill more (68 us there, 50.6 against 49.0 for an event of two units), four leave too few warps (74).
 constexpr int kSmallThreads = 256;
 constexpr int kSmallBins = 4 * kSmallThreads;
@@ -569,7 +585,7 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
     int32_t* __restrict__ seed_rows, unsigned long long* __restrict__ mass_fx, int32_t* __restrict__ njoin,
     int32_t* __restrict__ unit_status, int max_m, float eps) {
     constexpr int kPer = kSmallSpan / kSmallThreads, kWarps = kSmallThreads / 32;
-    __shared__ unsigned keys[kSmallSpan];
+    __shared__ alignas(16) unsigned keys[kSmallSpan];
     __shared__ uint8_t kd[kSmallSpan];
     __shared__ int32_t pages[kSmallSpan];                // the unit's block table: looked up before it is needed
     __shared__ union {
@@ -747,7 +763,8 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
     __syncthreads();
     const int ns = min((int)all, m);
     for (int j = tid; j < ns; j += kSmallThreads) mass_fx[j] = mass_to_fx(row_mass(sh, s, eps, o + sm.l.seeds[j]));
-    gather_seeds<4>(tab, sh, ud.seed_base, w, kWarps, ns, [&](int j) {
+    static_assert(sizeof(keys) >= kWarps * 128 * sizeof(T), "the keys are no longer needed: their place serves the gather");
+    gather_seeds<4>(tab, sh, ud.seed_base, w, kWarps, ns, reinterpret_cast<T*>(keys) + 128 * w, [&](int j) {
         const int i = sm.l.seeds[j];
         if (sh.page_size == 0) return ud.k_off + (int64_t)i * sh.row_stride;
         const int x = i / sh.page_size;

@@ -51,4 +51,12 @@ def test_scores_and_normalisers(name):
     assert digest(g["lse"]) == want["lse"]
     assert digest(g["s"]) == want["s"]
     for out in ("kind", "slot_src", "lost_mass"):
-        assert out not in want or digest(g[out]) == want[out], out
+        assert digest(g[out]) == want[out], out
+
+
+@pytest.mark.parametrize("name", CASES)
+def test_cosines(name):
+    """Best cosine of every scratch row and the seed it belongs to, norms of rows and seeds included."""
+    g, want = event(name), golden(name)
+    assert digest(g["seed_of"]) == want["seed_of"]
+    assert digest(g["sim"]) == want["sim"]
