@@ -17,8 +17,10 @@
 // finishes the row, the other takes the rest and hands its best seed over through shared memory.
 //
 // fp32 caches (SPLIT): the contraction takes the bf16 parts of the rows and the seeds (split.cu) in six products as the scoring
-// passes do (score_tc.cu), one tile of six 16 KB regions at a time, m <= 128; the row norms come from the split.  (16 units of
-// 8,448 rows, m = 96: 236 us on the SIMT kernel, 35 here.)
+// passes do (score_tc.cu), one tile of six 16 KB regions at a time, m <= 128; the row norms come from the split.  What that sum
+// cannot tell, which of two seeds within 8e-6 of one another a row is closer to, or on which side of tau it lies, is decided by the
+// plain fp32 cosines of assign_simt_kernel (see kClose): a row goes where that kernel sends it.  (16 units of 8,448 rows, m = 96:
+// 236 us on the SIMT kernel, 48 here, 33 without the plain cosines.)
 #include "tc_common.cuh"
 
 namespace cask {
@@ -135,9 +137,9 @@ __device__ __forceinline__ uint64_t row_norm2(const uint8_t* base, int lane, int
 // Best seed among the accumulator columns [c_lo, c_hi) of this thread's row: the greatest dot * 1/|k_seed|, the
 // first seed among equals.  PAIR = 1: a seed owns two adjacent columns (the hi and lo parts of its weighted key)
 // whose sum is its dot product.  A block of 32 columns costs a multiply and a maximum per seed; the position of
-// the maximum is looked for only in a block that beats everything before it.
-template <int PAIR>
-__device__ __forceinline__ void best_seed(uint32_t taddr, const float* inv, int c_lo, int c_hi, float& best, int& best_u) {
+// the maximum is looked for only in a block that beats everything before it.  SECOND: the second greatest value as well.
+template <int PAIR, bool SECOND = false>
+__device__ __forceinline__ void best_seed(uint32_t taddr, const float* inv, int c_lo, int c_hi, float& best, int& best_u, float& second) {
     constexpr int kPer = PAIR ? 16 : 32;          // seeds per block of 32 columns
     const uint32_t inv32 = smem_u32(inv);        // full blocks read the inverse norms 16 bytes at a time, shared-space
     for (int cc = c_lo; cc < c_hi; cc += 32) {
@@ -145,7 +147,11 @@ __device__ __forceinline__ void best_seed(uint32_t taddr, const float* inv, int 
         tc_ld32(taddr + cc, v);
         tc_wait_ld_regs(v);
         const int u0 = PAIR ? cc >> 1 : cc, u_hi = PAIR ? c_hi >> 1 : c_hi;
-        float bm = -INFINITY;
+        float bm = -INFINITY, b2 = -INFINITY;
+        auto take = [&](float x) {
+            if (SECOND) b2 = fmaxf(b2, fminf(bm, x));
+            bm = fmaxf(bm, x);
+        };
         if (cc + 32 <= c_hi) {
 #pragma unroll
             for (int x = 0; x < kPer; x += 4) {
@@ -154,7 +160,7 @@ __device__ __forceinline__ void best_seed(uint32_t taddr, const float* inv, int 
 #pragma unroll
                 for (int y = 0; y < 4; ++y) {
                     v[x + y] = (PAIR ? v[2 * (x + y)] + v[2 * (x + y) + 1] : v[x + y]) * nv[y];
-                    bm = fmaxf(bm, v[x + y]);
+                    take(v[x + y]);
                 }
             }
         } else {
@@ -162,9 +168,10 @@ __device__ __forceinline__ void best_seed(uint32_t taddr, const float* inv, int 
             for (int x = 0; x < kPer; ++x) {
                 const float dot = PAIR ? v[2 * x] + v[2 * x + 1] : v[x];
                 v[x] = (u0 + x < u_hi) ? dot * inv[u0 + x] : -INFINITY;
-                bm = fmaxf(bm, v[x]);
+                take(v[x]);
             }
         }
+        if (SECOND) second = fmaxf(fmaxf(second, b2), fminf(best, bm));
         if (bm > best) {
             best = bm;
             int at = kPer - 1;
@@ -172,6 +179,72 @@ __device__ __forceinline__ void best_seed(uint32_t taddr, const float* inv, int 
             for (int x = kPer - 2; x >= 0; --x)
                 if (v[x] == bm) at = x;
             best_u = u0 + at;
+        }
+    }
+}
+
+// fp32 rows whose best cosine is within kClose of another seed's or of tau are decided by the sums assign_simt_kernel takes, one
+// multiply-add after the other in the order of the channels.  A cosine of the two kernels differs by up to 1.2e-6 (768,000 of them;
+// a sum of 128 products is off by 7.6e-6 if all its roundings go one way), so two seeds 7.6e-6 apart come out in the same order
+// either way.  Without this, one event of 16 units of 8,448 rows in eight sent a row to another seed.
+constexpr float kClose = 1.f / 131072.f;
+
+// Of the seeds marked in `close` the one of greatest plain cosine, the first among equals; its cosine in sm.  Four seeds at a time.  The
+// loops stay rolled: the code runs once or twice a CTA, and fetching its instructions takes longer than they do.
+__device__ __noinline__ int plain_best(const float* __restrict__ K, const Shape& sh, const UnitDesc& ud, int row, const int* srow,
+                                       const float* __restrict__ seed_norm, const uint32_t (&close)[4], float& sm) {
+    const int d4 = sh.d / 4;
+    const float4* rp = reinterpret_cast<const float4*>(K + row_elem_off(sh, ud, ud.k_off, row));
+    sm = -INFINITY;
+    int best_u = -1, w = 0;
+    for (uint32_t left = close[0];;) {
+        int c[4], n = 0;
+        float nu[4];
+        const float4* sp[4];
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+            while (!left && w < 3) left = close[++w];
+            if (left) {
+                c[k] = 32 * w + __ffs(left) - 1;
+                left &= left - 1;
+                n = k + 1;
+            }
+            const int at = c[min(k, max(n - 1, 0))];
+            if (n) {
+                sp[k] = reinterpret_cast<const float4*>(K + row_elem_off(sh, ud, ud.k_off, CASK_IDX(srow[at], ud.T, sh.err)));
+                nu[k] = seed_norm[at];
+            }
+        }
+        if (n == 0) return best_u;
+        const float4 *s0 = sp[0], *s1 = sp[1], *s2 = sp[2], *s3 = sp[3];
+        // the rows into L1 first, a load a line and all of them in flight
+#pragma unroll 1
+        for (int x = 0; x < d4; x += 8) {
+            float t;
+            asm volatile("ld.global.ca.f32 %0, [%1];" : "=f"(t) : "l"(rp + x));
+            asm volatile("ld.global.ca.f32 %0, [%1];" : "=f"(t) : "l"(s0 + x));
+            asm volatile("ld.global.ca.f32 %0, [%1];" : "=f"(t) : "l"(s1 + x));
+            asm volatile("ld.global.ca.f32 %0, [%1];" : "=f"(t) : "l"(s2 + x));
+            asm volatile("ld.global.ca.f32 %0, [%1];" : "=f"(t) : "l"(s3 + x));
+        }
+        float a[4] = {0.f, 0.f, 0.f, 0.f}, m[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+        for (int x = 0; x < d4; ++x) {
+            const float4 r = rp[x], v[4] = {s0[x], s1[x], s2[x], s3[x]};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                a[k] = fmaf(r.w, v[k].w, fmaf(r.z, v[k].z, fmaf(r.y, v[k].y, fmaf(r.x, v[k].x, a[k]))));
+            m[0] = fmaf(r.x, r.x, m[0]);
+            m[1] = fmaf(r.y, r.y, m[1]);
+            m[2] = fmaf(r.z, r.z, m[2]);
+            m[3] = fmaf(r.w, r.w, m[3]);
+        }
+        const float nj = sqrtf((m[0] + m[1]) + (m[2] + m[3]));
+#pragma unroll 1
+        for (int k = 0; k < n; ++k) {
+            const float x = nj > 0.f && nu[k] > 0.f ? a[0] / (nj * nu[k]) : 0.f;
+            if (x > sm) { sm = x; best_u = c[k]; }
+            a[0] = a[1]; a[1] = a[2]; a[2] = a[3];
         }
     }
 }
@@ -271,7 +344,7 @@ template <bool FULL, bool SPLIT>
 __global__ void __launch_bounds__(kThreadsA, 1)
 assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmSeed,
                  const UnitDesc* __restrict__ desc, Shape sh, int total_tiles, int n_bufs, int sub_rows, int wpair,
-                 int seed_part_rows, const float* __restrict__ k_norm,
+                 int seed_part_rows, const float* __restrict__ K, const float* __restrict__ k_norm,
                  const float* __restrict__ s, const int32_t* __restrict__ plan,
                  const int32_t* __restrict__ seed_rows, const float* __restrict__ seed_norm,
                  uint8_t* __restrict__ kind, int32_t* __restrict__ seed_of, float* __restrict__ sim,
@@ -537,10 +610,10 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     ok = mbar_wait(&bar.d_full[eg], use & 1u, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    float best = -INFINITY;
+                    float best = -INFINITY, second = 0.f;
                     int best_u = -1;
-                    if (wpair) best_seed<1>(taddr, inv, c_split, mc, best, best_u);
-                    else best_seed<0>(taddr, inv, c_split, mc, best, best_u);
+                    if (wpair) best_seed<1>(taddr, inv, c_split, mc, best, best_u, second);
+                    else best_seed<0>(taddr, inv, c_split, mc, best, best_u, second);
                     tc_fence_before();
                     tail->x_val[eg][use & 1u][my_row] = best;
                     tail->x_idx[eg][use & 1u][my_row] = best_u;
@@ -599,10 +672,32 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 ok = mbar_wait(&bar.d_full[eg], use & 1u, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                float best = -INFINITY;
+                float best = -INFINITY, second = -INFINITY;
                 int best_u = -1;
-                if (wpair) best_seed<1>(taddr, inv, 0, c_split, best, best_u);
-                else best_seed<0>(taddr, inv, 0, c_split, best, best_u);
+                if (!SPLIT && wpair) best_seed<1>(taddr, inv, 0, c_split, best, best_u, second);
+                else best_seed<0, SPLIT>(taddr, inv, 0, c_split, best, best_u, second);
+                const bool cand = in_range && best_u >= 0 && kd == CASK_KIND_DROPPED;
+                uint32_t close[4] = {0u, 0u, 0u, 0u};            // SPLIT: the plain cosines decide between these seeds
+                const float least = best - kClose * nj_c;
+                const bool plain = SPLIT && cand && nj_c > 0.f && (second >= least || fabsf(best - tau * nj_c) <= kClose * nj_c);
+                if (SPLIT && __any_sync(0xffffffffu, plain)) {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        if (32 * b >= m) break;
+                        float v[32];
+                        tc_ld32(taddr + 32 * b, v);
+                        tc_wait_ld_regs(v);
+#pragma unroll
+                        for (int x = 0; x < 32; x += 4) {
+                            const uint4 q = lds128(smem_u32(inv) + (uint32_t)(32 * b + x) * 4u);
+                            if (v[x] * __uint_as_float(q.x) >= least) close[b] |= 1u << x;
+                            if (v[x + 1] * __uint_as_float(q.y) >= least) close[b] |= 2u << x;
+                            if (v[x + 2] * __uint_as_float(q.z) >= least) close[b] |= 4u << x;
+                            if (v[x + 3] * __uint_as_float(q.w) >= least) close[b] |= 8u << x;
+                        }
+                        if (m < 32 * b + 32) close[b] &= (1u << (m - 32 * b)) - 1u;
+                    }
+                }
                 tc_fence_before();
                 if (split == 2) {
                     // The other group's candidate has the larger seed indices, so it wins only when strictly
@@ -620,11 +715,11 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bar.d_empty[eg]);
 
-                const bool cand = in_range && best_u >= 0 && kd == CASK_KIND_DROPPED;
                 float sm_ = 0.f;
                 if (cand) {
                     const float nj = SPLIT ? nj_c : sqrtf(n2);              // best = <k_row, k_seed> / |k_seed| (0 for a zero seed)
                     sm_ = nj > 0.f ? best / nj : 0.f;
+                    if (SPLIT && plain) best_u = plain_best(K, sh, ud, i, srow, seed_norm + seed_base, close, sm_);
                     if (sim) sim[tok_off + i] = sm_;
                 }
                 const bool joined = cand && sm_ >= tau;
@@ -725,7 +820,7 @@ cudaError_t launch_assign_tc(const Launch& L, const cask_params& prm, const floa
     if (e != cudaSuccess) return e;
     Timed t(L, KID_ASSIGN);
     return launch_dependent(L.stream, kern, grid, kThreadsA, kSmemBytesA, tmK, tmSeed, L.desc, sh, L.total_atiles, n_bufs, sub_rows,
-                            wpair, (int)sum_m + 256, ws.k_norm, s, plan, ws.seed_rows, ws.seed_norm, kind, seed_of, sim, ws.grp,
+                            wpair, (int)sum_m + 256, split ? (const float*)L.k : nullptr, ws.k_norm, s, plan, ws.seed_rows, ws.seed_norm, kind, seed_of, sim, ws.grp,
                             ws.mass_fx, ws.njoin, ws.slot_lists ? ws.mem_row : nullptr, ws.mem_slot, L.max_m, prm.tau, prm.eps, ws.err);
 }
 
