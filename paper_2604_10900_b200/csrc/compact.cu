@@ -975,6 +975,7 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int t = tid; t <= slots; t += kLongThreads) start[t] = 0;
+    __syncthreads();                                         // (with given lists the counting begins at once)
     pdl_wait();
     const UnitDesc& ud = desc[u];
     const int T_ = ud.T;

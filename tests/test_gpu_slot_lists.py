@@ -56,3 +56,34 @@ def test_event_equals_the_staged_calls(prefix, decode, budget, reserve, dup, tau
         else:
             assert np.array_equal(g[name], s[name]), name
     assert (g["n_out"] == np.minimum(budget, g["plan"][:, 7])).all()
+
+
+def test_every_unit_of_several_waves_comes_out_the_same():
+    """460 copies of one unit, more than the compaction has CTAs on the device at once, with some 1,000 members on 2,000 slots: the later
+    CTAs wait for no kernel before them, and their slot counts have to start from zero all the same."""
+    import gpu_harness as gh
+    copies, T, P, B = 460, 32100, 60, 2000
+    w = wl.WORKLOADS["reasoning8k_b384"].with_(layers=1, kv_heads=1, group=2, window=32, head_dim=8, prefix=P, decode=T - P, budget=B,
+                                                reserve=1990, cluster_frac=0.0)
+    k, v, q = wl.make_unit(w, 0, 0, 0)
+    hb = wl.Batch(wl=w, k=np.tile(k, (copies, 1)), v=np.tile(v, (copies, 1)), q=np.tile(q[None], (copies, 1, 1, 1)),
+                  T=np.full(copies, T, np.int32), P=np.full(copies, P, np.int32), B=np.full(copies, B, np.int32),
+                  reserve=np.full(copies, 1990, np.int32), tok_off=np.arange(copies + 1, dtype=np.int64) * T,
+                  unit_ids=[(i, 0, 0) for i in range(copies)])
+    run = gh.GpuRun(hb, tau=0.9999)
+    for _ in range(3):
+        g = run.event()
+        assert run.ctx.device_flags() == 0
+        members = np.isin(g["kind"].reshape(copies, T), (4, 5)).sum(1)
+        # (a unit's scores depend in their last bits on the CTAs that share it, so units may differ by a tied row)
+        assert (g["n_out"] == B).all() and (members > 950).all() and (members <= 1024).all()
+        for u in range(copies):
+            a = g["assign"][u * T:(u + 1) * T]
+            wt = g["weight"][u * T:(u + 1) * T]
+            slots = np.bincount(a[a >= 0], weights=wt[a >= 0], minlength=B)
+            assert np.abs(slots - 1.0).max() <= 1e-5, u                      # every slot's weights add up to one
+            rows = g["slot_src"][u]
+            assert (np.diff(rows) > 0).all() and np.array_equal(a[rows], np.arange(B)), u
+            lone = np.bincount(a[a >= 0], minlength=B) == 1
+            got = g["k_out"][u][lone]
+            assert np.array_equal(got, wl.as_float32(k, w.dtype)[rows[lone]]), u
