@@ -468,7 +468,6 @@ constexpr int kFusedWarps = 8;
 // beside the staging in the longer units' one.
 constexpr int kSmallStage = 4096, kLongStage = 3072;
 constexpr int staging_bytes(int stage) { return kFusedWarps * 2 * stage; }
-constexpr int kMergeRows = 4;                // member rows in flight per warp
 
 template <typename T>
 struct RowSource {
@@ -487,21 +486,21 @@ struct RowSource {
 // rows (ascending row order, fp32, rounded once) and puts the result in the slot's place in the buffer, so every output row
 // is written once and the members' latency hides behind the copies.
 //   row_of(slot) -> cache row; first(slot) -> place in the list of the slot's first member (first(nk): the end).
-//   listed: member(place) -> cache row.  The members of all merged slots of the batch are then taken together: a lane looks one
-//   member up (page, score, carried mass, group mass), and the rows are loaded kRows at a time whatever slots they feed, so a
-//   batch of small groups waits once or twice for memory and not once a group.  (Eight rows spill, and the bf16 kernels are
-//   slower with them.)
+//   member(place) -> cache row.  The members of all merged slots of the batch are taken together: a lane looks one member up (page,
+//   score, carried mass, group mass), and the rows are loaded kRows at a time whatever slots they feed, so a batch of small
+//   groups waits once or twice for memory and not once a group.  (Eight rows spill, and the bf16 kernels are slower with them.)
+//   most: slots a batch has at the most.  With groups of hundreds of members a warp takes them one by one, or some warps would have
+//   several of them to add up and others none (32 units of 8,448 rows of which all others join: kernel 440 to 251 us).
 //   busy_slot: the first slot with members.  Its batch is taken first and the copies that wait for nothing last, since the slots
 //   with members lie together: their batches at the end were the tail of the kernel.
 // One group at a time in slot order -> members together -> busy batches first: 3,072 units of 640 rows 346 / 337 / 329 us, 288 of
 // them 44.8 / 40.9 / 36.5, 288 of 33,280 78 / 71 / 63, 112 of 8,448 40.7 / 38.7 / 35.4.
-//   else walk(slot, add) calls add(rows[kMergeRows], left) for a slot's members in order (rows past `left` repeat the last one).
 // CH > 0: head_dim == 32 * CH, a lane owns CH contiguous channels; CH == 0: any head_dim up to 256, channels lane, lane + 32, ...
-template <typename T, int CH, int STAGE, typename RowOf, typename First, typename Member, typename Walk>
+template <typename T, int CH, int STAGE, typename RowOf, typename First, typename Member>
 __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int parts, int part, uint8_t* staging,
                                              uint64_t (*bars)[2], int* next_batch, int* abort_word, T* __restrict__ k_out,
                                              T* __restrict__ v_out, float* __restrict__ slot_mass, int Bmax,
-                                             int32_t* __restrict__ err, bool listed, int busy_slot, RowOf row_of, First first, Member member, Walk walk) {
+                                             int32_t* __restrict__ err, int most, int busy_slot, RowOf row_of, First first, Member member) {
     using namespace tc;
     constexpr int kPer = CH > 0 ? CH : 8;
     constexpr int kRows = 4;                     // member rows in flight
@@ -511,7 +510,7 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, u = in.u, d = sh.d;
     const int64_t o = ud.tok_off;
     const uint32_t row_bytes = CH > 0 ? (uint32_t)(32 * CH * sizeof(T)) : (uint32_t)(d * sizeof(T));
-    const int sb = min(32, (int)(STAGE / 2 / row_bytes));                  // slots per batch
+    const int sb = min(min(32, (int)(STAGE / 2 / row_bytes)), most);       // slots per batch
     volatile int* abort_flag = abort_word;
     uint8_t* my = staging + w * 2 * STAGE;
     const int nb = (nk + sb - 1) / sb, first_b = min(busy_slot, max(nk - 1, 0)) / sb;
@@ -531,7 +530,7 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
         const int t = t0 + lane;
         const int f = lane < nv ? first(t) : 0, members = lane < nv ? first(t + 1) - f : 0;
         const bool merged = members > 1;
-        unsigned todo = __ballot_sync(0xffffffffu, merged);
+        const unsigned todo = __ballot_sync(0xffffffffu, merged);
         // the stores that read this buffer two batches ago must have read it
         if (lane == 0) {
             asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
@@ -584,120 +583,62 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
                 if (lane == 0) slot_mass[(size_t)u * Bmax + t0 + sl] = msum;
             };
             clear();
-            if (listed) {
-                const int count = merged ? members : 0;
-                int before = count;                // members of the batch's slots below this one
+            const int count = merged ? members : 0;
+            int before = count;                // members of the batch's slots below this one
 #pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int x = __shfl_up_sync(0xffffffffu, before, off);
-                    if (lane >= off) before += x;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, before, off);
+                if (lane >= off) before += x;
+            }
+            const int total = __shfl_sync(0xffffffffu, before, 31);
+            before -= count;
+            for (int e0 = 0; e0 < total; e0 += 32) {
+                const int n = min(32, total - e0), e = e0 + min(lane, n - 1);
+                int sl = 0;                    // slot of member e: the last one with at most e members below it
+#pragma unroll
+                for (int step = 16; step >= 1; step >>= 1) {
+                    const int x = __shfl_sync(0xffffffffu, before, sl + step);
+                    if (x <= e) sl += step;
                 }
-                const int total = __shfl_sync(0xffffffffu, before, 31);
-                before -= count;
-                for (int e0 = 0; e0 < total; e0 += 32) {
-                    const int n = min(32, total - e0), e = e0 + min(lane, n - 1);
-                    int sl = 0;                    // slot of member e: the last one with at most e members below it
-#pragma unroll
-                    for (int step = 16; step >= 1; step >>= 1) {
-                        const int x = __shfl_sync(0xffffffffu, before, sl + step);
-                        if (x <= e) sl += step;
-                    }
-                    const int in_group = e - __shfl_sync(0xffffffffu, before, sl);
-                    const int row = member(__shfl_sync(0xffffffffu, f, sl) + in_group);
-                    const unsigned ends = __ballot_sync(0xffffffffu, in_group + 1 == __shfl_sync(0xffffffffu, members, sl));
-                    const int64_t ko = row_elem_off(sh, ud, ud.k_off, row), vo = v_elem_off(sh, ud, u, row);
-                    const float ae = row_mass(sh, in.s, in.eps, o + row);
-                    const float mg = __shfl_sync(0xffffffffu, mg_t, sl);
-                    const float we = in.fw.s ? ae / mg : in.weight[o + row];
-                    for (int c0 = 0; c0 < n; c0 += kRows) {
-                        Vec kr[kRows], vr[kRows];
-                        if (CH > 0) {
-#pragma unroll
-                            for (int q = 0; q < kRows; ++q) {
-                                kr[q] = reinterpret_cast<const Vec*>(in.K + __shfl_sync(0xffffffffu, ko, c0 + q))[lane];
-                                vr[q] = reinterpret_cast<const Vec*>(in.V + __shfl_sync(0xffffffffu, vo, c0 + q))[lane];
-                            }
-                        }
+                const int in_group = e - __shfl_sync(0xffffffffu, before, sl);
+                const int row = member(__shfl_sync(0xffffffffu, f, sl) + in_group);
+                const unsigned ends = __ballot_sync(0xffffffffu, in_group + 1 == __shfl_sync(0xffffffffu, members, sl));
+                const int64_t ko = row_elem_off(sh, ud, ud.k_off, row), vo = v_elem_off(sh, ud, u, row);
+                const float ae = row_mass(sh, in.s, in.eps, o + row);
+                const float mg = __shfl_sync(0xffffffffu, mg_t, sl);
+                const float we = in.fw.s ? ae / mg : in.weight[o + row];
+                for (int c0 = 0; c0 < n; c0 += kRows) {
+                    Vec kr[kRows], vr[kRows];
+                    if (CH > 0) {
 #pragma unroll
                         for (int q = 0; q < kRows; ++q) {
-                            if (c0 + q >= n) break;
-                            const float wi = __shfl_sync(0xffffffffu, we, c0 + q);
-                            msum += __shfl_sync(0xffffffffu, ae, c0 + q);
-                            const int64_t kq = CH > 0 ? 0 : __shfl_sync(0xffffffffu, ko, c0 + q);
-                            const int64_t vq = CH > 0 ? 0 : __shfl_sync(0xffffffffu, vo, c0 + q);
-#pragma unroll
-                            for (int x = 0; x < kPer; ++x) {
-                                if (CH > 0) {
-                                    ak[x] = fmaf(wi, Elem<T>::ld(&kr[q].x[CH > 0 ? x : 0]), ak[x]);
-                                    av[x] = fmaf(wi, Elem<T>::ld(&vr[q].x[CH > 0 ? x : 0]), av[x]);
-                                } else if (lane + 32 * x < d) {
-                                    ak[x] = fmaf(wi, Elem<T>::ld(in.K + kq + lane + 32 * x), ak[x]);
-                                    av[x] = fmaf(wi, Elem<T>::ld(in.V + vq + lane + 32 * x), av[x]);
-                                }
-                            }
-                            if ((ends >> (c0 + q)) & 1u) {
-                                finish(__shfl_sync(0xffffffffu, sl, c0 + q));
-                                clear();
-                            }
+                            kr[q] = reinterpret_cast<const Vec*>(in.K + __shfl_sync(0xffffffffu, ko, c0 + q))[lane];
+                            vr[q] = reinterpret_cast<const Vec*>(in.V + __shfl_sync(0xffffffffu, vo, c0 + q))[lane];
                         }
                     }
-                }
-                todo = 0;
-            }
-            for (; todo; todo &= todo - 1) {
-                const int sl = __ffs(todo) - 1;
-                const float mg = __shfl_sync(0xffffffffu, mg_t, sl);
-                walk(t0 + sl, [&](const int (&rows)[kMergeRows], int left) {
-                    float wi[kMergeRows], ai[kMergeRows];
-                    int64_t ko[kMergeRows], vo[kMergeRows];
-                    // Offsets first, loads after, uses last, with no branch in between: a branch inside the loop over the
-                    // rows (paged or not, carried mass or not) makes every row wait for the one before it.
-                    if (sh.page_size == 0 && !sh.v_pos) {
 #pragma unroll
-                        for (int q = 0; q < kMergeRows; ++q) {
-                            ko[q] = ud.k_off + (int64_t)rows[q] * sh.row_stride;
-                            vo[q] = ud.v_off + (int64_t)rows[q] * sh.row_stride;
-                        }
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < kMergeRows; ++q) {
-                            ko[q] = row_elem_off(sh, ud, ud.k_off, rows[q]);
-                            vo[q] = v_elem_off(sh, ud, u, rows[q]);
-                        }
-                    }
-                    Vec kr[kMergeRows], vr[kMergeRows];
-#pragma unroll
-                    for (int q = 0; q < kMergeRows; ++q) {
-                        if (CH > 0) {
-                            kr[q] = reinterpret_cast<const Vec*>(in.K + ko[q])[lane];
-                            vr[q] = reinterpret_cast<const Vec*>(in.V + vo[q])[lane];
-                        }
-                        ai[q] = in.s[o + rows[q]] + in.eps;                            // row_mass()
-                        wi[q] = in.fw.s ? 0.f : in.weight[o + rows[q]];
-                    }
-                    if (sh.mass_in) {
-#pragma unroll
-                        for (int q = 0; q < kMergeRows; ++q) ai[q] += sh.mass_in[o + rows[q]];
-                    }
-#pragma unroll
-                    for (int q = 0; q < kMergeRows; ++q) {
-                        if (q >= left) break;
-                        if (in.fw.s) wi[q] = ai[q] / mg;
-                        msum += ai[q];
+                    for (int q = 0; q < kRows; ++q) {
+                        if (c0 + q >= n) break;
+                        const float wi = __shfl_sync(0xffffffffu, we, c0 + q);
+                        msum += __shfl_sync(0xffffffffu, ae, c0 + q);
+                        const int64_t kq = CH > 0 ? 0 : __shfl_sync(0xffffffffu, ko, c0 + q);
+                        const int64_t vq = CH > 0 ? 0 : __shfl_sync(0xffffffffu, vo, c0 + q);
 #pragma unroll
                         for (int x = 0; x < kPer; ++x) {
                             if (CH > 0) {
-                                ak[x] = fmaf(wi[q], Elem<T>::ld(&kr[q].x[CH > 0 ? x : 0]), ak[x]);
-                                av[x] = fmaf(wi[q], Elem<T>::ld(&vr[q].x[CH > 0 ? x : 0]), av[x]);
+                                ak[x] = fmaf(wi, Elem<T>::ld(&kr[q].x[CH > 0 ? x : 0]), ak[x]);
+                                av[x] = fmaf(wi, Elem<T>::ld(&vr[q].x[CH > 0 ? x : 0]), av[x]);
                             } else if (lane + 32 * x < d) {
-                                ak[x] = fmaf(wi[q], Elem<T>::ld(in.K + ko[q] + lane + 32 * x), ak[x]);
-                                av[x] = fmaf(wi[q], Elem<T>::ld(in.V + vo[q] + lane + 32 * x), av[x]);
+                                ak[x] = fmaf(wi, Elem<T>::ld(in.K + kq + lane + 32 * x), ak[x]);
+                                av[x] = fmaf(wi, Elem<T>::ld(in.V + vq + lane + 32 * x), av[x]);
                             }
                         }
+                        if ((ends >> (c0 + q)) & 1u) {
+                            finish(__shfl_sync(0xffffffffu, sl, c0 + q));
+                            clear();
+                        }
                     }
-                });
-                finish(sl);
-                clear();
+                }
             }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the merged rows, before the bulk stores read them
@@ -904,8 +845,8 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 3) compact_small_kernel(
     // ---- batches of slots
     const RowSource<T> in{K, V, s, weight, eps, fw, ud, sh, u};
     copy_batches<T, CH, kSmallStage>(
-        in, nk, parts, part, copy_smem, bars, &next_batch, &abort_, k_out, v_out, slot_mass, Bmax, err, true, busy_slot,
-        [&](int t) { return (int)src[t]; }, [&](int t) { return start[t]; }, [&](int e) { return (int)list[e]; }, [](int, auto) {});
+        in, nk, parts, part, copy_smem, bars, &next_batch, &abort_, k_out, v_out, slot_mass, Bmax, err, 32, busy_slot,
+        [&](int t) { return (int)src[t]; }, [&](int t) { return start[t]; }, [&](int e) { return (int)list[e]; });
     late_flags(fw, sh.n_units, err);
 }
 
@@ -914,8 +855,9 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 3) compact_small_kernel(
 // per (pass, warp) cell, and after one scan of the cells to list them, which yields the slots in order.  (Few rows of a long
 // unit are kept: everything after the counting is work on some hundreds of entries.  What a dropped row gets in the per-row
 // outputs, the selection kernel has written.)  Up to kListCap members sit in shared memory, placed slot by slot in row order by
-// counting the earlier ones of a slot; more (thousands of merged rows) are listed in the workspace, and every
-// representative's warp walks the list.
+// counting the earlier ones of a slot.  More (thousands of merged rows) are listed in the workspace and placed there by one warp, 32
+// at a time, while the others look up the slots of the next kListCap.  (Event of 32 units of 8,448 rows of which all others join:
+// 375 us; with every representative's warp walking the whole list 1,374, with a scan, a copy and a merge kernel 342.)
 // 8 units of 33,280 rows (1,024 kept) 33 us, where the scan, copy and merge kernels took 29 + 21 and two more launches; 16 fp32
 // units of 8,448 27 (21 + 20), 112 bf16 ones 35 (21 + 35), 288 of 33,280 63 (57 + 65), 112 of 13,312 with 2,048 kept 69 (19 + 74,
 // of which the copies run at the rate of HBM).
@@ -984,6 +926,14 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     int nk = LISTS ? given.n_kept[u] : -1, nm = 0;
     int n_joined = 0;                                        // given lists: members that are not seeds, the first ones
     bool in_smem = true, given_lists = false;
+    auto slot_of = [&](int i) {                              // slot whose anchor is row i, a seed; else -1
+        int lo = 0, hi = nk - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((src[mid] >> 1) <= i) lo = mid; else hi = mid - 1;
+        }
+        return nk > 0 && src[lo] == 2 * i + 1 ? lo : -1;
+    };
     if (LISTS && nk >= 0) {
         nm = given.n_seed[u] + fw.njoin[u];
         if (nm > kListCap) nk = -1;                          // (thousands of members: listed in the workspace below, in row order)
@@ -1124,30 +1074,40 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
             }
         __syncthreads();
         // ---- slot of every kept and merged row, their weights, the slot tables
-        auto slot_of_row = [&](int i) {                          // slot whose anchor is row i, a seed; else -1
-            int lo = 0, hi = nk - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if ((src[mid] >> 1) <= i) lo = mid; else hi = mid - 1;
+        // (four members a thread, the loads of each kind together: with thousands of members the loop is a chain of memory latencies)
+        constexpr int kU = 4;
+        for (int e0 = tid; e0 < nm; e0 += kU * kLongThreads) {
+            int row[kU], sd[kU], gi[kU], t[kU];
+            float am[kU];
+            uint8_t kd[kU];
+#pragma unroll
+            for (int q = 0; q < kU; ++q) {
+                const int e = min(e0 + q * kLongThreads, nm - 1);
+                row[q] = in_smem ? m_row[e] : mem_row[o + e];
+                t[q] = in_smem ? m_slot[e] : -3;
             }
-            return nk > 0 && src[lo] == 2 * i + 1 ? lo : -1;
-        };
-        for (int e = tid; e < nm; e += kLongThreads) {
-            const int i = in_smem ? m_row[e] : mem_row[o + e];
-            const bool mine = i >= f0 && i < f1;
-            const int sd = seed_of[o + i];                       // (a seed points at itself)
-            const int gi = fw.s && mine ? fw.grp[o + i] : -1;
-            const float a = gi >= 0 ? row_mass(sh, s, eps, o + i) : 0.f;
-            int t = in_smem ? m_slot[e] : -3;
-            if (t == -3 && ku[i] == CASK_KIND_SEED) t = slot_of_row(i);
-            else if (t < -1) {
-                t = slot_of_row(sd);
-                if (mine) assign[o + i] = t;
+#pragma unroll
+            for (int q = 0; q < kU; ++q) {
+                const bool mine = row[q] >= f0 && row[q] < f1;
+                sd[q] = seed_of[o + row[q]];                     // (a seed points at itself)
+                gi[q] = fw.s && mine ? fw.grp[o + row[q]] : -1;
+                kd[q] = in_smem ? (uint8_t)CASK_KIND_MERGED : ku[row[q]];
             }
-            if (in_smem) m_slot[e] = t;
-            else mem_slot[o + e] = t;
-            if (t >= 0) atomicAdd(&start[t], 1);
-            if (gi >= 0 && gi < fw.max_m) weight[o + i] = a / fx_to_mass(fw.mass_fx[(size_t)u * (fw.max_m + 1) + gi]);
+#pragma unroll
+            for (int q = 0; q < kU; ++q) am[q] = gi[q] >= 0 ? row_mass(sh, s, eps, o + row[q]) : 0.f;
+#pragma unroll
+            for (int q = 0; q < kU; ++q) {
+                if (e0 + q * kLongThreads >= nm) break;
+                const int i = row[q];
+                if (t[q] == -3 && kd[q] == CASK_KIND_SEED) t[q] = slot_of(i);
+                else if (t[q] < -1) {
+                    t[q] = slot_of(sd[q]);
+                    if (i >= f0 && i < f1) assign[o + i] = t[q];
+                }
+                if (in_smem) m_slot[e0 + q * kLongThreads] = t[q];
+                if (t[q] >= 0) atomicAdd(&start[t[q]], 1);
+                if (gi[q] >= 0 && gi[q] < fw.max_m) weight[o + i] = am[q] / fx_to_mass(fw.mass_fx[(size_t)u * (fw.max_m + 1) + gi[q]]);
+            }
         }
         for (int t = tid; t < nk; t += kLongThreads) {
             const int i = src[t] >> 1;
@@ -1214,29 +1174,60 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
             }
             list[start[t] + before] = m_row[e];
         }
+    else {
+        // The members in row order, kListCap at a time: their slots by all warps but the first, which places the kListCap before them.
+        // start[t] moves along and ends up as the end of slot t's members.  (The unit's other CTAs write the same.)
+        int* chunk[2] = {m_row, m_row + 2 * kListCap};              // rows, slots
+        auto look_up = [&](int e0, int* rows, int first, int step) {
+            constexpr int kU = 5;                                   // (224 threads: one round)
+            const int n = min(kListCap, nm - e0);
+            for (int x0 = first; x0 < n; x0 += kU * step) {
+                int row[kU], sd[kU];
+                uint8_t kd[kU];
+#pragma unroll
+                for (int q = 0; q < kU; ++q) row[q] = mem_row[o + e0 + min(x0 + q * step, n - 1)];
+#pragma unroll
+                for (int q = 0; q < kU; ++q) { kd[q] = ku[row[q]]; sd[q] = seed_of[o + row[q]]; }
+#pragma unroll
+                for (int q = 0; q < kU; ++q) {
+                    const int x = x0 + q * step;
+                    if (x >= n) break;
+                    rows[x] = row[q];
+                    rows[kListCap + x] = slot_of(kd[q] == CASK_KIND_SEED ? row[q] : sd[q]);
+                }
+            }
+        };
+        look_up(0, chunk[0], tid, kLongThreads);
+        __syncthreads();
+        for (int e0 = 0, b = 0; e0 < nm; e0 += kListCap, b ^= 1) {
+            if (w > 0) {
+                look_up(e0 + kListCap, chunk[b ^ 1], tid - 32, kLongThreads - 32);
+            } else {
+                const int* rows = chunk[b];
+                const int n = min(kListCap, nm - e0);
+                for (int x0 = 0; x0 < n; x0 += 32) {
+                    const int x = x0 + lane, t = x < n ? rows[kListCap + x] : -1;
+                    const unsigned same = __match_any_sync(0xffffffffu, t);
+                    const int at = t >= 0 ? start[t] + __popc(same & ((1u << lane) - 1u)) : 0;
+                    __syncwarp();
+                    if (t >= 0) {
+                        mem_slot[o + at] = rows[x];
+                        if (lane == 31 - __clz(same)) start[t] = at + 1;
+                    }
+                    __syncwarp();
+                }
+            }
+            __syncthreads();
+        }
+    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // bulk copies write over the list from here on
     __syncthreads();
     // ---- batches of slots
     const RowSource<T> in{K, V, s, weight, eps, fw, ud, sh, u};
     copy_batches<T, CH, kLongStage>(
-        in, nk, parts, part, copy_smem, bars, &next_batch, &abort_, k_out, v_out, slot_mass, Bmax, err, in_smem, busy_slot,
-        [&](int t) { return src[t] >> 1; }, [&](int t) { return start[t]; }, [&](int e) { return list[e]; },
-        [&](int t, auto add) {
-            for (int e0 = 0; e0 < nm; e0 += 32) {
-                const int e = e0 + lane;
-                const int row = e < nm ? mem_row[o + e] : 0;
-                unsigned hits = __ballot_sync(0xffffffffu, e < nm && mem_slot[o + e] == t);
-                while (hits) {
-                    int rows[kMergeRows], n = 0, at = 0;
-#pragma unroll
-                    for (int q = 0; q < kMergeRows; ++q) {
-                        if (hits) { at = __ffs(hits) - 1; hits &= hits - 1; ++n; }
-                        rows[q] = __shfl_sync(0xffffffffu, row, at);
-                    }
-                    add(rows, n);
-                }
-            }
-        });
+        in, nk, parts, part, copy_smem, bars, &next_batch, &abort_, k_out, v_out, slot_mass, Bmax, err, nm > 4 * nk ? 1 : 32, busy_slot,
+        [&](int t) { return src[t] >> 1; }, [&](int t) { return in_smem ? start[t] : t > 0 ? start[t - 1] : 0; },
+        [&](int e) { return in_smem ? list[e] : mem_slot[o + e]; });
     late_flags(fw, sh.n_units, err);
 }
 

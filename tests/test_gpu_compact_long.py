@@ -81,3 +81,31 @@ def test_every_division_of_a_unit_among_ctas_gives_the_same(copies):
         mem = np.nonzero(g["assign"][:T] == t)[0]
         want = (g["weight"][:T][mem, None].astype(np.float64) * kf[mem]).sum(0)
         assert np.abs(g["k_out"][0][t] - want).max() <= np.maximum(2e-2, np.abs(want) * 2.0 ** -7).max()
+
+
+def test_thousands_of_members_cost_a_fraction_more():
+    """An event in which every scratch row joins against one in which none does: more rows to add up, which takes about twice the
+    time (it was nine times when every group's warp looked through all of the unit's members)."""
+    import gpu_harness as gh
+    import torch
+    hb = wl.make_batch(wl.WORKLOADS["reasoning8k_b512"].with_(layers=4, kv_heads=4))
+
+    def best_ms(tau):
+        run = gh.GpuRun(hb, tau=tau)
+        run.out_struct.rho_core = run.out_struct.rho_rep = run.out_struct.dispersion = None        # (no diagnostics)
+        run.event()
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(5):
+                run.cb.cask_compress_event(run.ctx, run.batch, run.prm, run.out_struct, run.ws, run.ws_bytes)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        members = np.isin(run.out["kind"].cpu().numpy(), (4, 5)).sum() / hb.n_units
+        return min(times), members
+
+    (all_join, many), (none_joins, few) = best_ms(-1.0), best_ms(2.0)
+    assert many > 7500 and few < 200
+    assert all_join < 4.0 * none_joins, (all_join, none_joins)
