@@ -272,7 +272,7 @@ def other_workloads(args, device, local, peaks, headline: "Event"):
                    event_roofline=event_roofline(hb, n_out, kind, med, peaks), dominant_kernel=top,
                    dominant_kernel_ms=kern[top]["ms_per_launch"] * kern[top]["launches_per_step"],
                    kernels={k: round(v["ms_per_launch"] * v["launches_per_step"], 5) for k, v in kern.items()},
-                   score_path="tcgen05" if ev.ctx.used_tensor_path else "simt",
+                   score_path="tcgen05" if ev.ctx.score_path else "simt",
                    score_pass_sm_mhz=list(ev.ctx.score_clock_mhz()),
                    status_bits_seen=int(np.bitwise_or.reduce(status)),
                    l2="inputs larger than L2: %.2f GB of K/V read per step" % ((hb.k.nbytes + hb.v.nbytes) / 1e9))

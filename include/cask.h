@@ -200,8 +200,8 @@ int cask_profile_enable(cask_ctx* ctx, int on);
 int cask_profile_read(cask_ctx* ctx, float* ms, int64_t* launches);
 int cask_kernel_count(void);
 const char* cask_kernel_name(int id);
-/* 1 if the last cask_score / cask_compress_event scored a bf16 cache on the tensor cores.  An fp32 cache reads 0, also
- * where the three bf16 parts its numbers split into exactly are contracted there. */
+/* Which kernels the last cask_score / cask_compress_event scored with: 0 the SIMT kernels, 1 the tensor cores (a bf16
+ * cache), 2 the tensor cores through the three bf16 parts that the numbers of an fp32 cache are split into. */
 int cask_last_score_path_tensor(const cask_ctx* ctx);
 /* Device-side flags (CASK_ST_TIMEOUT, CASK_ST_BOUNDS) raised by the kernels of the last call of this
  * context; waits for the context's stream.  cask_consolidate_scratch ORs the flags raised up to the

@@ -259,8 +259,14 @@ class Context:
                 for i in range(n) if cnt[i]}
 
     @property
+    def score_path(self) -> int:
+        """Kernels of the last scoring call: 0 SIMT, 1 tensor cores (bf16), 2 tensor cores through the bf16 parts of an fp32 cache."""
+        return int(self._lib.cask_last_score_path_tensor(self.handle))
+
+    @property
     def used_tensor_path(self) -> bool:
-        return bool(self._lib.cask_last_score_path_tensor(self.handle))
+        """Did the last scoring call contract a bf16 cache as it is on the tensor cores?  (fp32: see score_path.)"""
+        return self.score_path == 1
 
     def score_clock_mhz(self):
         """(normaliser pass, score pass) SM clock in MHz of the last tensor-core scoring call (0: did not run)."""

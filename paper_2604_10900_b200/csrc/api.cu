@@ -50,7 +50,7 @@ struct cask_ctx {
     bool staged_pending = false;
     int64_t launches = 0;
     cudaError_t last_err = cudaSuccess;
-    int last_tc = 0;
+    int last_tc = 0;                 // see cask_last_score_path_tensor
     const int32_t* flags_dev = nullptr;   // flag word of the last call's workspace
     // host-buffer entry point: pinned staging for the row kinds coming back and the packed value rows going in
     char* hstage = nullptr;
@@ -332,7 +332,7 @@ int run_score(cask_ctx* ctx, const Launch& L, const cask_batch* b, const cask_pa
               float* lse_out, Workspace& W) {
     cudaError_t e;
     if (p->score_path == 0 && ctx->tmap_encode && score_tc_supported(L)) {
-        ctx->last_tc = L.sh.dtype == CASK_DTYPE_BF16;
+        ctx->last_tc = L.sh.dtype == CASK_DTYPE_BF16 ? 1 : 2;
         e = launch_score_tc(L, b->lse_in, s, lse_out, W, ctx->tmap_encode);
     } else {
         ctx->last_tc = 0;

@@ -99,3 +99,16 @@ def test_fp32_caches_through_their_bf16_parts(group, window, d, page, tail, budg
     big = simt["s"] > 1e-12
     assert (np.abs(g["s"] - simt["s"])[big] <= 1e-5 * simt["s"][big]).all()
 
+
+
+@pytest.mark.parametrize("dtype,d,score_path,want", [(wl.DTYPE_BF16, 128, 0, 1), (wl.DTYPE_FP32, 128, 0, 2), (wl.DTYPE_FP32, 64, 0, 2),
+                                                    (wl.DTYPE_FP32, 128, 1, 0), (wl.DTYPE_FP32, 200, 0, 0), (wl.DTYPE_BF16, 128, 1, 0)])
+def test_the_path_that_scored_is_told(dtype, d, score_path, want):
+    """The kernels that ran, and the clocks of the tensor-core passes wherever those ran."""
+    import gpu_harness as gh
+    w = wl.WORKLOADS["tiny"].with_(dtype=dtype, head_dim=d, decode=3000)
+    run = gh.GpuRun(wl.make_batch(w), score_path=score_path)
+    run.event()
+    assert run.ctx.score_path == want and run.ctx.used_tensor_path == (want == 1)
+    clocks = run.ctx.score_clock_mhz()
+    assert all(c > 100.0 for c in clocks) if want else clocks == (0.0, 0.0)
