@@ -346,9 +346,10 @@ template <> struct Elem<__nv_bfloat16> {
     static __device__ __forceinline__ void st(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
 };
 
-// x = h + m + l, exactly (see split.cu)
+// x = h + m + l, exactly (see split.cu).  A finite x that rounds to infinity (above bf16's greatest number) is rounded towards zero.
 __device__ __forceinline__ void split3(float x, __nv_bfloat16& h, __nv_bfloat16& m, __nv_bfloat16& l) {
     h = __float2bfloat16_rn(x);
+    if (__hisinf(h)) h = __float2bfloat16_rz(x);
     const float r = x - __bfloat162float(h);
     m = __float2bfloat16_rn(r);
     l = __float2bfloat16_rn(r - __bfloat162float(m));

@@ -1,5 +1,5 @@
 // fp32 rows as three bf16 parts for the tensor cores: x = h + m + l with h = bf16(x), m = bf16(x - h), l = x - h - m, 8 bits of
-// the 24-bit significand each, so the sum is exact (down to the smallest normal numbers of the last part).  Keys of every
+// the 24-bit significand each, so the sum is exact for every finite x, but for bits below 2^-133, the least that bf16 holds.  Keys of every
 // layout land dense, part after part: row tok_off[u] + i of part p at k_split + (p * sumT + tok_off[u] + i) * d; the queries
 // the same way.  The Euclidean norm of every key row, which the assignment needs, comes along.
 //

@@ -112,3 +112,22 @@ def test_the_path_that_scored_is_told(dtype, d, score_path, want):
     assert run.ctx.score_path == want and run.ctx.used_tensor_path == (want == 1)
     clocks = run.ctx.score_clock_mhz()
     assert all(c > 100.0 for c in clocks) if want else clocks == (0.0, 0.0)
+
+
+def test_fp32_numbers_above_the_greatest_bf16_number():
+    """Keys of up to 3.4e38, which bf16 would round to infinity, against queries that make ordinary logits of them."""
+    import gpu_harness as gh
+    from oracle import cask_oracle as orc
+    hb = wl.make_batch(wl.WORKLOADS["tiny"].with_(decode=1500))
+    rng = np.random.default_rng(0)
+    big = rng.permutation(len(hb.k))[:300]
+    hb.k[:, 5] = 0.0
+    hb.k[big, 5] = (rng.uniform(3.38, 3.4028234e38 / 1e38, len(big)) * 1e38 * rng.choice([-1, 1], len(big))).astype(np.float32)
+    assert (np.abs(hb.k[big, 5]) > 3.3961e38).any()               # beyond the last number that rounds to a finite bf16
+    hb.q[..., 5] = np.float32(2.0 ** -126) * rng.choice([1, 2, 4], hb.q.shape[:-1]).astype(np.float32)
+    run = gh.GpuRun(hb)
+    run.cb.cask_score(run.ctx, run.batch, run.prm, run.out["s"], run.out["lse"], run.ws, run.ws_bytes)
+    s = run.out["s"].cpu().numpy()
+    assert run.ctx.score_path == 2
+    want, _ = orc.score_batch(hb.k, hb.q, hb.tok_off)
+    assert (np.abs(s - want) <= 1e-5 * want + 1e-12).all()
