@@ -538,7 +538,7 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
         }
         __syncwarp();
         if (lane < nv && !merged) {
-            const int row = row_of(t);
+            const int row = CASK_IDX(row_of(t), ud.T, err);
             const T* kr = in.K + row_elem_off(sh, ud, ud.k_off, row);
             const T* vr = in.V + v_elem_off(sh, ud, u, row);
             const uint32_t bar = smem_u32(&bars[w][st]);
@@ -551,7 +551,7 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
         if (todo) {
             float mg_t = 0.f;                      // group mass of slot t (event path: the weights are formed here)
             if (in.fw.s && merged) {
-                const int gi = min(max(in.fw.grp[o + row_of(t)], 0), in.fw.max_m);
+                const int gi = min(max(CASK_IDX(in.fw.grp[o + row_of(t)], max(in.fw.max_m, 1), err), 0), in.fw.max_m);
                 mg_t = fx_to_mass(in.fw.mass_fx[(size_t)u * (in.fw.max_m + 1) + gi]);
             }
             float ak[kPer], av[kPer], msum;
@@ -601,7 +601,7 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
                     if (x <= e) sl += step;
                 }
                 const int in_group = e - __shfl_sync(0xffffffffu, before, sl);
-                const int row = member(__shfl_sync(0xffffffffu, f, sl) + in_group);
+                const int row = CASK_IDX(member(__shfl_sync(0xffffffffu, f, sl) + in_group), ud.T, err);
                 const unsigned ends = __ballot_sync(0xffffffffu, in_group + 1 == __shfl_sync(0xffffffffu, members, sl));
                 const int64_t ko = row_elem_off(sh, ud, ud.k_off, row), vo = v_elem_off(sh, ud, u, row);
                 const float ae = row_mass(sh, in.s, in.eps, o + row);
@@ -1083,7 +1083,7 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
 #pragma unroll
             for (int q = 0; q < kU; ++q) {
                 const int e = min(e0 + q * kLongThreads, nm - 1);
-                row[q] = in_smem ? m_row[e] : mem_row[o + e];
+                row[q] = in_smem ? m_row[e] : CASK_IDX(mem_row[o + e], T_, err);
                 t[q] = in_smem ? m_slot[e] : -3;
             }
 #pragma unroll
@@ -1185,7 +1185,7 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
                 int row[kU], sd[kU];
                 uint8_t kd[kU];
 #pragma unroll
-                for (int q = 0; q < kU; ++q) row[q] = mem_row[o + e0 + min(x0 + q * step, n - 1)];
+                for (int q = 0; q < kU; ++q) row[q] = CASK_IDX(mem_row[o + e0 + min(x0 + q * step, n - 1)], T_, err);
 #pragma unroll
                 for (int q = 0; q < kU; ++q) { kd[q] = ku[row[q]]; sd[q] = seed_of[o + row[q]]; }
 #pragma unroll

@@ -35,6 +35,11 @@ def _cases():
     yield "bf16_tensor_path", r8k.with_(layers=1, kv_heads=2, decode=1024 + 19), {}
     yield "bf16_paged", r8k.with_(layers=1, kv_heads=2, decode=900), dict(page_size=16)
     yield "bf16_many_seeds", wl.WORKLOADS["reasoning32k_b1024"].with_(layers=1, kv_heads=1, decode=3000), {}
+    yield "slot_lists", r8k.with_(layers=1, kv_heads=3, decode=5000, budget=200, reserve=120), {}
+    yield "slot_lists_given_up", r8k.with_(layers=1, kv_heads=2, decode=5000, budget=200, reserve=120), dict(tau=-1.0, page_size=64)
+    yield "thousands_of_members", r8k.with_(layers=1, kv_heads=2, decode=3000), dict(tau=-1.0)
+    yield "fp32_thousands_of_members", tiny.with_(decode=3000), dict(tau=-1.0)
+    yield "few_channels_long", tiny.with_(dtype=wl.DTYPE_BF16, head_dim=40, decode=2500), {}
     yield "short_units", wl.WORKLOADS["serving_steady_b512"].with_(layers=1, kv_heads=2, n_seqs=3), {}
 
 
@@ -70,4 +75,4 @@ def test_every_index_check_stays_silent_and_the_results_are_the_ordinary_builds(
             ran += 1
     finally:
         cb.use_library(None)
-    assert ran >= 14
+    assert ran >= 19
