@@ -27,6 +27,7 @@ struct FusedWeights {
 constexpr int kScanThreads = 1024;
 constexpr int kScanMaxIters = 63;      // rows per unit below 64,512: the one-scan path of slot_scan_kernel
 
+// ==== scan, copy and merge as kernels of their own: units above kLongMaxRows rows and budgets above kLongMaxSlots ================
 // ---- 1. per-unit ordered scan: slots, index map, member list -------------------------------
 __global__ void __launch_bounds__(kScanThreads) slot_scan_kernel(
     const UnitDesc* __restrict__ desc, const uint8_t* __restrict__ kind, const int32_t* __restrict__ seed_of,
@@ -1390,7 +1391,7 @@ cudaError_t run(const Launch& L, const cask_params& prm, const float* s, const u
     cudaError_t e;
     {
         Timed t(L, KID_SLOT_SCAN);
-        e = launch_dependent(L.stream, slot_scan_kernel, sh.n_units, L.max_T <= 2048 ? 256 : kScanThreads, 0, L.desc, kind, seed_of,
+        e = launch_dependent(L.stream, slot_scan_kernel, sh.n_units, kScanThreads, 0, L.desc, kind, seed_of,
                              weight, out.Bmax, out.n_out, out.slot_src, out.slot_kind, out.slot_mass, out.assign, ws.mem_row,
                              ws.mem_slot, ws.n_mem, ws.seed_slot, ws.n_seed, ws.max_B, fw, ws.err);
         if (e != cudaSuccess) return e;

@@ -109,3 +109,57 @@ def test_thousands_of_members_cost_a_fraction_more():
     (all_join, many), (none_joins, few) = best_ms(-1.0), best_ms(2.0)
     assert many > 7500 and few < 200
     assert all_join < 4.0 * none_joins, (all_join, none_joins)
+
+
+@pytest.mark.parametrize("specs,tau,page,dtype", [
+    # (rows, prefix, budget, reserve): more slots than the one-kernel compaction has room for, beside shorter units
+    ([(14000, 300, 12400, 12200), (1500, 20, 12300, 0), (13000, 12900, 12390, 50)], 0.9, 0, wl.DTYPE_BF16),
+    ([(14000, 300, 12400, 12200), (40, 8, 30, 25)], -1.0, 16, wl.DTYPE_FP32),
+    # more rows than it counts
+    ([(262129, 100, 120, 90), (5000, 10, 60, 55)], 0.9, 0, wl.DTYPE_BF16),
+    ([(262200, 261000, 150, 60), (70000, 5, 400, 400)], 0.5, 64, wl.DTYPE_BF16),
+])
+def test_budgets_and_units_beyond_the_one_kernel_compaction(specs, tau, page, dtype):
+    """The event against the staged calls with the same scores, whose selection, weights and status come from kernels of their own."""
+    import gpu_harness as gh
+    base = wl.WORKLOADS["tiny"].with_(dtype=dtype, head_dim=8, group=2, window=16, cluster_frac=0.6, n_centres=0)
+    parts = [wl.make_unit(base.with_(prefix=p, decode=t - p), i, 0, 0) for i, (t, p, b, r) in enumerate(specs)]
+    T, P, B, R = (np.array(x, np.int32) for x in zip(*specs))
+    hb = wl.Batch(wl=base, k=np.concatenate([p[0] for p in parts]), v=np.concatenate([p[1] for p in parts]),
+                  q=np.stack([p[2] for p in parts]), T=T, P=P, B=B, reserve=R,
+                  tok_off=np.concatenate([[0], np.cumsum(T)]).astype(np.int64), unit_ids=[(i, 0, 0) for i in range(len(T))])
+    run = gh.GpuRun(hb, tau=tau, page_size=page)
+    run.ctx.profile_enable(True)
+    g = run.event()
+    assert run.ctx.device_flags() == 0 and "slot_scan" in run.ctx.profile_read()
+    st = gh.GpuRun(hb, tau=tau, page_size=page)
+    o, args, ws = st.out, (st.ctx, st.batch, st.prm), (st.ws, st.ws_bytes)
+    st.cb.cask_score(*args, o["s"], o["lse"], *ws)
+    st.cb.cask_prefix_evict(*args, o["s"], o["kind"], o["plan"], *ws)
+    st.cb.cask_select_core(*args, o["s"], o["plan"], o["kind"], *ws)
+    st.cb.cask_consolidate_scratch(*args, o["s"], o["plan"], o["kind"], o["seed_of"], o["weight"], o["sim"], o["unit_status"],
+                                   o["lost_mass"], *ws)
+    st.cb.cask_compact(*args, o["s"], o["kind"], o["seed_of"], o["weight"], st.out_struct, *ws)
+    h = st.numpy_outputs()
+    merged = 0
+    kf, vf = wl.as_float32(hb.k, dtype), wl.as_float32(hb.v, dtype)
+    for name in g:
+        if name not in ("k_out", "v_out"):
+            assert np.array_equal(g[name], h[name]), name
+    for u in range(len(specs)):
+        a, k = int(hb.tok_off[u]), int(g["n_out"][u])
+        assert k == min(int(T[u]), int(B[u]))
+        assert np.array_equal(g["k_out"][u][:k], h["k_out"][u][:k]) and np.array_equal(g["v_out"][u][:k], h["v_out"][u][:k])
+        # the rows themselves, in 64 bits
+        kind, to, wt = (g[x][a:a + int(T[u])] for x in ("kind", "assign", "weight"))
+        keep = np.nonzero(np.isin(kind, (1, 2, 3, 4)))[0]
+        assert np.array_equal(g["slot_src"][u][:k], keep) and np.array_equal(to[keep], np.arange(k))
+        mem = np.nonzero(to >= 0)[0]
+        for name, x in (("k_out", kf), ("v_out", vf)):
+            want = np.zeros((k, 8))
+            np.add.at(want, to[mem], wt[mem, None].astype(np.float64) * x[a + mem])
+            tol = 1e-4 * np.abs(want) + 1e-5 if dtype == wl.DTYPE_FP32 else np.maximum(2e-2, np.abs(want) * 2.0 ** -7)
+            assert (np.abs(g[name][u][:k] - want) <= tol).all()
+        merged += int((kind == 5).sum())
+        assert (g["slot_src"][u][k:] == -1).all() and (g["slot_kind"][u][k:] == 0).all() and (g["slot_mass"][u][k:] == 0).all()
+    assert merged > 0
