@@ -65,7 +65,7 @@ struct cask_ctx {
     void* tmap_encode = nullptr;     // cuTensorMapEncodeTiled, resolved at creation
     void* ptr_attribute = nullptr;   // cuPointerGetAttribute
     int sms = 0;                     // multiprocessors of the device
-    uint64_t smem_allowed = 0;       // see allow_smem
+    SmemKept smem;                   // see allow_smem
     Profiler prof;
     ProfImpl prof_impl;
 };
@@ -322,7 +322,7 @@ int prepare(cask_ctx* ctx, const cask_batch* b, const cask_params* p, void* ws, 
     L.tmap_encode = ctx->tmap_encode;
     L.force_simt = p->score_path;
     L.sms = ctx->sms;
-    L.smem_allowed = &ctx->smem_allowed;
+    L.smem = &ctx->smem;
     L.launches = &ctx->launches;
     L.prof = &ctx->prof;
     return CASK_OK;

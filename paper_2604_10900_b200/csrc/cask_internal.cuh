@@ -93,16 +93,34 @@ struct Launch {
     int force_simt;
     int sms;                  // multiprocessors of the context's device (0: not known)
     RowDefaults fill;         // what the scoring call may write beside the scores
-    uint64_t* smem_allowed;   // kernels that this context has given their dynamic shared memory already (NULL: none kept)
+    struct SmemKept* smem;    // what this context has found out about its kernels' shared memory (NULL: nothing is kept)
 };
 
-// Lets a kernel use `bytes` of dynamic shared memory: once per context and kernel (`bit`, below 64, names the kernel).
+// Kernels that a context has given their dynamic shared memory already, by their bits, and the static shared memory that the
+// compiler gave each of them.
+struct SmemKept {
+    uint64_t allowed = 0;
+    int fixed[64] = {};
+};
+
+// Lets a kernel use `bytes` of dynamic shared memory: once per context and kernel (`bit`, below 64, names the kernel).  *fixed: its
+// static shared memory.
 template <typename K>
-inline cudaError_t allow_smem(const Launch& L, int bit, K kern, size_t bytes) {
-    if (L.smem_allowed && (*L.smem_allowed >> bit) & 1) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && L.smem_allowed) *L.smem_allowed |= (uint64_t)1 << bit;
-    return e;
+inline cudaError_t allow_smem(const Launch& L, int bit, K kern, size_t bytes, size_t* fixed = nullptr) {
+    if (L.smem && (L.smem->allowed >> bit) & 1) {
+        if (fixed) *fixed = (size_t)L.smem->fixed[bit];
+        return cudaSuccess;
+    }
+    cudaFuncAttributes attr{};
+    cudaError_t e = cudaFuncGetAttributes(&attr, kern);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+    if (fixed) *fixed = attr.sharedSizeBytes;
+    if (L.smem) {
+        L.smem->allowed |= (uint64_t)1 << bit;
+        L.smem->fixed[bit] = (int)attr.sharedSizeBytes;
+    }
+    return cudaSuccess;
 }
 constexpr int kSmemBitScore = 0, kSmemBitAssign = 28, kSmemBitConsolidate = 32, kSmemBitCopy = 40;   // first bit of each file's kernels
 
@@ -110,12 +128,13 @@ constexpr int kSmemBitScore = 0, kSmemBitAssign = 28, kSmemBitConsolidate = 32, 
 // CTAs that start while the kernel before them leaves go to the SMs that are free first, as many as fit: 288 CTAs of which
 // three fit an SM ran on 97 of the 148.  (288 units of 640 rows, selection kernel: event 175 to 169 us; eight units of 33,280
 // rows, compaction: 183 to 178.  Not for kernels beside the scoring passes: the row combine, padded so, cost an event of
-// 3.6 ms 0.1 ms.)  `fixed`: the kernel's static shared memory.
+// 3.6 ms 0.1 ms.)  `fixed`: the kernel's static shared memory, as allow_smem gives it.
 constexpr size_t kMaxSpread = 116 << 10;             // the most that spreading asks for (one CTA per SM)
+constexpr size_t kReserved = 1024;                   // what the system takes of the shared memory of every CTA
 inline size_t spread_smem(const Launch& L, int64_t grid, size_t fixed, size_t need) {
     const int64_t per_sm = (grid + L.sms - 1) / std::max(L.sms, 1);
     if (L.sms < 1 || per_sm > 7) return need;
-    constexpr size_t kSm = 228 << 10, kReserved = 1024;
+    constexpr size_t kSm = 228 << 10;
     const size_t least = kSm / (size_t)(per_sm + 1) + 256;           // per CTA: one more than per_sm does not fit
     return std::max(need, least > fixed + kReserved ? (least - fixed - kReserved + 127) / 128 * 128 : 0);
 }

@@ -1360,13 +1360,14 @@ cudaError_t run(const Launch& L, const cask_params& prm, const float* s, const u
         auto kern = sh.d == 128 ? compact_small_kernel<T, 4> : sh.d == 64 ? compact_small_kernel<T, 2> : compact_small_kernel<T, 0>;
         constexpr int smem = staging_bytes(kSmallStage);
         static_assert(smem <= kMaxSpread, "");
-        cudaError_t e = allow_smem(L, kSmemBitCopy + 2 + 3 * (sizeof(T) == 4) + (sh.d == 128 ? 0 : sh.d == 64 ? 1 : 2), kern, kMaxSpread);
+        size_t fixed = 0;
+        cudaError_t e = allow_smem(L, kSmemBitCopy + 2 + 3 * (sizeof(T) == 4) + (sh.d == 128 ? 0 : sh.d == 64 ? 1 : 2), kern, kMaxSpread, &fixed);
         if (e != cudaSuccess) return e;
         // as many CTAs per unit as fit the device at once, so that a few units' rows move at more than a few SMs' rate
         const int parts = std::max(1, std::min(8, 3 * (L.sms > 0 ? L.sms : 128) / std::max(sh.n_units, 1)));
         Timed t(L, KID_GATHER_MERGE);
         return launch_dependent(L.stream, kern, sh.n_units * parts, kFusedWarps * 32,
-                                spread_smem(L, (int64_t)sh.n_units * parts, 8576, smem), L.desc, sh, (const T*)L.k,
+                                spread_smem(L, (int64_t)sh.n_units * parts, fixed, smem), L.desc, sh, (const T*)L.k,
                                 (const T*)L.v, kind, seed_of, s, weight, prm.eps, out.Bmax, parts, out.n_out, out.slot_src,
                                 out.slot_kind, out.slot_mass, out.assign, (T*)out.k_out, (T*)out.v_out, fw, ws.err);
     }
@@ -1376,14 +1377,15 @@ cudaError_t run(const Launch& L, const cask_params& prm, const float* s, const u
         auto kern = lists ? (sh.d == 128 ? compact_long_kernel<T, 4, true> : sh.d == 64 ? compact_long_kernel<T, 2, true> : compact_long_kernel<T, 0, true>)
                           : (sh.d == 128 ? compact_long_kernel<T, 4, false> : sh.d == 64 ? compact_long_kernel<T, 2, false> : compact_long_kernel<T, 0, false>);
         const int bit = kSmemBitCopy + 8 + 6 * lists + 3 * (sizeof(T) == 4) + (sh.d == 128 ? 0 : sh.d == 64 ? 1 : 2);
-        cudaError_t e = allow_smem(L, bit, kern, std::max(kMaxSpread, long_smem(kLongMaxSlots)));
+        size_t fixed = 0;
+        cudaError_t e = allow_smem(L, bit, kern, std::max(kMaxSpread, long_smem(kLongMaxSlots)), &fixed);
         if (e != cudaSuccess) return e;
         const GivenLists given{ws.n_mem, ws.n_seed, ws.seed_slot, ws.seed_rows, ws.max_B};
-        const int per_sm = std::max(1, std::min(3, (int)((227 << 10) / (long_smem(table) + 5632))));      // + static and reserved
+        const int per_sm = std::max(1, std::min(3, (int)((227 << 10) / (long_smem(table) + fixed + kReserved))));
         const int parts = std::max(1, std::min(16, per_sm * (L.sms > 0 ? L.sms : 128) / std::max(sh.n_units, 1)));
         Timed t(L, KID_GATHER_MERGE);
         return launch_dependent(L.stream, kern, sh.n_units * parts, kLongThreads,
-                                spread_smem(L, (int64_t)sh.n_units * parts, 4352, long_smem(table)), L.desc, sh, (const T*)L.k,
+                                spread_smem(L, (int64_t)sh.n_units * parts, fixed, long_smem(table)), L.desc, sh, (const T*)L.k,
                                 (const T*)L.v, kind, seed_of, s, weight, prm.eps, out.Bmax, table, parts, out.n_out, out.slot_src,
                                 out.slot_kind, out.slot_mass, out.assign, ws.mem_row, ws.mem_slot, given, (T*)out.k_out,
                                 (T*)out.v_out, fw, ws.err);

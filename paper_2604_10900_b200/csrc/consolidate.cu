@@ -1102,9 +1102,10 @@ cudaError_t run(const Launch& L, const cask_params& prm, const float* s, const i
                              seed_of, sim, ws.grp, ws.seed_rows, ws.mass_fx, ws.njoin, unit_status, max_m, assign, weight, sl);
     } else if (fused) {
         Timed t(L, KID_SEEDS);
-        e = allow_smem(L, kSmemBitConsolidate + (sizeof(T) == 4), decide_small_kernel<T>, kMaxSpread);
+        size_t fixed = 0;
+        e = allow_smem(L, kSmemBitConsolidate + (sizeof(T) == 4), decide_small_kernel<T>, kMaxSpread, &fixed);
         if (e == cudaSuccess)
-            e = launch_dependent(L.stream, decide_small_kernel<T>, sh.n_units, kSmallThreads, spread_smem(L, sh.n_units, 17648, 0), L.desc, sh,
+            e = launch_dependent(L.stream, decide_small_kernel<T>, sh.n_units, kSmallThreads, spread_smem(L, sh.n_units, fixed, 0), L.desc, sh,
                                  tab, s, const_cast<int32_t*>(plan), kind, seed_of, sim, ws.grp, ws.seed_rows, ws.mass_fx, ws.njoin,
                                  unit_status, max_m, prm.eps);
     } else {
