@@ -1214,10 +1214,12 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     // Whether a pass may start while the kernel before it still runs (launch_dependent).  Its warps then take the slots that kernel's
     // leave, and where those are not the first ones of the SM the CTA runs up to 8 % slower, tile for tile, from the first to the
     // last: with the score pass of 288 units of 33,280 rows, a third of the CTAs (pass 1,260 to 1,360 us).  So a pass starts early
-    // only where it is short: the score pass below 24 tiles a CTA (events, early and not: 288 units of 33,280 rows 3,710 and 3,603
-    // us, 112 of 13,312 575 and 558, 112 of 8,448 403.4 and 399.5, 128 of 4,608 with 31 tiles 182.4 and 180.9; 8 of 33,280 with 28
-    // tiles 160 to 168 and 160, 288 of 640 144.1 and 149.3, 8 of 640 52.9 and 55.7), the normaliser pass, which finds few CTAs in
-    // its way, below 256 (288 units of 33,280 rows 3,603 and 3,574; 112 of 8,448 399.5 and 403.5).
+    // only where it is short.  Score pass, events early and not, by tiles a CTA: 7 tiles 105.2 and 107.2 us, 11 131.5 and 132.0,
+    // 14 160.1 and 163.6, 18 191.4 and 194.7, 21 213.9 and 215.8, 25 233.2 and 236.1, 28 261.3 and 262.4 (units of 8,448 rows, 512
+    // query rows), but 28 160 to 168 and 160 (8 of 33,280), 31 182.4 and 180.9 (128 of 4,608 at head_dim 64), 50 403.4 and 399.5 (112
+    // of 8,448), 112 746 and 743, 506 3,710 and 3,603: the line lies where the sign begins to depend on the shape.  Normaliser pass,
+    // which finds few CTAs in its way: early is better by 0.4 to 1.5 % up to 28 tiles, from 112 to 506 the two are within the
+    // 1 % that the runs differ by (506: 3,603 and 3,574, 3,549 and 3,510).
     const int bit = kSmemBitScore + 2 * (NB >> 1) + 6 * PLAIN + 12 * SPLIT;
     cudaError_t e = lse_in ? cudaSuccess : allow_smem(L, bit, norm, smem);
     if (e == cudaSuccess) e = allow_smem(L, bit + 1, mass, smem);

@@ -20,7 +20,12 @@ pytestmark = pytest.mark.gpu
     (5, 78, 128, 64, 9),      # 390 rows: six of its rows, window not a multiple of 16
     (2, 130, 128, 16, 100),   # 260 rows: the third block half filled, no fourth
     (3, 128, 96, 0, 64),      # 384 rows: three whole blocks
-    (15, 60, 128, 0, 20),     # 900 rows: two row groups of 448 and 452
+    (7, 64, 96, 16, 90),      # 448 rows below head_dim 113: the general form of the kernels
+    (3, 100, 64, 0, 31),      # 300 rows there
+    (10, 48, 128, 0, 61),     # 480 rows, a block of 32 columns in two heads
+    (13, 60, 128, 64, 77),    # 780 rows: two row groups of 416 and 364, the fourth block a quarter filled and empty
+    (14, 64, 128, 0, 99),     # 896 rows: two row groups of 448
+    (15, 60, 128, 0, 20),     # 900 rows: two row groups of 480 and 420
     (7, 96, 72, 0, 33),       # 672 rows: three row groups of two blocks
     (8, 128, 128, 0, 77),     # 1,024 rows: two row groups of four blocks
     (9, 128, 128, 128, 10),   # 1,152 rows: five row groups, the last one short
