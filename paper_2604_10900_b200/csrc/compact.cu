@@ -1,6 +1,8 @@
 // Compaction to the budget (Sec. 2.3: |R| <= B) with the weighted K/V merge of Sec. 2.4:
 //   slot order = ascending anchor row; kinds 1..3 and lone seeds are byte copies;
 //   a seed with joiners holds sum_i w_i k_i, sum_i w_i v_i (members in ascending row order).
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace cask {
@@ -899,7 +901,7 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     __shared__ unsigned totals, wsum[kFusedWarps];
     __shared__ int list[kListCap];                                         // members slot by slot
     int* src = reinterpret_cast<int*>(copy_smem + staging_bytes(kLongStage));   // [slots] 2 * row + (1: a seed) of a slot, ascending
-    int* start = src + slots;                                              // [slots + 1] first of a slot's members
+    int* start = src + slots + 1;                                          // [slots + 1] first of a slot's members (start[-1]: 0)
     // in the staging area until the copies begin: row and slot of the members; kept rows and members before every cell
     int* m_row = reinterpret_cast<int*>(copy_smem);
     int* m_slot = m_row + kListCap;
@@ -917,7 +919,7 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
         busy_slot = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int t = tid; t <= slots; t += kLongThreads) start[t] = 0;
+    for (int t = tid; t <= slots + 1; t += kLongThreads) start[t - 1] = 0;
     __syncthreads();                                         // (with given lists the counting begins at once)
     pdl_wait();
     const UnitDesc& ud = desc[u];
@@ -1075,41 +1077,46 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
             }
         __syncthreads();
         // ---- slot of every kept and merged row, their weights, the slot tables
-        // (four members a thread, the loads of each kind together: with thousands of members the loop is a chain of memory latencies)
-        constexpr int kU = 4;
-        for (int e0 = tid; e0 < nm; e0 += kU * kLongThreads) {
-            int row[kU], sd[kU], gi[kU], t[kU];
-            float am[kU];
-            uint8_t kd[kU];
+        // (With thousands of members the loop is a chain of memory latencies: four a thread then, the loads of each kind together.  A few
+        // hundred are one round either way, and take 2 to 8 us longer with the loads of three more.)
+        auto settle_members = [&](auto u_) {
+            constexpr int kU = decltype(u_)::value;
+            for (int e0 = tid; e0 < nm; e0 += kU * kLongThreads) {
+                int row[kU], sd[kU], gi[kU], t[kU];
+                float am[kU];
+                uint8_t kd[kU];
 #pragma unroll
-            for (int q = 0; q < kU; ++q) {
-                const int e = min(e0 + q * kLongThreads, nm - 1);
-                row[q] = in_smem ? m_row[e] : CASK_IDX(mem_row[o + e], T_, err);
-                t[q] = in_smem ? m_slot[e] : -3;
-            }
-#pragma unroll
-            for (int q = 0; q < kU; ++q) {
-                const bool mine = row[q] >= f0 && row[q] < f1;
-                sd[q] = seed_of[o + row[q]];                     // (a seed points at itself)
-                gi[q] = fw.s && mine ? fw.grp[o + row[q]] : -1;
-                kd[q] = in_smem ? (uint8_t)CASK_KIND_MERGED : ku[row[q]];
-            }
-#pragma unroll
-            for (int q = 0; q < kU; ++q) am[q] = gi[q] >= 0 ? row_mass(sh, s, eps, o + row[q]) : 0.f;
-#pragma unroll
-            for (int q = 0; q < kU; ++q) {
-                if (e0 + q * kLongThreads >= nm) break;
-                const int i = row[q];
-                if (t[q] == -3 && kd[q] == CASK_KIND_SEED) t[q] = slot_of(i);
-                else if (t[q] < -1) {
-                    t[q] = slot_of(sd[q]);
-                    if (i >= f0 && i < f1) assign[o + i] = t[q];
+                for (int q = 0; q < kU; ++q) {
+                    const int e = min(e0 + q * kLongThreads, nm - 1);
+                    row[q] = in_smem ? m_row[e] : CASK_IDX(mem_row[o + e], T_, err);
+                    t[q] = in_smem ? m_slot[e] : -3;
                 }
-                if (in_smem) m_slot[e0 + q * kLongThreads] = t[q];
-                if (t[q] >= 0) atomicAdd(&start[t[q]], 1);
-                if (gi[q] >= 0 && gi[q] < fw.max_m) weight[o + i] = am[q] / fx_to_mass(fw.mass_fx[(size_t)u * (fw.max_m + 1) + gi[q]]);
+#pragma unroll
+                for (int q = 0; q < kU; ++q) {
+                    const bool mine = row[q] >= f0 && row[q] < f1;
+                    sd[q] = seed_of[o + row[q]];                     // (a seed points at itself)
+                    gi[q] = fw.s && mine ? fw.grp[o + row[q]] : -1;
+                    kd[q] = in_smem ? (uint8_t)CASK_KIND_MERGED : ku[row[q]];
+                }
+#pragma unroll
+                for (int q = 0; q < kU; ++q) am[q] = gi[q] >= 0 ? row_mass(sh, s, eps, o + row[q]) : 0.f;
+#pragma unroll
+                for (int q = 0; q < kU; ++q) {
+                    if (e0 + q * kLongThreads >= nm) break;
+                    const int i = row[q];
+                    if (t[q] == -3 && kd[q] == CASK_KIND_SEED) t[q] = slot_of(i);
+                    else if (t[q] < -1) {
+                        t[q] = slot_of(sd[q]);
+                        if (i >= f0 && i < f1) assign[o + i] = t[q];
+                    }
+                    if (in_smem) m_slot[e0 + q * kLongThreads] = t[q];
+                    if (t[q] >= 0) atomicAdd(&start[t[q]], 1);
+                    if (gi[q] >= 0 && gi[q] < fw.max_m) weight[o + i] = am[q] / fx_to_mass(fw.mass_fx[(size_t)u * (fw.max_m + 1) + gi[q]]);
+                }
             }
-        }
+        };
+        if (in_smem) settle_members(std::integral_constant<int, 1>{});
+        else settle_members(std::integral_constant<int, 4>{});
         for (int t = tid; t < nk; t += kLongThreads) {
             const int i = src[t] >> 1;
             if (i < f0 || i >= f1) continue;
@@ -1178,7 +1185,7 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     else {
         // The members in row order, kListCap at a time: their slots by all warps but the first, which places the kListCap before them.
         // start[t] moves along and ends up as the end of slot t's members.  (The unit's other CTAs write the same.)
-        int* chunk[2] = {m_row, m_row + 2 * kListCap};              // rows, slots
+        auto chunk = [&](int b) { return m_row + 2 * kListCap * b; };       // rows, slots
         auto look_up = [&](int e0, int* rows, int first, int step) {
             constexpr int kU = 5;                                   // (224 threads: one round)
             const int n = min(kListCap, nm - e0);
@@ -1198,13 +1205,13 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
                 }
             }
         };
-        look_up(0, chunk[0], tid, kLongThreads);
+        look_up(0, chunk(0), tid, kLongThreads);
         __syncthreads();
         for (int e0 = 0, b = 0; e0 < nm; e0 += kListCap, b ^= 1) {
             if (w > 0) {
-                look_up(e0 + kListCap, chunk[b ^ 1], tid - 32, kLongThreads - 32);
+                look_up(e0 + kListCap, chunk(b ^ 1), tid - 32, kLongThreads - 32);
             } else {
-                const int* rows = chunk[b];
+                const int* rows = chunk(b);
                 const int n = min(kListCap, nm - e0);
                 for (int x0 = 0; x0 < n; x0 += 32) {
                     const int x = x0 + lane, t = x < n ? rows[kListCap + x] : -1;
@@ -1225,10 +1232,11 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     __syncthreads();
     // ---- batches of slots
     const RowSource<T> in{K, V, s, weight, eps, fw, ud, sh, u};
+    const int at = in_smem ? 0 : -1;                         // (placed in the workspace: start[t] is the end of slot t's members)
+    const int* members = in_smem ? list : mem_slot + o;
     copy_batches<T, CH, kLongStage>(
         in, nk, parts, part, copy_smem, bars, &next_batch, &abort_, k_out, v_out, slot_mass, Bmax, err, nm > 4 * nk ? 1 : 32, busy_slot,
-        [&](int t) { return src[t] >> 1; }, [&](int t) { return in_smem ? start[t] : t > 0 ? start[t - 1] : 0; },
-        [&](int e) { return in_smem ? list[e] : mem_slot[o + e]; });
+        [&](int t) { return src[t] >> 1; }, [&](int t) { return start[t + at]; }, [&](int e) { return members[e]; });
     late_flags(fw, sh.n_units, err);
 }
 
