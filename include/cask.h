@@ -246,7 +246,8 @@ int cask_selftest_wait_timeout(cask_ctx* ctx, uint64_t limit_ns, void* ws, size_
  */
 int cask_selftest_exp_rate(cask_ctx* ctx, int32_t iters, void* ws, size_t ws_bytes, double* rate_host);
 
-/* Bytes of workspace that any call below needs for this batch (host-only arithmetic). */
+/* Bytes of workspace that any call below needs for this batch (host-only arithmetic).  For an fp32 cache with head_dim
+ * <= 128 that includes three bf16 parts of every key and query: one and a half times their own bytes. */
 size_t cask_workspace_bytes(const cask_batch* batch, const cask_params* params);
 
 /*
