@@ -10,8 +10,8 @@
 // One persistent CTA per SM, 20 warps:
 //   warp 0      TMA producer (one lane): Q once per segment, K tiles through a ring of 2 to 4 stages
 //   warps 1-2   one lane each issues tcgen05.mma and the commits: warp 1 for the even accumulator
-//               slots, warp 2 for the odd ones, so that one keeps the tensor pipe fed while the other
-//               waits for a slot to be released (warp 1 also owns the TMEM allocation)
+//               slots, warp 2 for the odd ones (pass S with four blocks: slots 0-1 and 2-3), so that one keeps the
+//               tensor pipe fed while the other waits for a slot to be released (warp 1 also owns the TMEM allocation)
 //   warps 4-19  epilogue: tcgen05.ld of the fp32 accumulators + the exponentials
 // The 512 TMEM columns are four accumulator slots of 128 columns (one 128-row block of
 // queries each).  The epilogue warps form two groups of eight (two per TMEM lane quadrant, 64
@@ -484,6 +484,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     constexpr int kStages = C::kStages, kTps = C::kTps;
     constexpr int kRows = 128;                               // query rows per slot
     constexpr uint32_t kQRegionBytes = C::kQRegionBytes;
+    constexpr bool kPairs = PASS == 1 && NB == 4;            // a contraction fills two neighbouring slots
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* q_smem = smem;
@@ -669,6 +670,52 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                         if (!ok) break;
                         if (mine) tc_commit(&bar.d_full[j]);
                         if (t == nt - 1) tc_commit(&bar.q_empty[0]);
+                    }
+                    continue;
+                }
+                // Pass S with four query blocks: blocks 2i and 2i + 1 lie behind one another in shared memory and their slots in TMEM, so
+                // one instruction contracts the tile with both (N = 256; issuer i).  It reads the tile's operand once instead of twice:
+                // 2,048 clk a tile where the 128-column form takes 2,280, and 7 % less energy, which is time under the power limit
+                // (alone, back to back: 1,733 against 1,610 TFLOP/s sustained; cta_group::2 with M = N = 256 gives no more).  Score
+                // pass: 3,072 units of 640 rows 340 to 315 us, 112 of 8,448 139 to 133, 288 of 33,280 1,493 to 1,479.
+                if constexpr (kPairs) {
+                    const int i0 = 2 * j0;                            // first of the issuer's two blocks
+                    for (int t = 0; t < nt && ok; ++t, ++kit) {
+                        const int st = kit % kStages;
+                        ok = mbar_wait<true>(&bar.k_full[st], (kit / kStages) & 1u, abort_flag);
+                        if (!ok) break;
+                        const int cols = min(256, (rgs.per - kRows * i0 + 63) & ~63);          // (the rows of 64-row halves in use; <= 0: none)
+                        const bool two = cols > kRows;
+                        if (t == 0) {
+                            ok = mbar_wait<true>(&bar.q_full[i0], seg & 1u, abort_flag);
+                            if (ok) ok = mbar_wait<true>(&bar.q_full[i0 + 1], seg & 1u, abort_flag);
+                            if (!ok) break;
+                        }
+                        if (cols > 0) {
+                            ok = mbar_wait<true>(&bar.d_empty[i0], (use[0] & 1u) ^ 1u, abort_flag);
+                            if (ok && two) ok = mbar_wait<true>(&bar.d_empty[i0 + 1], (use[0] & 1u) ^ 1u, abort_flag);
+                            if (!ok) break;
+                            ++use[0];
+                            tc_fence_after();
+                            const uint32_t kst_lo = k_lo + st * (kKStageBytes >> 4);
+                            const uint32_t qblk_lo = q_lo + ((j0 * 2 * kQRegionBytes) >> 4), idesc = umma_idesc(cols);
+                            tc_mma_lo<false>(tmem_base + 128 * i0, kst_lo, qblk_lo, idesc);
+#pragma unroll
+                            for (int kk = 1; kk < 8; ++kk) {
+                                const int kb = kk >> 2, ks = kk & 3;
+                                if (kk >= n_ks) break;
+                                tc_mma_lo<true>(tmem_base + 128 * i0, kst_lo + ((kb * kKRegionBytes + ks * 32) >> 4),
+                                                qblk_lo + ((kb * kQRegionBytes + ks * 32) >> 4), idesc);
+                            }
+                            tc_commit(&bar.d_full[i0]);
+                            if (two) tc_commit(&bar.d_full[i0 + 1]);
+                        }
+                        tc_commit(&bar.k_empty[st]);
+                        if (t == nt - 1) {
+                            // last use of the segment's query blocks
+                            tc_commit(&bar.q_empty[i0]);
+                            tc_commit(&bar.q_empty[i0 + 1]);
+                        }
                     }
                     continue;
                 }
