@@ -261,18 +261,11 @@ struct TileWalk {
     }
 };
 
-// CTA that owns tile x when `total` tiles are split over `grid` CTAs as in TileWalk::init.
-template <typename I>
-__device__ __forceinline__ int owner_cta_as(I x, I total, I grid) {
-    I b = (x * grid) / total;
-    while (b + 1 < grid && (total * (b + 1)) / grid <= x) ++b;
-    while (b > 0 && (total * b) / grid > x) --b;
-    return (int)b;
-}
-// 32-bit divisions when total * grid fits (a 64-bit division is a sequence of a hundred instructions)
-__device__ __forceinline__ int owner_cta(long long x, long long total, long long grid) {
-    if (total * grid < (1ll << 31)) return owner_cta_as<uint32_t>((uint32_t)x, (uint32_t)total, (uint32_t)grid);
-    return owner_cta_as<long long>(x, total, grid);
+// CTA that owns tile x when `total` tiles are split over `grid` CTAs as in TileWalk::init: the last b with total * b / grid <= x, that
+// is with b * total < (x + 1) * grid.  (32-bit division when it fits: a 64-bit one is a sequence of a hundred instructions.)
+__device__ __forceinline__ int owner_cta(int x, int total, int grid) {
+    const unsigned long long n = (unsigned long long)(x + 1) * grid - 1;
+    return n < (1ull << 32) ? (int)((uint32_t)n / (uint32_t)total) : (int)(n / (uint32_t)total);
 }
 
 // First normaliser partial of a row and their number, for a unit's (and row group's) tiles [tile0, tile0 + n_tiles).
@@ -298,7 +291,8 @@ __device__ __noinline__ void fill_rows(const RowDefaults& f, int64_t first, int 
 // logit into its share of the score, roww * 2^(y - rowm) = 2^(y + rc), rc = log2(roww) - rowm.  rowm is the greatest reference of
 // the row's (reference, sum) partials (one per CTA of the normaliser pass that had tiles of the unit, and column half; NB = 1:
 // and group), roww = 1/(rows * sum 2^(y - rowm)), the sums added in the order of the partials.  With caller-supplied natural-log
-// normalisers: rowm = lse*log2(e), roww = 1/rows.  `n` threads share the rows; `first` hands the normalisers out.
+// normalisers: rowm = lse*log2(e), roww = 1/rows.  `n` threads share the rows; `first` hands the normalisers out.  part_step: floats
+// from a partial of a row to the next (rgs.per).
 //
 // The score pass makes its own tables when most CTAs have one segment or two (units x row groups up to the CTAs): the epilogue's
 // threads the first one, the warp that has nothing else to do the later ones, ahead of time.  That saves a launch with the
@@ -309,7 +303,7 @@ template <int kU>                            // partials in flight per row
 __device__ __forceinline__ void make_row_table(int u, int rg, int lo, int cnt, bool first, const RowGroups& rgs, int nb,
                                                const float* __restrict__ part_m, const float* __restrict__ part_l,
                                                const float* __restrict__ lse_in, float* __restrict__ lse_out, float* __restrict__ rc,
-                                               int limit, int idx, int n) {
+                                               int limit, int idx, int n, int part_step) {
     const int rows = rgs.count(rg), parts = nb == 1 ? 4 : 2;
     const size_t ou = (size_t)u * rgs.rows + rg * rgs.per;
     const float inv_rows = 1.f / (float)rgs.rows;
@@ -322,7 +316,7 @@ __device__ __forceinline__ void make_row_table(int u, int rg, int lo, int cnt, b
         }
         return;
     }
-    const size_t p0 = ((size_t)parts * (u * rgs.groups + rg) + lo) * rgs.per;
+    const size_t p0 = ((size_t)parts * (u * rgs.groups + rg) + lo) * part_step;
     for (int r = idx; r < limit; r += n) {
         if (r >= rows) { rc[r] = -1.0e30f; continue; }
         const float *pm = part_m + p0 + r, *pl = part_l + p0 + r;
@@ -330,7 +324,7 @@ __device__ __forceinline__ void make_row_table(int u, int rg, int lo, int cnt, b
         auto load = [&](int b, bool sums) {
 #pragma unroll
             for (int x = 0; x < kU; ++x) {
-                const int at = min(b + x, cnt - 1) * rgs.per;
+                const int at = min(b + x, cnt - 1) * part_step;
                 vm[x] = pm[at];
                 if (sums) vl[x] = pl[at];
             }
@@ -355,10 +349,10 @@ __device__ __forceinline__ void make_row_table(int u, int rg, int lo, int cnt, b
 __device__ __noinline__ void row_table(int u, int rg, int T, int tile0, bool first, const RowGroups& rgs, int nb, int total_tiles,
                                        int grid, const float* __restrict__ part_m, const float* __restrict__ part_l,
                                        const float* __restrict__ lse_in, float* __restrict__ lse_out, float* __restrict__ rc, int idx,
-                                       int n) {
+                                       int n, int part_step) {
     int lo = 0, cnt = 1;
     if (!lse_in) partial_range(tile0, T, nb, total_tiles, grid, lo, cnt);
-    make_row_table<8>(u, rg, lo, cnt, first, rgs, nb, part_m, part_l, lse_in, lse_out, rc, 512, idx, n);
+    make_row_table<8>(u, rg, lo, cnt, first, rgs, nb, part_m, part_l, lse_in, lse_out, rc, 512, idx, n, part_step);
 }
 
 __device__ __forceinline__ void copy_table(const float* __restrict__ tables, int u, int rg, const RowGroups& rgs, float* rc, int idx, int n) {
@@ -383,7 +377,7 @@ __global__ void __launch_bounds__(kRowThreads) score_row_tables(const UnitDesc* 
     }
     __syncthreads();
     make_row_table<4>(u, rg, range[0], range[1], true, rgs, nb, part_m, part_l, nullptr, lse_out,
-                      tables + (size_t)u * rgs.rows + rg * rgs.per, rgs.count(rg), threadIdx.x, kRowThreads);
+                      tables + (size_t)u * rgs.rows + rg * rgs.per, rgs.count(rg), threadIdx.x, kRowThreads, rgs.per);
 }
 
 // Rows by which query block b is turned inside its 128 TMEM lanes in the normaliser pass: lane l holds row (l + turn) mod 128 of
@@ -479,7 +473,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 const UnitDesc* __restrict__ desc, Shape sh, RowGroups rgs, float scale2, int total_tiles, int sub_rows,
                 float* __restrict__ part_m, float* __restrict__ part_l, const float* __restrict__ lse_in,
                 float* __restrict__ lse_out, const float* __restrict__ tables, float* __restrict__ s, int64_t s_group_stride,
-                const __grid_constant__ RowDefaults fill, int32_t* __restrict__ err) {
+                const __grid_constant__ RowDefaults fill, int ahead, const float* __restrict__ scratch, int32_t* __restrict__ err) {
     using C = Cfg<NB, SPLIT>;
     constexpr int kStages = C::kStages, kTps = C::kTps;
     constexpr int kRows = 128;                               // query rows per slot
@@ -519,7 +513,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tail->tmem_base;
-    pdl_wait();
+    // Pass S started under pass N (`ahead`): descriptors, keys and queries are older than pass N, so the keys and queries are
+    // fetched and contracted at once, and only what needs the normalisers waits for its end.  (The fence: nothing that this SM's L1
+    // still holds of the descriptors of an earlier call is read.)
+    if (PASS == 0 || !ahead) pdl_wait();
+    else __threadfence();
 
     TileWalk<!PLAIN || SPLIT> wk;
     wk.init(desc, sh.n_units, total_tiles, rgs.groups);
@@ -774,6 +772,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         }
     } else if (warp == 3) {
         // ================= pass S: row tables of the later segments, up to two segments ahead; row defaults =================
+        if (PASS == 1 && ahead) pdl_wait();
         if (PASS == 1 && wk.valid()) {
             bool ok = true;
             auto fill_segment = [&](const TileWalk<!PLAIN || SPLIT>& f) {
@@ -790,7 +789,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     if (tables) copy_table(tables, wk.u, wk.rg(), rgs, tail->rc[buf], lane, 32);
                     else
                         row_table(wk.u, wk.rg(), wk.T, wk.tile0, wk.t == wk.tile0, rgs, NB, total_tiles, gridDim.x, part_m, part_l, lse_in,
-                                  lse_out, tail->rc[buf], lane, 32);
+                                  lse_out, tail->rc[buf], lane, 32, rgs.per);
                     __syncwarp();
                     // table 0's barrier counts the epilogue's warps: stand in for them
                     if (lane < (buf == 0 ? kEpiWarps : 1)) mbar_arrive(&bar.rw_full[buf]);
@@ -828,18 +827,26 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
         for (int i = 0; i < kStates; ++i) { mm[i] = kNegBig; l_run[i] = 0.f; }
 
+        if (PASS == 1 && ahead) {
+            // The code of the row tables once through on nothing while pass N still runs: fetching its instructions is most of what
+            // the first table costs (one partial address for all, out of `scratch`, into the room of the key sums).
+            if (!tables && wk.valid())
+                row_table(wk.u, 0, wk.T, wk.tile0, false, rgs, NB, total_tiles, gridDim.x, scratch, scratch, nullptr, nullptr,
+                          &tail->red[0][0][0], etid, 32 * kEpiWarps, 0);
+            pdl_wait();
+        }
         if (PASS == 1 && wk.valid()) {
             if (tables) copy_table(tables, wk.u, wk.rg(), rgs, tail->rc[0], etid, 32 * kEpiWarps);
             else
                 row_table(wk.u, wk.rg(), wk.T, wk.tile0, wk.t == wk.tile0, rgs, NB, total_tiles, gridDim.x, part_m, part_l, lse_in, lse_out,
-                          tail->rc[0], etid, 32 * kEpiWarps);
+                          tail->rc[0], etid, 32 * kEpiWarps, rgs.per);
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar.rw_full[0]);
             TileWalk<!PLAIN || SPLIT> nx = wk;
             nx.next_segment();
             if (spread_unit(nx)) {                       // the second table as well: see there
                 row_table(nx.u, nx.rg(), nx.T, nx.tile0, nx.t == nx.tile0, rgs, NB, total_tiles, gridDim.x, part_m, part_l, lse_in, lse_out,
-                          tail->rc[1], etid, 32 * kEpiWarps);
+                          tail->rc[1], etid, 32 * kEpiWarps, rgs.per);
                 asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
                 if (etid == 0) mbar_arrive(&bar.rw_full[1]);
             }
@@ -1260,20 +1267,21 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     const auto norm = score_tc_kernel<0, NB, PLAIN, SPLIT>, mass = score_tc_kernel<1, NB, PLAIN, SPLIT>;
     // Whether a pass may start while the kernel before it still runs (launch_dependent).  Its warps then take the slots that kernel's
     // leave, and where those are not the first ones of the SM the CTA runs up to 8 % slower, tile for tile, from the first to the
-    // last: with the score pass of 288 units of 33,280 rows, a third of the CTAs (pass 1,260 to 1,360 us).  So a pass starts early
-    // only where it is short.  Score pass, events early and not, by tiles a CTA: 7 tiles 105.2 and 107.2 us, 11 131.5 and 132.0,
-    // 14 160.1 and 163.6, 18 191.4 and 194.7, 21 213.9 and 215.8, 25 233.2 and 236.1, 28 261.3 and 262.4 (units of 8,448 rows, 512
-    // query rows), but 28 160 to 168 and 160 (8 of 33,280), 31 182.4 and 180.9 (128 of 4,608 at head_dim 64), 50 403.4 and 399.5 (112
-    // of 8,448), 112 746 and 743, 506 3,710 and 3,603: the line lies where the sign begins to depend on the shape.  Normaliser pass,
-    // which finds few CTAs in its way: early is better by 0.4 to 1.5 % up to 28 tiles, from 112 to 506 the two are within the
-    // 1 % that the runs differ by (506: 3,603 and 3,574, 3,549 and 3,510).
+    // last: with the score pass of 288 units of 33,280 rows, a third of the CTAs (pass 1,260 to 1,360 us).
+    // With given normalisers the score pass gains nothing but the launch, and starts early only where it is short: 7 to 28 tiles a CTA
+    // 0.4 to 2 % better (units of 8,448 rows, 512 query rows), but 28 of eight units of 33,280 rows 160 to 168 and 160 us.
+    // Behind the normaliser pass it has its first keys, queries and contractions done and its code fetched by the end of that pass
+    // (`ahead`): events of 8 units of 640 rows 54.0 to 49.9 us (0.3 tiles a CTA), two fp32 ones of 1,024 52.1 to 50.0, 128 of 4,608 at
+    // head_dim 64 (31 tiles) 182 to 176; from 50 to 112 tiles even, within the runs' 0.7 %, 506 tiles 3,575 and 3,582.
+    // Normaliser pass, which finds few CTAs in its way: early is better by 0.4 to 1.5 % up to 28 tiles, from 112 to 506 the two are
+    // within the 1 % that the runs differ by (506: 3,603 and 3,574, 3,549 and 3,510).
     const int bit = kSmemBitScore + 2 * (NB >> 1) + 6 * PLAIN + 12 * SPLIT;
     cudaError_t e = lse_in ? cudaSuccess : allow_smem(L, bit, norm, smem);
     if (e == cudaSuccess) e = allow_smem(L, bit + 1, mass, smem);
     if (e == cudaSuccess && !lse_in) {
         Timed t(L, KID_SCORE_NORM);
         e = launch_kernel(total < 256 * grid, L.stream, norm, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
-                             ws.part_l, nullptr, nullptr, nullptr, nullptr, 0, RowDefaults{}, ws.err);
+                             ws.part_l, nullptr, nullptr, nullptr, nullptr, 0, RowDefaults{}, 0, nullptr, ws.err);
     }
     const bool ahead = !lse_in && sh.n_units * rg.groups > grid;       // the row tables by a kernel of their own
     if (e == cudaSuccess && ahead) {
@@ -1284,8 +1292,10 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     }
     if (e == cudaSuccess) {
         Timed t(L, KID_SCORE_MASS);
-        e = launch_kernel(total < 24 * grid, L.stream, mass, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
-                             ws.part_l, lse_in, lse_out, ahead ? ws.rowm : nullptr, rg.groups > 1 ? ws.s_part : s, rg.groups > 1 ? L.sum_T : 0, L.fill, ws.err);
+        const bool early = total < (lse_in ? 24 : 256) * grid;
+        e = launch_kernel(early, L.stream, mass, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
+                             ws.part_l, lse_in, lse_out, ahead ? ws.rowm : nullptr, rg.groups > 1 ? ws.s_part : s, rg.groups > 1 ? L.sum_T : 0, L.fill,
+                             early && !lse_in, ws.roww, ws.err);
         ws.filled = L.fill.kind != nullptr;
         if (e == cudaSuccess && rg.groups > 1) {
             const int per = kFoldThreads * kFoldKeys;
