@@ -483,27 +483,28 @@ struct RowSource {
     int u;
 };
 
-// A warp takes a batch of consecutive slots: bulk copies of their rows into its staging buffer, then two bulk stores, because
-// consecutive slots are contiguous in the output; two buffers, so the copies of a batch run under the stores of the one
-// before.  A slot that others joined is not copied: while the batch's copies are in flight the warp adds up the members'
-// rows (ascending row order, fp32, rounded once) and puts the result in the slot's place in the buffer, so every output row
-// is written once and the members' latency hides behind the copies.
+// Two kinds of work, handed out to the warps of a unit's CTAs one after the other:
+//   * the slots that others joined, `per_item` of them at a time: their members' rows are added up (ascending row order, fp32, rounded
+//     once) and written out.  A lane looks one member up (page, score, carried mass, group mass) and the rows are loaded kRows at
+//     a time whatever slots they feed.  (Eight rows spill, and the bf16 kernels are slower with them.)  They come first: a
+//     group is a chain of memory latencies, three and one more per four members.
+//   * batches of consecutive slots: bulk copies of the rows of the other ones into the warp's staging buffer, then bulk stores, two
+//     for a batch without merged slots, because consecutive slots are contiguous in the output; two buffers, so the copies of a
+//     batch run under the stores of the one before.
+// per_item: one group where the chip is not full, so that no warp has several of them to add up while others have none, else four,
+// which share their latencies.  With the groups of a batch of slots added up by the warp that copies the batch, a few warps had
+// most of the members of a unit, since the slots with members lie together, and the kernel waited for them.  Event of 128 units of
+// 4,608 rows at head_dim 64 178 to 173 us, 8 of 33,280 164.4 to 160.6, 112 of 13,312 556 to 549, 3,072 of 640 1,190 to 1,164, 8 of
+// 640 50.0 to 48.3.
 //   row_of(slot) -> cache row; first(slot) -> place in the list of the slot's first member (first(nk): the end).
-//   member(place) -> cache row.  The members of all merged slots of the batch are taken together: a lane looks one member up (page,
-//   score, carried mass, group mass), and the rows are loaded kRows at a time whatever slots they feed, so a batch of small
-//   groups waits once or twice for memory and not once a group.  (Eight rows spill, and the bf16 kernels are slower with them.)
-//   most: slots a batch has at the most.  With groups of hundreds of members a warp takes them one by one, or some warps would have
-//   several of them to add up and others none (32 units of 8,448 rows of which all others join: kernel 440 to 251 us).
-//   busy_slot: the first slot with members.  Its batch is taken first and the copies that wait for nothing last, since the slots
-//   with members lie together: their batches at the end were the tail of the kernel.
-// One group at a time in slot order -> members together -> busy batches first: 3,072 units of 640 rows 346 / 337 / 329 us, 288 of
-// them 44.8 / 40.9 / 36.5, 288 of 33,280 78 / 71 / 63, 112 of 8,448 40.7 / 38.7 / 35.4.
+//   member(place) -> cache row; busy(i), i < n_busy -> slots, all those with two members or more among them.
 // CH > 0: head_dim == 32 * CH, a lane owns CH contiguous channels; CH == 0: any head_dim up to 256, channels lane, lane + 32, ...
-template <typename T, int CH, int STAGE, typename RowOf, typename First, typename Member>
+template <typename T, int CH, int STAGE, typename RowOf, typename First, typename Member, typename Busy>
 __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int parts, int part, uint8_t* staging,
-                                             uint64_t (*bars)[2], int* next_batch, int* abort_word, T* __restrict__ k_out,
+                                             uint64_t (*bars)[2], int* next_item, int* abort_word, T* __restrict__ k_out,
                                              T* __restrict__ v_out, float* __restrict__ slot_mass, int Bmax,
-                                             int32_t* __restrict__ err, int most, int busy_slot, RowOf row_of, First first, Member member) {
+                                             int32_t* __restrict__ err, int per_item, int n_busy, RowOf row_of, First first, Member member,
+                                             Busy busy) {
     using namespace tc;
     constexpr int kPer = CH > 0 ? CH : 8;
     constexpr int kRows = 4;                     // member rows in flight
@@ -513,45 +514,24 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, u = in.u, d = sh.d;
     const int64_t o = ud.tok_off;
     const uint32_t row_bytes = CH > 0 ? (uint32_t)(32 * CH * sizeof(T)) : (uint32_t)(d * sizeof(T));
-    const int sb = min(min(32, (int)(STAGE / 2 / row_bytes)), most);       // slots per batch
+    const int sb = min(32, (int)(STAGE / 2 / row_bytes));                  // slots per batch
     volatile int* abort_flag = abort_word;
     uint8_t* my = staging + w * 2 * STAGE;
-    const int nb = (nk + sb - 1) / sb, first_b = min(busy_slot, max(nk - 1, 0)) / sb;
+    const int nb = (nk + sb - 1) / sb, n_items = (n_busy + per_item - 1) / per_item;
     uint32_t it = 0;
     bool ok = true;
     while (ok) {
         int b = 0;
-        if (lane == 0) b = atomicAdd(next_batch, 1);
+        if (lane == 0) b = atomicAdd(next_item, 1);
         b = __shfl_sync(0xffffffffu, b, 0) * parts + part;
-        if (b >= nb) break;
-        b += first_b;
-        const int t0 = (b >= nb ? b - nb : b) * sb;
-        const int nv = min(sb, nk - t0);
-        const uint32_t st = it & 1u;
-        uint8_t* kbuf = my + st * STAGE;
-        uint8_t* vbuf = kbuf + STAGE / 2;
-        const int t = t0 + lane;
-        const int f = lane < nv ? first(t) : 0, members = lane < nv ? first(t + 1) - f : 0;
-        const bool merged = members > 1;
-        const unsigned todo = __ballot_sync(0xffffffffu, merged);
-        // the stores that read this buffer two batches ago must have read it
-        if (lane == 0) {
-            asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-            mbar_expect_tx(&bars[w][st], (uint32_t)(nv - __popc(todo)) * 2u * row_bytes);
-        }
-        __syncwarp();
-        if (lane < nv && !merged) {
-            const int row = CASK_IDX(row_of(t), ud.T, err);
-            const T* kr = in.K + row_elem_off(sh, ud, ud.k_off, row);
-            const T* vr = in.V + v_elem_off(sh, ud, u, row);
-            const uint32_t bar = smem_u32(&bars[w][st]);
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"(smem_u32(kbuf + lane * row_bytes)), "l"(kr), "r"(row_bytes), "r"(bar) : "memory");
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"(smem_u32(vbuf + lane * row_bytes)), "l"(vr), "r"(row_bytes), "r"(bar) : "memory");
-            slot_mass[(size_t)u * Bmax + t] = row_mass(sh, in.s, in.eps, o + row);
-        }
-        if (todo) {
+        if (b >= n_items + nb) break;
+        if (b < n_items) {
+            // ---- merged slots, a lane a slot
+            const bool mine = lane < per_item && b * per_item + lane < n_busy;
+            const int t = mine ? busy(b * per_item + lane) : 0;
+            const int f = mine ? first(t) : 0, members = mine ? first(t + 1) - f : 0;
+            const bool merged = members > 1;
+            if (!__any_sync(0xffffffffu, merged)) continue;
             float mg_t = 0.f;                      // group mass of slot t (event path: the weights are formed here)
             if (in.fw.s && merged) {
                 const int gi = min(max(CASK_IDX(in.fw.grp[o + row_of(t)], max(in.fw.max_m, 1), err), 0), in.fw.max_m);
@@ -564,8 +544,8 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
                 for (int x = 0; x < kPer; ++x) { ak[x] = 0.f; av[x] = 0.f; }
             };
             auto finish = [&](int sl) {
-                T* kw = reinterpret_cast<T*>(kbuf + sl * row_bytes);
-                T* vw = reinterpret_cast<T*>(vbuf + sl * row_bytes);
+                T* kw = k_out + ((size_t)u * Bmax + sl) * d;
+                T* vw = v_out + ((size_t)u * Bmax + sl) * d;
                 if (CH > 0) {
                     Vec k1, v1;
 #pragma unroll
@@ -583,11 +563,11 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
                             Elem<T>::st(vw + lane + 32 * x, av[x]);
                         }
                 }
-                if (lane == 0) slot_mass[(size_t)u * Bmax + t0 + sl] = msum;
+                if (lane == 0) slot_mass[(size_t)u * Bmax + sl] = msum;
             };
             clear();
             const int count = merged ? members : 0;
-            int before = count;                // members of the batch's slots below this one
+            int before = count;                // members of the item's slots below this one
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
                 const int x = __shfl_up_sync(0xffffffffu, before, off);
@@ -637,28 +617,55 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
                             }
                         }
                         if ((ends >> (c0 + q)) & 1u) {
-                            finish(__shfl_sync(0xffffffffu, sl, c0 + q));
+                            finish(__shfl_sync(0xffffffffu, t, __shfl_sync(0xffffffffu, sl, c0 + q)));
                             clear();
                         }
                     }
                 }
             }
+            continue;
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the merged rows, before the bulk stores read them
+        // ---- rows to copy
+        const int t0 = (b - n_items) * sb;
+        const int nv = min(sb, nk - t0);
+        const uint32_t st = it & 1u;
+        uint8_t* kbuf = my + st * STAGE;
+        uint8_t* vbuf = kbuf + STAGE / 2;
+        const int t = t0 + lane;
+        const bool copied = lane < nv && first(t + 1) - first(t) < 2;
+        const int n_copied = __popc(__ballot_sync(0xffffffffu, copied));
+        // the stores that read this buffer two batches ago must have read it (every lane has groups of its own)
+        asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        if (lane == 0) mbar_expect_tx(&bars[w][st], (uint32_t)n_copied * 2u * row_bytes);
+        __syncwarp();
+        if (copied) {
+            const int row = CASK_IDX(row_of(t), ud.T, err);
+            const T* kr = in.K + row_elem_off(sh, ud, ud.k_off, row);
+            const T* vr = in.V + v_elem_off(sh, ud, u, row);
+            const uint32_t bar = smem_u32(&bars[w][st]);
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(smem_u32(kbuf + lane * row_bytes)), "l"(kr), "r"(row_bytes), "r"(bar) : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(smem_u32(vbuf + lane * row_bytes)), "l"(vr), "r"(row_bytes), "r"(bar) : "memory");
+            slot_mass[(size_t)u * Bmax + t] = row_mass(sh, in.s, in.eps, o + row);
+        }
         ok = mbar_wait(&bars[w][st], (it >> 1) & 1u, abort_flag);
         __syncwarp();
         if (!ok) break;
-        if (lane == 0) {
-            const size_t dst = ((size_t)u * Bmax + t0) * d;
+        // a batch without merged slots in two pieces, else slot by slot
+        const bool whole = n_copied == nv;
+        if (whole ? lane == 0 : copied) {
+            const size_t dst = ((size_t)u * Bmax + t) * d;
+            const uint32_t from = lane * row_bytes, bytes = whole ? (uint32_t)nv * row_bytes : row_bytes;
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                         ::"l"(k_out + dst), "r"(smem_u32(kbuf)), "r"((uint32_t)nv * row_bytes) : "memory");
+                         ::"l"(k_out + dst), "r"(smem_u32(kbuf) + from), "r"(bytes) : "memory");
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                         ::"l"(v_out + dst), "r"(smem_u32(vbuf)), "r"((uint32_t)nv * row_bytes) : "memory");
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                         ::"l"(v_out + dst), "r"(smem_u32(vbuf) + from), "r"(bytes) : "memory");
         }
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         ++it;
     }
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (!ok && lane == 0) {
         // a copy that was started may still be landing: give the barrier a bounded chance to complete
         for (uint32_t k = 0; k < 4096 && !mbar_try(&bars[w][it & 1u], (it >> 1) & 1u); ++k) {}
@@ -710,9 +717,10 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 3) compact_small_kernel(
     static_assert(kIters * kFusedWarps == 32, "one cell per lane");
     extern __shared__ __align__(128) uint8_t copy_smem[];
     __shared__ uint64_t bars[kFusedWarps][2];
-    __shared__ int abort_, next_batch, busy_slot;              // busy_slot: the first one with members
+    __shared__ int abort_, next_item, n_busy;
     __shared__ unsigned cell[32], totals, wsum[kFusedWarps];
     __shared__ int16_t src[kSmallRows], list[kSmallRows];      // row of a slot; members slot by slot
+    __shared__ int16_t busy[kSmallRows / 2];                   // slots with two members or more
     __shared__ int start[kSmallRows + 1];                      // first of a slot's members
     // tables of the scan, in the staging area until the copies begin
     int16_t* slot_of = reinterpret_cast<int16_t*>(copy_smem);  // slot a row feeds
@@ -725,8 +733,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 3) compact_small_kernel(
     if (tid == 0) {
         for (int i = 0; i < kFusedWarps; ++i) { mbar_init(&bars[i][0], 1); mbar_init(&bars[i][1], 1); }
         abort_ = 0;
-        next_batch = 0;
-        busy_slot = 0;
+        next_item = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int t = tid; t <= kSmallRows; t += kThreads) start[t] = 0;
@@ -814,9 +821,9 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 3) compact_small_kernel(
     }
     __syncthreads();
     {
-        int c[kIters], sum = 0;
+        int c[kIters], sum = 0;                     // members, slots with two or more << 16 (in slot order: every CTA of the unit the same)
 #pragma unroll
-        for (int q = 0; q < kIters; ++q) { c[q] = start[kIters * tid + q]; sum += c[q]; }
+        for (int q = 0; q < kIters; ++q) { c[q] = start[kIters * tid + q]; sum += c[q] + ((c[q] > 1) << 16); }
         int incl = sum;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -829,11 +836,11 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 3) compact_small_kernel(
         for (int x = 0; x < w; ++x) run += (int)wsum[x];
 #pragma unroll
         for (int q = 0; q < kIters; ++q) {
-            start[kIters * tid + q] = run;
-            if (run == 0 && c[q] > 0) busy_slot = kIters * tid + q;
-            run += c[q];
+            start[kIters * tid + q] = run & 0xFFFF;
+            if (c[q] > 1) busy[run >> 16] = (int16_t)(kIters * tid + q);
+            run += c[q] + ((c[q] > 1) << 16);
         }
-        if (tid == kThreads - 1) start[kSmallRows] = run;
+        if (tid == kThreads - 1) { start[kSmallRows] = run & 0xFFFF; n_busy = run >> 16; }
     }
     __syncthreads();
     for (int e = tid; e < nm; e += kThreads) {
@@ -848,8 +855,9 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 3) compact_small_kernel(
     // ---- batches of slots
     const RowSource<T> in{K, V, s, weight, eps, fw, ud, sh, u};
     copy_batches<T, CH, kSmallStage>(
-        in, nk, parts, part, copy_smem, bars, &next_batch, &abort_, k_out, v_out, slot_mass, Bmax, err, 32, busy_slot,
-        [&](int t) { return (int)src[t]; }, [&](int t) { return start[t]; }, [&](int e) { return (int)list[e]; });
+        in, nk, parts, part, copy_smem, bars, &next_item, &abort_, k_out, v_out, slot_mass, Bmax, err, parts > 1 ? 1 : 4, n_busy,
+        [&](int t) { return (int)src[t]; }, [&](int t) { return start[t]; }, [&](int e) { return (int)list[e]; },
+        [&](int i) { return (int)busy[i]; });
     late_flags(fw, sh.n_units, err);
 }
 
@@ -897,9 +905,10 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     using namespace tc;
     extern __shared__ __align__(128) uint8_t copy_smem[];
     __shared__ uint64_t bars[kFusedWarps][2];
-    __shared__ int abort_, next_batch, busy_slot;              // busy_slot: the first one with members
+    __shared__ int abort_, next_item, n_busy;
     __shared__ unsigned totals, wsum[kFusedWarps];
     __shared__ int list[kListCap];                                         // members slot by slot
+    __shared__ uint16_t busy[kListCap / 2];                                // slots with two members or more
     int* src = reinterpret_cast<int*>(copy_smem + staging_bytes(kLongStage));   // [slots] 2 * row + (1: a seed) of a slot, ascending
     int* start = src + slots + 1;                                          // [slots + 1] first of a slot's members (start[-1]: 0)
     // in the staging area until the copies begin: row and slot of the members; kept rows and members before every cell
@@ -915,8 +924,7 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     if (tid == 0) {
         for (int i = 0; i < kFusedWarps; ++i) { mbar_init(&bars[i][0], 1); mbar_init(&bars[i][1], 1); }
         abort_ = 0;
-        next_batch = 0;
-        busy_slot = 0;
+        next_item = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int t = tid; t <= slots + 1; t += kLongThreads) start[t - 1] = 0;
@@ -1142,8 +1150,12 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     // ---- counts -> first places, then every member's place: the first one of its slot, plus the earlier members of the slot
     {
         const int per = (nk + kLongThreads - 1) / kLongThreads, t0 = min(nk, tid * per), t1 = min(nk, t0 + per);
+        // (members in shared memory, at most kListCap: the slots with two or more are counted along in the upper half, in slot order, so
+        // that every CTA of the unit numbers them the same way)
+        auto step = [&](int n) { return n + (in_smem && n > 1 ? 1 << 16 : 0); };
+        const int low = in_smem ? 0xFFFF : -1;
         int sum = 0;
-        for (int t = t0; t < t1; ++t) sum += start[t];
+        for (int t = t0; t < t1; ++t) sum += step(start[t]);
         int incl = sum;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -1156,11 +1168,11 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
         for (int x = 0; x < w; ++x) run += (int)wsum[x];
         for (int t = t0; t < t1; ++t) {
             const int n = start[t];
-            start[t] = run;
-            if (run == 0 && n > 0) busy_slot = t;
-            run += n;
+            start[t] = run & low;
+            if (n > 1 && in_smem) busy[run >> 16] = (uint16_t)t;
+            run += step(n);
         }
-        if (tid == kLongThreads - 1) start[nk] = run;        // the last thread ends on the total
+        if (tid == kLongThreads - 1) { start[nk] = run & low; n_busy = in_smem ? run >> 16 : nk; }        // the last thread ends on the total
     }
     __syncthreads();
     if (in_smem)
@@ -1235,8 +1247,9 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     const int at = in_smem ? 0 : -1;                         // (placed in the workspace: start[t] is the end of slot t's members)
     const int* members = in_smem ? list : mem_slot + o;
     copy_batches<T, CH, kLongStage>(
-        in, nk, parts, part, copy_smem, bars, &next_batch, &abort_, k_out, v_out, slot_mass, Bmax, err, nm > 4 * nk ? 1 : 32, busy_slot,
-        [&](int t) { return src[t] >> 1; }, [&](int t) { return start[t + at]; }, [&](int e) { return members[e]; });
+        in, nk, parts, part, copy_smem, bars, &next_item, &abort_, k_out, v_out, slot_mass, Bmax, err, parts > 1 || !in_smem ? 1 : 4,
+        n_busy, [&](int t) { return src[t] >> 1; }, [&](int t) { return start[t + at]; },
+        [&](int e) { return members[e]; }, [&](int i) { return in_smem ? (int)busy[i] : i; });
     late_flags(fw, sh.n_units, err);
 }
 
