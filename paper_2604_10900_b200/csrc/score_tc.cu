@@ -829,9 +829,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 
         if (PASS == 1 && ahead) {
             // The code of the row tables once through on nothing while pass N still runs: fetching its instructions is most of what
-            // the first table costs (one partial address for all, out of `scratch`, into the room of the key sums).
+            // the first table costs (one partial address for all, out of `scratch`, into the room of the key sums).  A unit of one tile
+            // (the 1): one round over the partials, whatever the segment's own unit has.  The rounds of a unit that many CTAs share go on
+            // when pass N, short there, is long over: event of four units of 9,000 rows 79.4 us with them, 72.5 without.
             if (!tables && wk.valid())
-                row_table(wk.u, 0, wk.T, wk.tile0, false, rgs, NB, total_tiles, gridDim.x, scratch, scratch, nullptr, nullptr,
+                row_table(wk.u, 0, 1, wk.tile0, false, rgs, NB, total_tiles, gridDim.x, scratch, scratch, nullptr, nullptr,
                           &tail->red[0][0][0], etid, 32 * kEpiWarps, 0);
             pdl_wait();
         }

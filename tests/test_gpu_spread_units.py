@@ -29,3 +29,27 @@ def test_scores_of_few_long_units(units, decode, group, window):
     for u in range(units):
         a = int(hb.tok_off[u])
         assert abs(float(got["s"][a:a + int(hb.T[u])].sum()) - 1.0) < 1e-4
+
+
+def _kernel_us(hb, name, **kw):
+    """Shortest of eight profiled times of one kernel of the event, and the event's normalisers."""
+    import gpu_harness as gh
+    run = gh.GpuRun(hb, **kw)
+    run.out_struct.rho_core = run.out_struct.rho_rep = run.out_struct.dispersion = None        # (no diagnostics)
+    best = np.inf
+    for _ in range(8):
+        run.ctx.profile_enable(True)
+        g = run.event()
+        best = min(best, run.ctx.profile_read()[name]["ms"] * 1e3)
+        run.ctx.profile_enable(False)
+    return best, g["lse"]
+
+
+def test_a_rows_partials_are_walked_once():
+    """One unit on all CTAs has two partials a CTA and row, and their fold is most of the score pass: three times what the pass takes
+    with given normalisers, which has none (five times when a trial run of the table's code went over as many again)."""
+    hb = wl.make_batch(wl.WORKLOADS["reasoning8k_b384"].with_(layers=1, kv_heads=1, group=4, window=128, prefix=100, decode=18800, budget=512,
+                                                              reserve=256))
+    own, lse = _kernel_us(hb, "score_mass")
+    given, _ = _kernel_us(hb, "score_mass", lse_in=lse)
+    assert own < 4.0 * given, (own, given)
