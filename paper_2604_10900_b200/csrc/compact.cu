@@ -491,11 +491,15 @@ struct RowSource {
 //   * batches of consecutive slots: bulk copies of the rows of the other ones into the warp's staging buffer, then bulk stores, two
 //     for a batch without merged slots, because consecutive slots are contiguous in the output; two buffers, so the copies of a
 //     batch run under the stores of the one before.
-// per_item: one group where the chip is not full, so that no warp has several of them to add up while others have none, else four,
-// which share their latencies.  With the groups of a batch of slots added up by the warp that copies the batch, a few warps had
-// most of the members of a unit, since the slots with members lie together, and the kernel waited for them.  Event of 128 units of
-// 4,608 rows at head_dim 64 178 to 173 us, 8 of 33,280 164.4 to 160.6, 112 of 13,312 556 to 549, 3,072 of 640 1,190 to 1,164, 8 of
-// 640 50.0 to 48.3.
+// With the groups of a batch of slots added up by the warp that copies the batch, a few warps had most of the members of a unit, since the
+// slots with members lie together, and the kernel waited for them.  Kernel alone, with them and now: 128 units of 4,608 rows at head_dim
+// 64 35.8 and 31.2 us, 112 of 13,312 71.9 and 65.8, 112 of 9,000 32.8 and 27.6, 3,072 of 640 300 and 290, 8 of 640 17.2 and 14.9.
+// per_item (kernel alone, us): one where a unit has several CTAs, so that no warp has several groups to add up while others have none: 8
+// units of 3,000 rows 17.1, with four 21.3; 112 of 1,900 31.3, 36.9.  Else four, which share their latencies: 240 units of 1,024
+// of which all others join 62.0, with one 72.1; 3,072 of 640 338, 362 (eight: 337).
+// Units of more than kListCap members have no list of the slots with members, and all slots are looked through: eight consecutive ones
+// at a time, 240 units of 9,000 rows (2,048 kept) of which all others join 561, with one 703; of 3,000 (1,536) 211, 296; but one
+// where groups have more than four members on average: 112 of 9,000 (512) 313, with four 381, with eight 530.
 //   row_of(slot) -> cache row; first(slot) -> place in the list of the slot's first member (first(nk): the end).
 //   member(place) -> cache row; busy(i), i < n_busy -> slots, all those with two members or more among them.
 // CH > 0: head_dim == 32 * CH, a lane owns CH contiguous channels; CH == 0: any head_dim up to 256, channels lane, lane + 32, ...
@@ -699,7 +703,7 @@ __device__ __forceinline__ void write_status(const FusedWeights& fw, int u) {
 
 // ---- units of at most kSmallRows rows: scan, copy and merge in one kernel -----------------------------------------------
 // `parts` CTAs per unit, each with the unit's whole scan in shared memory (a thousand rows: cheaper than a kernel that hands
-// it over) and every parts-th batch of slots (copy_batches).  Bound by HBM and, with few units, by latency; three CTAs of
+// it over) and every parts-th item of work (copy_batches).  Bound by HBM and, with few units, by latency; three CTAs of
 // 74 KB per SM keep about 140 KB in flight.
 // 3,072 paged units of 640 rows (512 kept, bf16, d = 128): 314 us = 5.1 TB/s of rows in and out, where the scan, copy and merge
 // kernels took 29 + 420; 288 such units 35 us (80 before), 8 units 15 (33 before, each with its launch).
@@ -1246,8 +1250,9 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     const RowSource<T> in{K, V, s, weight, eps, fw, ud, sh, u};
     const int at = in_smem ? 0 : -1;                         // (placed in the workspace: start[t] is the end of slot t's members)
     const int* members = in_smem ? list : mem_slot + o;
+    const int per_item = in_smem ? (parts > 1 ? 1 : 4) : (nm > 4 * nk ? 1 : 8);
     copy_batches<T, CH, kLongStage>(
-        in, nk, parts, part, copy_smem, bars, &next_item, &abort_, k_out, v_out, slot_mass, Bmax, err, parts > 1 || !in_smem ? 1 : 4,
+        in, nk, parts, part, copy_smem, bars, &next_item, &abort_, k_out, v_out, slot_mass, Bmax, err, per_item,
         n_busy, [&](int t) { return src[t] >> 1; }, [&](int t) { return start[t + at]; },
         [&](int e) { return members[e]; }, [&](int i) { return in_smem ? (int)busy[i] : i; });
     late_flags(fw, sh.n_units, err);

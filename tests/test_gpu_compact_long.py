@@ -111,6 +111,33 @@ def test_thousands_of_members_cost_a_fraction_more():
     assert all_join < 4.0 * none_joins, (all_join, none_joins)
 
 
+def test_members_of_small_groups_share_their_latencies():
+    """Full chip, thousands of members a unit in groups of one or two beside the seed: compaction with all scratch rows joined against none
+    (2.2 times; 3.1 when every slot, copied ones too, was handed out by itself)."""
+    import gpu_harness as gh
+    w = wl.WORKLOADS["reasoning8k_b512"].with_(layers=1, kv_heads=1, prefix=200, decode=2800, budget=1536, reserve=768)
+    k, v, q = wl.make_unit(w, 0, 0, 0)
+    n, T = 240, 3000
+    full = lambda x: np.full(n, x, np.int32)
+    hb = wl.Batch(wl=w, k=np.tile(k, (n, 1)), v=np.tile(v, (n, 1)), q=np.tile(q[None], (n, 1, 1, 1)), T=full(T), P=full(200), B=full(1536),
+                  reserve=full(768), tok_off=np.arange(n + 1, dtype=np.int64) * T, unit_ids=[(i, 0, 0) for i in range(n)])
+
+    def best_us(tau):
+        run = gh.GpuRun(hb, tau=tau)
+        run.out_struct.rho_core = run.out_struct.rho_rep = run.out_struct.dispersion = None        # (no diagnostics)
+        best = np.inf
+        for _ in range(8):
+            run.ctx.profile_enable(True)
+            run.event()
+            best = min(best, run.ctx.profile_read()["gather_merge"]["ms"] * 1e3)
+            run.ctx.profile_enable(False)
+        return best, np.isin(run.out["kind"].cpu().numpy(), (4, 5)).sum() / n
+
+    (joined, many), (none, few) = best_us(-1.0), best_us(2.0)
+    assert 1024 < many < 4 * 1536 and few < 1024
+    assert joined < 2.65 * none, (joined, none)
+
+
 @pytest.mark.parametrize("specs,tau,page,dtype", [
     # (rows, prefix, budget, reserve): more slots than the one-kernel compaction has room for, beside shorter units
     ([(14000, 300, 12400, 12200), (1500, 20, 12300, 0), (13000, 12900, 12390, 50)], 0.9, 0, wl.DTYPE_BF16),
