@@ -159,7 +159,6 @@ __global__ void __launch_bounds__(kSelThreads, PER_SM) decide_long_kernel(
     extern __shared__ unsigned row_bits[];               // LISTS: [2][sl.words] kept rows, seeds
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     constexpr int kU = 8 / PER_SM;                       // rows a thread has in flight
-    constexpr int kSweep = 2 * kU;                       // (the first two sweeps of long units, which keep nothing of a row)
     pdl_wait();
     const int u = blockIdx.x;
     const UnitDesc& ud = desc[u];
@@ -179,8 +178,8 @@ __global__ void __launch_bounds__(kSelThreads, PER_SM) decide_long_kernel(
     unsigned mn[2] = {0xffffffffu, 0xffffffffu}, mx[2] = {0u, 0u};
     const int first = sel_p ? 0 : P, last = sel_a || sel_b ? hi : P;      // rows whose scores are looked at
     if constexpr (LISTS) {
-        if (sel_p) sweep_keys<kSweep>(su, 0, P, [&](unsigned k) { mn[0] = min(mn[0], k); mx[0] = max(mx[0], k); });
-        if (sel_a || sel_b) sweep_keys<kSweep>(su, P, hi, [&](unsigned k) { mn[1] = min(mn[1], k); mx[1] = max(mx[1], k); });
+        if (sel_p) sweep_keys<kU>(su, 0, P, [&](unsigned k) { mn[0] = min(mn[0], k); mx[0] = max(mx[0], k); });
+        if (sel_a || sel_b) sweep_keys<kU>(su, P, hi, [&](unsigned k) { mn[1] = min(mn[1], k); mx[1] = max(mx[1], k); });
         for (int x = tid; x < 2 * sl.words; x += kSelThreads) row_bits[x] = 0u;
     } else {
         for (int i0 = first + tid; i0 < last; i0 += kU * kSelThreads) {
@@ -217,8 +216,8 @@ __global__ void __launch_bounds__(kSelThreads, PER_SM) decide_long_kernel(
     }
     // ---- sweep 2: histograms
     if constexpr (LISTS) {
-        if (sel_p) sweep_keys<kSweep>(su, 0, P, [&](unsigned k) { atomicAdd(&sm.h.hist[0][(k - base[0]) >> shift[0]], 1u); });
-        if (sel_a || sel_b) sweep_keys<kSweep>(su, P, hi, [&](unsigned k) { atomicAdd(&sm.h.hist[1][(k - base[1]) >> shift[1]], 1u); });
+        if (sel_p) sweep_keys<kU>(su, 0, P, [&](unsigned k) { atomicAdd(&sm.h.hist[0][(k - base[0]) >> shift[0]], 1u); });
+        if (sel_a || sel_b) sweep_keys<kU>(su, P, hi, [&](unsigned k) { atomicAdd(&sm.h.hist[1][(k - base[1]) >> shift[1]], 1u); });
     } else {
         for (int i0 = first + tid; i0 < last; i0 += kU * kSelThreads) {
             float x[kU];
