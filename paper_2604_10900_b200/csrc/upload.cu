@@ -26,10 +26,13 @@ __global__ void __launch_bounds__(kThreads) desc_from_host(const uint4* __restri
                                                            uint4* __restrict__ err) {
     const int i = blockIdx.x * kThreads + threadIdx.x;
     uint4 d = make_uint4(0u, 0u, 0u, 0u);
-    // (Volatile: the compiler moves a plain load behind the wait, and the bus's latency with it: 3,072 units 13 us, 288 units 3 us.)
+    // (Volatile: the compiler moves a plain load behind the wait, and the bus's latency with it: events of 100 to 600 units 2 to 3 us.)
     if (i < n16)
         asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(d.x), "=r"(d.y), "=r"(d.z), "=r"(d.w) : "l"(src + i));
-    pdl_wait();
+    // (No early start of the next kernel: the normaliser pass's CTAs then found these in their way, where the kernel before leaves room
+    // for some of them only.  432 units of 640 rows, compaction CTAs on all but 12 places of the chip: event 212.8 to 204.4 us, 207 with
+    // the staging read behind the wait; 296 to 1,332 units within 1 %.)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (i == 0) *err = make_uint4(0u, 0u, 0u, 0u);
     if (i < n16) dst[i] = d;
 }
