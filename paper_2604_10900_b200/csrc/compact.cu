@@ -498,8 +498,9 @@ struct RowSource {
 // units of 3,000 rows 17.1, with four 21.3; 112 of 1,900 31.3, 36.9.  Else four, which share their latencies: 240 units of 1,024
 // of which all others join 62.0, with one 72.1; 3,072 of 640 338, 362 (eight: 337).
 // Units of more than kListCap members have no list of the slots with members, and all slots are looked through: eight consecutive ones
-// at a time, 240 units of 9,000 rows (2,048 kept) of which all others join 561, with one 703; of 3,000 (1,536) 211, 296; but one
-// where groups have more than four members on average: 112 of 9,000 (512) 313, with four 381, with eight 530.
+// at a time, 240 units of 9,000 rows (2,048 kept) of which all others join 559, with one 703; of 3,000 (1,536) 211, 296.  But one where
+// groups have more than four members on average, 112 of 9,000 (512) 313, with four 381, with eight 530; or more than two and there are
+// fewer than four items of eight a warp: 112 of 1,900 (512) 92, with eight 99; 40 of them 60, 76.
 //   row_of(slot) -> cache row; first(slot) -> place in the list of the slot's first member (first(nk): the end).
 //   member(place) -> cache row; busy(i), i < n_busy -> slots, all those with two members or more among them.
 // CH > 0: head_dim == 32 * CH, a lane owns CH contiguous channels; CH == 0: any head_dim up to 256, channels lane, lane + 32, ...
@@ -1250,7 +1251,10 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     const RowSource<T> in{K, V, s, weight, eps, fw, ud, sh, u};
     const int at = in_smem ? 0 : -1;                         // (placed in the workspace: start[t] is the end of slot t's members)
     const int* members = in_smem ? list : mem_slot + o;
-    const int per_item = in_smem ? (parts > 1 ? 1 : 4) : (nm > 4 * nk ? 1 : 8);
+    int one = nm > 4 * nk || (nm > 2 * nk && nk < 256 * parts);
+    // (Opaque: known to depend on the counts, it makes other code of the whole kernel, 25 % slower at head_dim 64; in fp32 14 % faster.)
+    asm volatile("" : "+r"(one));
+    const int per_item = in_smem ? (parts > 1 ? 1 : 4) : (one ? 1 : 8);
     copy_batches<T, CH, kLongStage>(
         in, nk, parts, part, copy_smem, bars, &next_item, &abort_, k_out, v_out, slot_mass, Bmax, err, per_item,
         n_busy, [&](int t) { return src[t] >> 1; }, [&](int t) { return start[t + at]; },
