@@ -142,7 +142,8 @@ inline size_t spread_smem(const Launch& L, int64_t grid, size_t fixed, size_t ne
 // Kernels of a call follow one another by programmatic dependent launch: a kernel launched with launch_dependent() may start
 // while the one before it still runs, sets itself up (barriers, TMEM, descriptors of the operands) and calls pdl_wait() before
 // it touches anything that kernel wrote.  pdl_wait() returns when every kernel before has completed, and only then lets the
-// next one start, so that at most two kernels of a call are on the device.  Together with the descriptors' upload by a kernel
+// next one start, so that at most two kernels of a call are on the device.  (The order of the two is relied upon: the score pass, started
+// under the normaliser pass, reads what was complete when that pass came back from its wait without waiting itself.)  Together with the descriptors' upload by a kernel
 // (upload.cu): events on 8 units of 640 rows 85.5 to 73.1 us, 128 units of 4,608 rows at head_dim 64 230 to 219, 16 fp32 units
 // of 8,448 rows 331 to 307, events of milliseconds unchanged.
 __device__ __forceinline__ void pdl_wait() {

@@ -1252,7 +1252,7 @@ __global__ void __launch_bounds__(kLongThreads, 3) compact_long_kernel(
     const int at = in_smem ? 0 : -1;                         // (placed in the workspace: start[t] is the end of slot t's members)
     const int* members = in_smem ? list : mem_slot + o;
     int one = nm > 4 * nk || (nm > 2 * nk && nk < 256 * parts);
-    // (Opaque: known to depend on the counts, it makes other code of the whole kernel, 25 % slower at head_dim 64; in fp32 14 % faster.)
+    // (Opaque: with the counts in view the compiler makes other code of the whole kernel, 25 % slower at head_dim 64.)
     asm volatile("" : "+r"(one));
     const int per_item = in_smem ? (parts > 1 ? 1 : 4) : (one ? 1 : 8);
     copy_batches<T, CH, kLongStage>(

@@ -66,7 +66,7 @@ constexpr int kSlots = 4;                 // accumulator slots of 128 TMEM colum
 constexpr int kEpiWarp0 = 4;
 constexpr int kEpiWarps = 4 * kSlots;
 constexpr int kThreadsTc = (kEpiWarp0 + kEpiWarps) * 32;
-constexpr int kIssuers = 2;               // one per epilogue group
+constexpr int kIssuers = 2;               // two slots each: an epilogue group's, or (pass S, NB = 4) two neighbours
 constexpr uint32_t kQBlockBytes = 128 * 128;           // one 128-row query block inside a region
 constexpr uint32_t kKRegionBytes = 128 * 128;          // 128 keys x 64 bf16
 constexpr uint32_t kKStageBytes = 2 * kKRegionBytes;
@@ -513,9 +513,12 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tail->tmem_base;
-    // Pass S started under pass N (`ahead`): descriptors, keys and queries are older than pass N, so the keys and queries are
-    // fetched and contracted at once, and only what needs the normalisers waits for its end.  (The fence: nothing that this SM's L1
-    // still holds of the descriptors of an earlier call is read.)
+    // Pass S started under pass N (`ahead`): keys and queries are fetched and contracted at once, and only what needs the
+    // normalisers waits for the end of pass N.  What is read before that (descriptors, block table, keys, queries, the parts of fp32 rows)
+    // was complete, in the memory that all SMs see, when pass N came back from its wait, and pass S is not let go before all of that
+    // pass's CTAs have come back: pdl_wait() waits first and releases afterwards.  With score_row_tables between the two, pass N itself is
+    // over.  Nothing changes it while pass S runs.  (The fence drops what this SM's L1 may hold of an earlier call's; reading past the
+    // L1 instead costs eight units of 640 rows 0.3 us of 49.6.)
     if (PASS == 0 || !ahead) pdl_wait();
     else __threadfence();
 
@@ -673,41 +676,39 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 }
                 // Pass S with four query blocks: blocks 2i and 2i + 1 lie behind one another in shared memory and their slots in TMEM, so
                 // one instruction contracts the tile with both (N = 256; issuer i).  It reads the tile's operand once instead of twice:
-                // 2,048 clk a tile where the 128-column form takes 2,280, and 7 % less energy, which is time under the power limit
-                // (alone, back to back: 1,733 against 1,610 TFLOP/s sustained; cta_group::2 with M = N = 256 gives no more).  Score
+                // 2,048 clk a tile where the 128-column form takes 2,280 (a loop of nothing but these instructions on one tile).  Score
                 // pass: 3,072 units of 640 rows 340 to 315 us, 112 of 8,448 139 to 133, 288 of 33,280 1,493 to 1,479.
                 if constexpr (kPairs) {
                     const int i0 = 2 * j0;                            // first of the issuer's two blocks
+                    // the rows of 64-row halves in use (row_plan takes four blocks from 257 rows a group up: both issuers have some)
+                    const int cols = min(256, (rgs.per - kRows * i0 + 63) & ~63);
+                    const bool two = cols > kRows;
+                    const uint32_t idesc = umma_idesc(cols), qblk_lo = q_lo + ((j0 * 2 * kQRegionBytes) >> 4);
                     for (int t = 0; t < nt && ok; ++t, ++kit) {
                         const int st = kit % kStages;
                         ok = mbar_wait<true>(&bar.k_full[st], (kit / kStages) & 1u, abort_flag);
                         if (!ok) break;
-                        const int cols = min(256, (rgs.per - kRows * i0 + 63) & ~63);          // (the rows of 64-row halves in use; <= 0: none)
-                        const bool two = cols > kRows;
                         if (t == 0) {
                             ok = mbar_wait<true>(&bar.q_full[i0], seg & 1u, abort_flag);
                             if (ok) ok = mbar_wait<true>(&bar.q_full[i0 + 1], seg & 1u, abort_flag);
                             if (!ok) break;
                         }
-                        if (cols > 0) {
-                            ok = mbar_wait<true>(&bar.d_empty[i0], (use[0] & 1u) ^ 1u, abort_flag);
-                            if (ok && two) ok = mbar_wait<true>(&bar.d_empty[i0 + 1], (use[0] & 1u) ^ 1u, abort_flag);
-                            if (!ok) break;
-                            ++use[0];
-                            tc_fence_after();
-                            const uint32_t kst_lo = k_lo + st * (kKStageBytes >> 4);
-                            const uint32_t qblk_lo = q_lo + ((j0 * 2 * kQRegionBytes) >> 4), idesc = umma_idesc(cols);
-                            tc_mma_lo<false>(tmem_base + 128 * i0, kst_lo, qblk_lo, idesc);
+                        ok = mbar_wait<true>(&bar.d_empty[i0], (use[0] & 1u) ^ 1u, abort_flag);
+                        if (ok && two) ok = mbar_wait<true>(&bar.d_empty[i0 + 1], (use[0] & 1u) ^ 1u, abort_flag);
+                        if (!ok) break;
+                        ++use[0];
+                        tc_fence_after();
+                        const uint32_t kst_lo = k_lo + st * (kKStageBytes >> 4);
+                        tc_mma_lo<false>(tmem_base + 128 * i0, kst_lo, qblk_lo, idesc);
 #pragma unroll
-                            for (int kk = 1; kk < 8; ++kk) {
-                                const int kb = kk >> 2, ks = kk & 3;
-                                if (kk >= n_ks) break;
-                                tc_mma_lo<true>(tmem_base + 128 * i0, kst_lo + ((kb * kKRegionBytes + ks * 32) >> 4),
-                                                qblk_lo + ((kb * kQRegionBytes + ks * 32) >> 4), idesc);
-                            }
-                            tc_commit(&bar.d_full[i0]);
-                            if (two) tc_commit(&bar.d_full[i0 + 1]);
+                        for (int kk = 1; kk < 8; ++kk) {
+                            const int kb = kk >> 2, ks = kk & 3;
+                            if (kk >= n_ks) break;
+                            tc_mma_lo<true>(tmem_base + 128 * i0, kst_lo + ((kb * kKRegionBytes + ks * 32) >> 4),
+                                            qblk_lo + ((kb * kQRegionBytes + ks * 32) >> 4), idesc);
                         }
+                        tc_commit(&bar.d_full[i0]);
+                        if (two) tc_commit(&bar.d_full[i0 + 1]);
                         tc_commit(&bar.k_empty[st]);
                         if (t == nt - 1) {
                             // last use of the segment's query blocks
@@ -1274,7 +1275,8 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     // 0.4 to 2 % better (units of 8,448 rows, 512 query rows), but 28 of eight units of 33,280 rows 160 to 168 and 160 us.
     // Behind the normaliser pass it has its first keys, queries and contractions done and its code fetched by the end of that pass
     // (`ahead`): events of 8 units of 640 rows 54.0 to 49.9 us (0.3 tiles a CTA), two fp32 ones of 1,024 52.1 to 50.0, 128 of 4,608 at
-    // head_dim 64 (31 tiles) 182 to 176; from 50 to 112 tiles even, within the runs' 0.7 %, 506 tiles 3,575 and 3,582.
+    // head_dim 64 (31 tiles) 182 to 176; 24 to 60 tiles 0.5 to 2.5 % (100 units of 11,366 rows 485.7 to 479.4), 90 to 200 up to 1.5, 250 and
+    // 300 even, 400 and 600 up to 1 % worse (400 units of 28,416 rows 4,259 and 4,305).
     // Normaliser pass, which finds few CTAs in its way: early is better by 0.4 to 1.5 % up to 28 tiles, from 112 to 506 the two are
     // within the 1 % that the runs differ by (506: 3,603 and 3,574, 3,549 and 3,510).
     const int bit = kSmemBitScore + 2 * (NB >> 1) + 6 * PLAIN + 12 * SPLIT;
@@ -1285,8 +1287,8 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
         e = launch_kernel(total < 256 * grid, L.stream, norm, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
                              ws.part_l, nullptr, nullptr, nullptr, nullptr, 0, RowDefaults{}, 0, nullptr, ws.err);
     }
-    const bool ahead = !lse_in && sh.n_units * rg.groups > grid;       // the row tables by a kernel of their own
-    if (e == cudaSuccess && ahead) {
+    const bool own_tables = !lse_in && sh.n_units * rg.groups > grid;       // the row tables by a kernel of their own
+    if (e == cudaSuccess && own_tables) {
         Timed t(L, KID_ROW_COMBINE);
         // (never early: its CTAs would hold slots of the score pass that follows; 288 units of 640 rows 149.4 to 148.2 us)
         e = launch_kernel(false, L.stream, score_row_tables, sh.n_units * rg.groups, kRowThreads, 0, L.desc, rg, NB, total, grid, ws.part_m,
@@ -1296,7 +1298,7 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
         Timed t(L, KID_SCORE_MASS);
         const bool early = total < (lse_in ? 24 : 256) * grid;
         e = launch_kernel(early, L.stream, mass, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
-                             ws.part_l, lse_in, lse_out, ahead ? ws.rowm : nullptr, rg.groups > 1 ? ws.s_part : s, rg.groups > 1 ? L.sum_T : 0, L.fill,
+                             ws.part_l, lse_in, lse_out, own_tables ? ws.rowm : nullptr, rg.groups > 1 ? ws.s_part : s, rg.groups > 1 ? L.sum_T : 0, L.fill,
                              early && !lse_in, ws.roww, ws.err);
         ws.filled = L.fill.kind != nullptr;
         if (e == cudaSuccess && rg.groups > 1) {
