@@ -706,7 +706,7 @@ __device__ __forceinline__ void write_status(const FusedWeights& fw, int u) {
 // `parts` CTAs per unit, each with the unit's whole scan in shared memory (a thousand rows: cheaper than a kernel that hands
 // it over) and every parts-th item of work (copy_batches).  Bound by HBM and, with few units, by latency; three CTAs of
 // 74 KB per SM keep about 140 KB in flight.
-// 3,072 paged units of 640 rows (512 kept, bf16, d = 128): 314 us = 5.1 TB/s of rows in and out, where the scan, copy and merge
+// 3,072 paged units of 640 rows (512 kept, bf16, d = 128): 301 us = 5.3 TB/s of rows in and out, where the scan, copy and merge
 // kernels took 29 + 420; 288 such units 35 us (80 before), 8 units 15 (33 before, each with its launch).
 constexpr int kSmallRows = 1024;
 

@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kSelThreads, PER_SM) decide_long_kernel(
             }
             for (; some; some &= some - 1) {
                 const int at = __ffs(some) - 1, i = i0 + at * kSelThreads;
-                float xi = x[0];                             // (picked out of the registers: a second load is another latency a row)
+                float xi = x[0];                             // (out of the registers: a second load is another latency a row, 300 units of 9,000 34.9 us for 33.1)
 #pragma unroll
                 for (int q = 1; q < kU; ++q) xi = at == q ? x[q] : xi;
                 const unsigned key = order_key(xi);
