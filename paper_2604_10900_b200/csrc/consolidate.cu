@@ -576,18 +576,23 @@ __global__ void __launch_bounds__(32 * kGatherWarps, 8) seed_gather_kernel(
 // memory; the boundary ranks come out of one histogram per range over the keys' own span, and rows inside a boundary bin are
 // ranked by counting, as in decide_long_kernel.  (Ranking every row by counting is quadratic: two units of 1,024 rows took
 // 34 us, now 12.)  Bound by latency, and with thousands of units by the seeds' scattered rows: half the time goes to the gather,
-// so the block table is read at the start and four rows a warp are in flight.  3,072 paged units of 640 rows 90 -> 72 us (80 with
-// the norms summed as they are, see gather_seeds).  Five
-// CTAs an SM: six spill more (68 us there, 50.6 against 49.0 for an event of two units), four leave too few warps (74).
-constexpr int kSmallThreads = 256;
-constexpr int kSmallBins = 4 * kSmallThreads;
-template <typename T>
-__global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
+// so the block table is read at the start and four rows a warp are in flight.
+// Threads a unit (THREADS, PER_SM): every step but the gather is a chain of short latencies, and the gather takes m / (4 * warps) rounds of
+// one more, so a unit that has an SM to itself gets as many threads as it has use for: 1,024, or 512 where it has no more rows.
+// With several units an SM the chains of one hide behind those of the others: 512 up to three units an SM, then 256.
+// Event in us with 256, 512 and 1,024: 8 units of 640 rows 50.5, 44.5, 44.5; 4 of 1,000 (m = 128) 61.8, 52.6, 50.6; 100 of 1,000 118, 108, 106;
+// 148 of 330 55.3, 54.1, 55.1; 200 of 640 115, 109, 113; 288 of 640 146, 137, 141; 440 of 640 191, 188; 600 of 1,000 410, 412; 1,200
+// of 640 462, 461; 3,072 of 640 1,136, 1,155.  256 threads four an SM, which spill nothing: kernel of those 3,072 78.9 to 70.5 us, where five
+// an SM (48 registers) spilled 96 bytes a thread; 512 three an SM (40 registers) 90.6.
+constexpr int kSmallBins = 1024;
+template <typename T, int THREADS, int PER_SM>
+__global__ void __launch_bounds__(THREADS, PER_SM) decide_small_kernel(
     const UnitDesc* __restrict__ desc, Shape sh, SeedTable<T> tab, const float* __restrict__ s, int32_t* __restrict__ plan,
     uint8_t* __restrict__ kind, int32_t* __restrict__ seed_of, float* __restrict__ sim, int32_t* __restrict__ grp,
     int32_t* __restrict__ seed_rows, unsigned long long* __restrict__ mass_fx, int32_t* __restrict__ njoin,
     int32_t* __restrict__ unit_status, int max_m, float eps) {
-    constexpr int kPer = kSmallSpan / kSmallThreads, kWarps = kSmallThreads / 32;
+    constexpr int kPer = kSmallSpan / THREADS, kWarps = THREADS / 32, kPerBin = kSmallBins / THREADS;
+    static_assert(kSmallSpan == kSmallBins && kPer >= 1 && kWarps <= 32, "rows and bins go to the threads alike");
     __shared__ alignas(16) unsigned keys[kSmallSpan];
     __shared__ uint8_t kd[kSmallSpan];
     __shared__ int32_t pages[kSmallSpan];                // the unit's block table: looked up before it is needed
@@ -611,14 +616,14 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
     const bool sel_p = P > pkeep && pkeep > 0, sel_a = c > 0 && c < span, sel_b = m > 0 && c + m < span;
     unsigned key[kPer];
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) key[q] = tid + q * kSmallThreads < T_ ? order_key(s[o + tid + q * kSmallThreads]) : 0u;
+    for (int q = 0; q < kPer; ++q) key[q] = tid + q * THREADS < T_ ? order_key(s[o + tid + q * THREADS]) : 0u;
     if (sh.page_size > 0)
-        for (int x = tid; x * sh.page_size < T_; x += kSmallThreads) pages[x] = sh.bt[ud.bt0 + x];
+        for (int x = tid; x * sh.page_size < T_; x += THREADS) pages[x] = sh.bt[ud.bt0 + x];
     // ---- key spans of the prefix (0) and the scratch range (1)
     unsigned mn[2] = {0xffffffffu, 0xffffffffu}, mx[2] = {0u, 0u};
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-        const int i = tid + q * kSmallThreads;
+        const int i = tid + q * THREADS;
         keys[i] = key[q];
         if (i < P) { mn[0] = min(mn[0], key[q]); mx[0] = max(mx[0], key[q]); }
         else if (i < hi) { mn[1] = min(mn[1], key[q]); mx[1] = max(mx[1], key[q]); }
@@ -646,16 +651,16 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
     auto bin_of = [&](int q, int g) { return (int)((key[q] - base[g]) >> shift[g]); };
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-        const int i = tid + q * kSmallThreads;
+        const int i = tid + q * THREADS;
         if (i < P ? sel_p : (i < hi && (sel_a || sel_b))) atomicAdd(&sm.hist[i >= P][i < P ? bin_of(q, 0) : bin_of(q, 1)], 1u);
     }
     __syncthreads();
-    // ---- bins that hold the ranks pkeep, c and c + m: each thread has four bins of either histogram, in descending order
+    // ---- bins that hold the ranks pkeep, c and c + m: each thread has kPerBin bins of either histogram, in descending order
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
-        unsigned h[4], tot = 0;
+        unsigned h[kPerBin], tot = 0;
 #pragma unroll
-        for (int x = 0; x < 4; ++x) { h[x] = sm.hist[g][kSmallBins - 1 - 4 * tid - x]; tot += h[x]; }
+        for (int x = 0; x < kPerBin; ++x) { h[x] = sm.hist[g][kSmallBins - 1 - kPerBin * tid - x]; tot += h[x]; }
         unsigned incl = tot;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -664,15 +669,14 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
         }
         if (lane == 31) wsum[g][w] = incl;
         __syncthreads();
-        unsigned before = incl - tot;
-        for (int x = 0; x < w; ++x) before += wsum[g][x];
+        unsigned before = incl - tot + __reduce_add_sync(0xffffffffu, lane < w ? wsum[g][lane] : 0u);
         const unsigned rank[2] = {(unsigned)(g == 0 ? (sel_p ? pkeep : 0) : (sel_a ? c : 0)), (unsigned)(g == 1 && sel_b ? c + m : 0)};
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
+        for (int x = 0; x < kPerBin; ++x) {
 #pragma unroll
             for (int k = 0; k < 2; ++k)
                 if (rank[k] > before && rank[k] <= before + h[x]) {
-                    bin[g + k] = kSmallBins - 1 - 4 * tid - x;
+                    bin[g + k] = kSmallBins - 1 - kPerBin * tid - x;
                     krem[g + k] = rank[k] - before;
                 }
             before += h[x];
@@ -687,7 +691,7 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
     // ---- kinds; rows inside a boundary bin are listed (the lists take the histograms' place)
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-        const int i = tid + q * kSmallThreads;
+        const int i = tid + q * THREADS;
         uint8_t k = CASK_KIND_DROPPED;
         int list = -1;
         if (i < P) {
@@ -711,7 +715,7 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
     __syncthreads();
     for (int x = 0; x < 3; ++x) {
         const int n = (int)n_cand[x];
-        for (int t = tid; t < n; t += kSmallThreads) {
+        for (int t = tid; t < n; t += THREADS) {
             const int i = sm.l.cand[x][t];
             const unsigned me = keys[i];
             unsigned ahead = 0;
@@ -730,7 +734,7 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
         }
     }
     __syncthreads();
-    // ---- outputs; the seeds in ascending row order (a warp's 128 rows are contiguous: one ballot a step, one scan over warps)
+    // ---- outputs; the seeds in ascending row order (a warp's rows are contiguous: one ballot a step, one sum over warps)
     const int i0 = w * (kSmallSpan / kWarps);
     unsigned ballots[kPer], mine = 0;
 #pragma unroll
@@ -741,11 +745,9 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
     }
     if (lane == 0) wsum[0][w] = mine;
     __syncthreads();
-    unsigned rank = 0, all = 0;
-    for (int x = 0; x < kWarps; ++x) {
-        if (x < w) rank += wsum[0][x];
-        all += wsum[0][x];
-    }
+    const unsigned of_warp = lane < kWarps ? wsum[0][lane] : 0u;
+    const unsigned all = __reduce_add_sync(0xffffffffu, of_warp);
+    unsigned rank = __reduce_add_sync(0xffffffffu, lane < w ? of_warp : 0u);
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
         const int i = i0 + 32 * q + lane;
@@ -765,9 +767,11 @@ __global__ void __launch_bounds__(kSmallThreads, 5) decide_small_kernel(
     }
     __syncthreads();
     const int ns = min((int)all, m);
-    for (int j = tid; j < ns; j += kSmallThreads) mass_fx[j] = mass_to_fx(row_mass(sh, s, eps, o + sm.l.seeds[j]));
-    static_assert(sizeof(keys) >= kWarps * 128 * sizeof(T), "the keys are no longer needed: their place serves the gather");
-    gather_seeds<4>(tab, sh, ud.seed_base, w, kWarps, ns, reinterpret_cast<T*>(keys) + 128 * w, [&](int j) {
+    for (int j = tid; j < ns; j += THREADS) mass_fx[j] = mass_to_fx(row_mass(sh, s, eps, o + sm.l.seeds[j]));
+    constexpr size_t kPass = kWarps * 128 * sizeof(T);       // for the gather: the keys are no longer needed, but may be too small a place
+    __shared__ alignas(16) uint8_t more[kPass > sizeof(keys) ? kPass : 16];
+    T* pass = reinterpret_cast<T*>(kPass > sizeof(keys) ? more : reinterpret_cast<uint8_t*>(keys)) + 128 * w;
+    gather_seeds<4>(tab, sh, ud.seed_base, w, kWarps, ns, pass, [&](int j) {
         const int i = sm.l.seeds[j];
         if (sh.page_size == 0) return ud.k_off + (int64_t)i * sh.row_stride;
         const int x = i / sh.page_size;
@@ -1106,9 +1110,11 @@ cudaError_t run(const Launch& L, const cask_params& prm, const float* s, const i
     } else if (fused) {
         Timed t(L, KID_SEEDS);
         size_t fixed = 0;
-        e = allow_smem(L, kSmemBitConsolidate + (sizeof(T) == 4), decide_small_kernel<T>, kMaxSpread, &fixed);
+        const int way = sh.n_units <= L.sms && L.max_T > 512 ? 2 : sh.n_units <= 3 * L.sms ? 1 : 0;      // see decide_small_kernel
+        const auto kern = way == 0 ? decide_small_kernel<T, 256, 4> : way == 1 ? decide_small_kernel<T, 512, 2> : decide_small_kernel<T, 1024, 1>;
+        e = allow_smem(L, kSmemBitConsolidate + 3 * (sizeof(T) == 4) + way, kern, kMaxSpread, &fixed);
         if (e == cudaSuccess)
-            e = launch_dependent(L.stream, decide_small_kernel<T>, sh.n_units, kSmallThreads, spread_smem(L, sh.n_units, fixed, 0), L.desc, sh,
+            e = launch_dependent(L.stream, kern, sh.n_units, 256 << way, spread_smem(L, sh.n_units, fixed, 0), L.desc, sh,
                                  tab, s, const_cast<int32_t*>(plan), kind, seed_of, sim, ws.grp, ws.seed_rows, ws.mass_fx, ws.njoin,
                                  unit_status, max_m, prm.eps);
     } else {

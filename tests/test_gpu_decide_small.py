@@ -56,3 +56,47 @@ def test_short_units_equal_the_staged_calls(prefix, decode, budget, reserve, dup
         else:
             assert np.array_equal(g[name], s[name]), name
     assert (g["n_out"] == np.minimum(budget, g["plan"][:, 7])).all()
+
+
+@pytest.mark.parametrize("prefix,decode,budget,reserve,dup,page,dtype,head_dim", [
+    (0, 65, 40, 40, 0, 0, BF16, 128),
+    (0, 1024, 700, 700, 0, 16, BF16, 128),       # 1,024 rows, several rounds of seeds
+    (500, 500, 300, 200, 1, 16, BF16, 128),      # a bin with every prefix row, one with every decode row
+    (212, 300, 400, 250, 0, 0, FP32, 64),        # 512 rows
+    (213, 300, 400, 250, 0, 1, BF16, 256),       # one more, a page per row
+])
+def test_threads_by_the_number_of_units(prefix, decode, budget, reserve, dup, page, dtype, head_dim):
+    """The selection of a short unit runs with 256 to 1,024 threads, by how many units there are: three units alone, and copies of them in
+    batches of more than one and more than three units a multiprocessor.  The normalisers are given and the 512 query rows fill a tile's four
+    slots (the fp32 units are a single step of tiles), so that a unit's scores do not depend on the batch."""
+    import gpu_harness as gh
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = wl.WORKLOADS["reasoning8k_b384"].with_(layers=1, kv_heads=3, group=16, window=32, prefix=prefix, decode=decode, budget=budget,
+                                                reserve=reserve, dtype=dtype, head_dim=head_dim)
+    one = wl.make_batch(w)
+    if dup:
+        one.k[:] = one.k[0]
+    T = prefix + decode
+    lse = np.random.default_rng(1).uniform(5.0, 9.0, (3, 512)).astype(np.float32)
+
+    def event(copies):
+        n = 3 * copies
+        full = lambda x: np.full(n, x, np.int32)
+        hb = wl.Batch(wl=w, k=np.tile(one.k, (copies, 1)), v=np.tile(one.v, (copies, 1)), q=np.tile(one.q, (copies, 1, 1, 1)), T=full(T), P=full(prefix),
+                      B=full(budget), reserve=full(reserve), tok_off=np.arange(n + 1, dtype=np.int64) * T, unit_ids=[(i, 0, 0) for i in range(n)])
+        run = gh.GpuRun(hb, page_size=page, lse_in=np.tile(lse, (copies, 1)))
+        g = run.event()
+        assert run.ctx.device_flags() == 0
+        return {name: x.reshape(copies, -1) for name, x in g.items()}
+
+    want = event(1)
+    for copies in (sms // 3 + 2, sms + 2):
+        for name, x in event(copies).items():
+            if name in ("k_out", "v_out"):
+                x, y = x.reshape(3 * copies, budget, -1), want[name].reshape(3, budget, -1)
+                for u in range(3 * copies):
+                    k = int(want["n_out"][0][u % 3])
+                    assert np.array_equal(x[u][:k], y[u % 3][:k]), name
+            else:
+                assert (x.view(np.uint8) == want[name].view(np.uint8)).all(), name
