@@ -292,7 +292,8 @@ int prepare(cask_ctx* ctx, const cask_batch* b, const cask_params* p, void* ws, 
     }
     if (own_stage) {
         bool reads_staging = false;
-        e = upload_descriptors(ctx->stream, stage, b->n_units, W.desc, W.err, &reads_staging);
+        e = upload_descriptors(ctx->stream, stage, b->n_units, W.desc, W.err,
+                               !b->lse_in || !given_score_long(b->dtype, b->head_dim, b->group * b->window, tile0, ctx->sms), &reads_staging);
         if (e == cudaSuccess && reads_staging) {
             e = cudaEventRecord(ctx->staged, ctx->stream);
             ctx->staged_pending = e == cudaSuccess;

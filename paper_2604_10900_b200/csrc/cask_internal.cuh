@@ -219,8 +219,9 @@ struct Workspace {
 };
 
 // ---- kernels (defined in the .cu files) --------------------------------------
-// Descriptors into the workspace, flag words cleared (upload.cu).  *reads_staging: the kernel still reads `staged` (page-locked).
-cudaError_t upload_descriptors(cudaStream_t stream, const UnitDesc* staged, int n, UnitDesc* dst, int32_t* err, bool* reads_staging);
+// Descriptors into the workspace, flag words cleared (upload.cu).  release: the kernel that follows may start beside this one.
+// *reads_staging: the kernel still reads `staged` (page-locked).
+cudaError_t upload_descriptors(cudaStream_t stream, const UnitDesc* staged, int n, UnitDesc* dst, int32_t* err, bool release, bool* reads_staging);
 cudaError_t launch_score_simt(const Launch& L, const float* lse_in, float* s, float* lse_out,
                               Workspace& ws);
 cudaError_t launch_row_combine(const Launch& L, const float* lse_in, float* lse_out, Workspace& ws);
@@ -284,6 +285,8 @@ cudaError_t launch_split_rows(const Launch& L, Workspace& ws, bool queries);
 
 // Tensor-core scoring (tcgen05 + TMA); returns cudaErrorNotSupported when the shape does not fit.
 bool score_tc_supported(const Launch& L);
+// Does the score pass of a batch with given normalisers have so many tiles a CTA that it should find the SMs empty (see launch_passes)?
+bool given_score_long(int dtype, int d, int rows, int total_tiles, int sms);
 struct ScoreTcSizes {
     size_t part_floats;      // floats per normaliser-partial table
     size_t s_parts;          // partial scores per cache row (0: the score pass writes the scores themselves)

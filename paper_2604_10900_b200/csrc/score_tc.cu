@@ -1233,6 +1233,11 @@ ScoreTcSizes score_tc_sizes(int dtype, int d, int rows, int n_units) {
                         pl.rg.groups > 1 ? (size_t)pl.rg.groups : 0};
 }
 
+constexpr int kGivenLong = 24;        // tiles a CTA
+bool given_score_long(int dtype, int d, int rows, int total_tiles, int sms) {
+    return shape_fits(dtype, d, rows) && (int64_t)total_tiles * row_plan(rows, dtype).rg.groups >= (int64_t)kGivenLong * (sms > 0 ? sms : 128);
+}
+
 // Rows per TMA box of the key stream: a whole 128-key tile for a contiguous cache, one page piece for
 // a paged one (0: the page size does not tile 128 rows).
 static int key_box_rows(const Shape& sh) {
@@ -1271,8 +1276,10 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     // Whether a pass may start while the kernel before it still runs (launch_dependent).  Its warps then take the slots that kernel's
     // leave, and where those are not the first ones of the SM the CTA runs up to 8 % slower, tile for tile, from the first to the
     // last: with the score pass of 288 units of 33,280 rows, a third of the CTAs (pass 1,260 to 1,360 us).
-    // With given normalisers the score pass gains nothing but the launch, and starts early only where it is short: 7 to 28 tiles a CTA
-    // 0.4 to 2 % better (units of 8,448 rows, 512 query rows), but 28 of eight units of 33,280 rows 160 to 168 and 160 us.
+    // With given normalisers the score pass gains nothing but the launch: 7 to 23 tiles a CTA 0.4 to 2 % better beside the descriptor
+    // kernel (units of 8,448 rows, 512 query rows).  Longer passes (given_score_long) are launched the same way, but that kernel does not
+    // release them, so that they start when it and the last CTAs of the call before are gone, without the 4 us of an ordinary launch:
+    // eight units of 33,280 rows 159.9 to 157.2 us (168 beside those CTAs), 288 of 2,000 201.8 to 198.2, 112 of 4,608 121.6 to 119.1.
     // Behind the normaliser pass it has its first keys, queries and contractions done and its code fetched by the end of that pass
     // (`ahead`): events of 8 units of 640 rows 54.0 to 49.9 us (0.3 tiles a CTA), two fp32 ones of 1,024 52.1 to 50.0, 128 of 4,608 at
     // head_dim 64 (31 tiles) 182 to 176; 24 to 60 tiles 0.5 to 2.5 % (100 units of 11,366 rows 485.7 to 479.4), 90 to 200 up to 1.5, 250 and
@@ -1296,7 +1303,7 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     }
     if (e == cudaSuccess) {
         Timed t(L, KID_SCORE_MASS);
-        const bool early = total < (lse_in ? 24 : 256) * grid;
+        const bool early = lse_in || total < 256 * grid;
         e = launch_kernel(early, L.stream, mass, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
                              ws.part_l, lse_in, lse_out, own_tables ? ws.rowm : nullptr, rg.groups > 1 ? ws.s_part : s, rg.groups > 1 ? L.sum_T : 0, L.fill,
                              early && !lse_in, ws.roww, ws.err);

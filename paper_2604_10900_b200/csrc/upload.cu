@@ -15,8 +15,10 @@ struct DescParams { UnitDesc d[kParamUnits]; };
 static_assert(sizeof(UnitDesc) % 16 == 0, "descriptors move 16 bytes at a time");
 
 __global__ void __launch_bounds__(kThreads) desc_from_params(const __grid_constant__ DescParams in, int n16, uint4* __restrict__ dst,
-                                                             uint4* __restrict__ err) {
-    pdl_wait();
+                                                             uint4* __restrict__ err, bool release) {
+    // (see pdl_wait; no early start of a long score pass with given normalisers, see launch_passes)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (release) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint4* src = reinterpret_cast<const uint4*>(&in);
     if (threadIdx.x == 0) *err = make_uint4(0u, 0u, 0u, 0u);
     for (int i = threadIdx.x; i < n16; i += kThreads) dst[i] = src[i];
@@ -39,13 +41,13 @@ __global__ void __launch_bounds__(kThreads) desc_from_host(const uint4* __restri
 
 }  // namespace
 
-cudaError_t upload_descriptors(cudaStream_t stream, const UnitDesc* staged, int n, UnitDesc* dst, int32_t* err, bool* reads_staging) {
+cudaError_t upload_descriptors(cudaStream_t stream, const UnitDesc* staged, int n, UnitDesc* dst, int32_t* err, bool release, bool* reads_staging) {
     const int n16 = (int)(n * sizeof(UnitDesc) / 16);
     *reads_staging = n > kParamUnits;
     if (n <= kParamUnits) {
         DescParams prm;
         for (int u = 0; u < n; ++u) prm.d[u] = staged[u];
-        return launch_dependent(stream, desc_from_params, 1, kThreads, 0, prm, n16, (uint4*)dst, (uint4*)err);
+        return launch_dependent(stream, desc_from_params, 1, kThreads, 0, prm, n16, (uint4*)dst, (uint4*)err, release);
     }
     return launch_dependent(stream, desc_from_host, (n16 + kThreads - 1) / kThreads, kThreads, 0, (const uint4*)staged, n16,
                             (uint4*)dst, (uint4*)err);
