@@ -208,13 +208,17 @@ Workspace carve(char* base, const cask_batch* b, const Sizes& z) {
     w.grp = (int32_t*)take(sumT * 4);
     w.mass_fx = (unsigned long long*)take(n * ((size_t)z.max_m + 1) * 8);
     w.njoin = (int32_t*)take(n * 4);
+    const size_t chunked = assign_many(b->dtype, b->chan_w != nullptr, z.max_m, z.sum_T) ? sumT : 0;
+    w.row_best = (float*)take(chunked * 8);
+    w.row_best_u = (int32_t*)take(chunked * 4);
+    w.close = (int32_t*)take(chunked * 4);
     w.mem_row = (int32_t*)take(sumT * 4);
     w.mem_slot = (int32_t*)take(sumT * 4);
     w.n_mem = (int32_t*)take(n * 4);
     w.seed_slot = (int32_t*)take(n * (size_t)std::max(z.max_B, 1) * 4);
     w.n_seed = (int32_t*)take(n * 4);
     w.max_B = std::max(z.max_B, 1);
-    w.err = (int32_t*)take(16);
+    w.err = (int32_t*)take(32);
     w.stats_a = (float*)take((n + 4) * (size_t)b->head_dim * 4);      // per-unit coefficients + one table of band constants
     w.bytes = off;
     return w;
@@ -301,7 +305,7 @@ int prepare(cask_ctx* ctx, const cask_batch* b, const cask_params* p, void* ws, 
     } else {
         // a slice of a host batch, on the copy stream: a kernel here would wait for room beside the other slices' kernels
         e = cudaMemcpyAsync(W.desc, stage, sizeof(UnitDesc) * (size_t)b->n_units, cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(W.err, 0, 16, ctx->stream);      // device-side flags of this call
+        if (e == cudaSuccess) e = cudaMemsetAsync(W.err, 0, 32, ctx->stream);      // device-side flags of this call
     }
     if (e != cudaSuccess) return fail_cuda(ctx, e);
     ctx->flags_dev = W.err;

@@ -1,6 +1,6 @@
 // Assignment of scratch rows to seeds on the tensor cores (Sec. 2.5: cosine as the base merge
 // geometry): D[row, seed] = <k_row, k_seed> for 128-row tiles of the decode region against the
-// unit's m <= 256 gathered seed keys, then per row the argmax of the cosine and the threshold tau.  Any head_dim up to 128:
+// unit's gathered seed keys, then per row the argmax of the cosine and the threshold tau.  Any head_dim up to 128:
 // TMA fills the channels past a shorter row with zeros (128 units of 4,608 rows at head_dim 64: 430 to 35 us against the
 // SIMT kernel that served them before).
 //
@@ -15,6 +15,14 @@
 // With m <= 128 seeds in every unit the TMEM holds four buffers of 128 columns, one per group.  With more
 // seeds it holds two buffers of 256 columns and two groups share each: one takes the first seed columns and
 // finishes the row, the other takes the rest and hands its best seed over through shared memory.
+//
+// More than 256 seeds (MANY): their columns are taken in chunks of at most 128, a launch each, with four buffers.  A row's greatest and second
+// greatest value and the former's seed go from launch to launch through the workspace; the launch with a unit's last chunk finishes its
+// rows.  Rows that the sums of the tensor cores cannot tell (see kClose) are listed, and assign_close_kernel decides them by the sums of
+// assign_simt_kernel, which served these shapes before: a row goes where that kernel sends it.  Chunks of 128 and four buffers, not of
+// 256 and two: a pass of the former takes half of one of the latter (0.44 and 0.87 ms for 9.6 M rows).  Event of 16 units of 15,276 rows
+// (380 seeds) 1,283 to 250 us, 104 of 27,043 (270) 11,242 to 1,377, 4 of 9,000 (860) 517 to 204, 8 of 1,024 (434) 155 to 88, one of
+// 3,000 (1,386) 251 to 145.
 //
 // fp32 caches (SPLIT): the contraction takes the bf16 parts of the rows and the seeds (split.cu) in six products as the scoring
 // passes do (score_tc.cu), one tile of six 16 KB regions at a time, m <= 128; the row norms come from the split.  What that sum
@@ -70,20 +78,34 @@ struct ASmemTail {
 constexpr size_t kSmemBytesA = 1024 + kSeedBytes + kStages * kKStageBytes + sizeof(ASmemTail);
 static_assert(2 * kRegions * kKRegionBytes <= kSeedBytes + kStages * kKStageBytes, "SPLIT: seeds and one tile, six regions each");
 
+// MANY: the seeds of a launch, and what goes from one to the next.
+struct Chunk {
+    int c0, width;                   // seeds [c0, c0 + width) of every unit
+    float2* best;                    // [sumT] greatest and second greatest dot product / seed norm of a row so far
+    int32_t* best_u;                 // [sumT] the former's seed
+    int32_t *close, *n_close;        // [sumT], [1] rows left to assign_close_kernel
+};
+
 // Walks this CTA's contiguous range of scratch tiles, unit by unit.
 struct TileWalk {
     const UnitDesc* desc;
     int g, g_end, u, n_units;
-    __device__ void init(const UnitDesc* d, int n_units_, int total) {
+    int c0;                          // units of no more seeds are passed over
+    __device__ void init(const UnitDesc* d, int n_units_, int total, int first_seed) {
         desc = d;
         n_units = n_units_;
+        c0 = first_seed;
         g = (int)(((long long)total * blockIdx.x) / gridDim.x);
         g_end = (int)(((long long)total * (blockIdx.x + 1)) / gridDim.x);
         u = warp_find_unit(n_units, g, [&](int v) { return d[v].atile0; });
         skip_empty();
     }
     __device__ void skip_empty() {
-        while (u < n_units - 1 && g >= desc[u].atile0 + desc[u].n_atiles) ++u;
+        for (;;) {
+            while (u < n_units - 1 && g >= desc[u].atile0 + desc[u].n_atiles) ++u;
+            if (c0 == 0 || g >= g_end || desc[u].plan[CASK_PLAN_M] > c0) return;
+            g = min(g_end, desc[u].atile0 + desc[u].n_atiles);
+        }
     }
     __device__ bool valid() const { return g < g_end; }
     __device__ int tile_in_unit() const { return g - desc[u].atile0; }
@@ -256,7 +278,7 @@ __device__ __noinline__ int plain_best(const float* __restrict__ K, const Shape&
 // 64 rows, where the tile's copies and its epilogue need some 1,900 between them.  512 units of 4,700 to 33,000 rows in pages of 64
 // 616 -> 525 us, 3,072 units of 640 rows in pages of 16 105 -> 76; as a call of its own 530 and 85.)
 __device__ __forceinline__ void produce_paged(const CUtensorMap* tmK, const CUtensorMap* tmSeed, const UnitDesc* __restrict__ desc,
-                                              const Shape& sh, int g, int g_end, int u, int sub_rows, int wpair, int n_kb, bool dual,
+                                              const Shape& sh, int g, int g_end, int u, int c0, int sub_rows, int wpair, int n_kb, bool dual,
                                               uint8_t* b_smem, uint8_t* k_smem, ASmemTail* tail) {
     ABarriers& bar = tail->bar;
     volatile int* abort_flag = &tail->abort;
@@ -266,12 +288,12 @@ __device__ __forceinline__ void produce_paged(const CUtensorMap* tmK, const CUte
     const int pieces = 1 << tile_shift, my_tile = lane >> tile_shift, my_piece = lane & (pieces - 1);
     const uint32_t seed_region = dual ? 128u * 128u : kSeedRegionBytes;
     // descriptors of the units first_u + lane
-    int first_u = u - 32, c_at0 = 0, c_nat = 0, c_bt0 = 0, c_P = 0, c_T = 0, c_seed = 0;
+    int first_u = u - 32, c_at0 = 0, c_nat = 0, c_bt0 = 0, c_P = 0, c_T = 0, c_seed = 0, c_m = 0;
     auto cache_units = [&]() {
         if (u - first_u < 32) return;
         first_u = u;
         const UnitDesc& d = desc[min(u + lane, sh.n_units - 1)];
-        c_at0 = d.atile0; c_nat = d.n_atiles; c_bt0 = d.bt0; c_P = d.P; c_T = d.T; c_seed = d.seed_base;
+        c_at0 = d.atile0; c_nat = d.n_atiles; c_bt0 = d.bt0; c_P = d.P; c_T = d.T; c_seed = d.seed_base + c0; c_m = d.plan[CASK_PLAN_M];
     };
     struct Batch { int n, row0, T, seed; bool fresh; int page, in_page; };
     int last_u = -1;
@@ -280,11 +302,16 @@ __device__ __forceinline__ void produce_paged(const CUtensorMap* tmK, const CUte
         if (g >= g_end) return b;
         cache_units();
         int at0 = __shfl_sync(0xffffffffu, c_at0, u - first_u), nat = __shfl_sync(0xffffffffu, c_nat, u - first_u);
-        while (u < sh.n_units - 1 && g >= at0 + nat) {
-            ++u;
-            cache_units();
-            at0 = __shfl_sync(0xffffffffu, c_at0, u - first_u);
-            nat = __shfl_sync(0xffffffffu, c_nat, u - first_u);
+        for (;;) {
+            while (u < sh.n_units - 1 && g >= at0 + nat) {
+                ++u;
+                cache_units();
+                at0 = __shfl_sync(0xffffffffu, c_at0, u - first_u);
+                nat = __shfl_sync(0xffffffffu, c_nat, u - first_u);
+            }
+            if (c0 == 0 || __shfl_sync(0xffffffffu, c_m, u - first_u) > c0) break;
+            g = min(g_end, at0 + nat);
+            if (g >= g_end) return b;
         }
         const int P = __shfl_sync(0xffffffffu, c_P, u - first_u), bt0 = __shfl_sync(0xffffffffu, c_bt0, u - first_u);
         b.T = __shfl_sync(0xffffffffu, c_T, u - first_u);
@@ -340,7 +367,7 @@ __device__ __forceinline__ void produce_paged(const CUtensorMap* tmK, const CUte
 }
 
 // FULL: head_dim 113..128 (the compiler then knows the numbers of channel halves and contraction steps)
-template <bool FULL, bool SPLIT>
+template <bool FULL, bool SPLIT, bool MANY>
 __global__ void __launch_bounds__(kThreadsA, 1)
 assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmSeed,
                  const UnitDesc* __restrict__ desc, Shape sh, int total_tiles, int n_bufs, int sub_rows, int wpair,
@@ -350,7 +377,8 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                  uint8_t* __restrict__ kind, int32_t* __restrict__ seed_of, float* __restrict__ sim,
                  int32_t* __restrict__ grp, unsigned long long* __restrict__ mass_fx,
                  int32_t* __restrict__ njoin, int32_t* __restrict__ mem_row, int32_t* __restrict__ mem_seed, int max_m, float tau,
-                 float eps, int32_t* __restrict__ err) {
+                 float eps, int32_t* __restrict__ err, const Chunk chunk) {
+    const int c0 = MANY ? chunk.c0 : 0;                  // first seed of the launch
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* b_smem = smem;
@@ -394,12 +422,12 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     pdl_wait();
 
     TileWalk wk;
-    wk.init(desc, sh.n_units, total_tiles);
+    wk.init(desc, sh.n_units, total_tiles, c0);
 
     if (warp == 0) {
         // ================= TMA producer =================
         if (!SPLIT && sh.page_size) {
-            produce_paged(&tmK, &tmSeed, desc, sh, wk.g, wk.g_end, wk.u, sub_rows, wpair, n_kb, dual, b_smem, k_smem, tail);
+            produce_paged(&tmK, &tmSeed, desc, sh, wk.g, wk.g_end, wk.u, c0, sub_rows, wpair, n_kb, dual, b_smem, k_smem, tail);
         } else if (lane == 0) {
             uint32_t kit = 0, ucount = 0;
             bool ok = true;
@@ -437,8 +465,8 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (!ok) break;
                 mbar_expect_tx(&bar.b_full[sb], n_kb * seed_region);
                 uint8_t* bdst = b_smem + sb * 2 * seed_region;
-                tma_load_2d(bdst, &tmSeed, &bar.b_full[sb], 0, ud.seed_base << wpair);
-                if (n_kb == 2) tma_load_2d(bdst + seed_region, &tmSeed, &bar.b_full[sb], 64, ud.seed_base << wpair);
+                tma_load_2d(bdst, &tmSeed, &bar.b_full[sb], 0, (ud.seed_base + c0) << wpair);
+                if (n_kb == 2) tma_load_2d(bdst + seed_region, &tmSeed, &bar.b_full[sb], 64, (ud.seed_base + c0) << wpair);
                 ++ucount;
                 const int krow0 = (int)(ud.k_off / sh.row_stride) + ud.P + wk.tile_in_unit() * kTileRows;
                 const int nt = wk.run();
@@ -470,7 +498,8 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             const uint32_t b_lo = umma_desc_lo(smem_u32(b_smem)), k_lo = umma_desc_lo(smem_u32(k_smem));
             while (wk.valid() && ok) {
                 const UnitDesc& ud = desc[wk.u];
-                const int m = max(0, min(plan[wk.u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
+                const int m_all = max(0, min(plan[wk.u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
+                const int m = MANY ? min(m_all - c0, chunk.width) : m_all;
                 const uint32_t idesc = umma_idesc(max(16, ((m << wpair) + 15) & ~15));
                 if constexpr (SPLIT) {
                     ok = mbar_wait(&bar.b_full[0], ucount & 1u, abort_flag);
@@ -562,9 +591,12 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             const int u = wk.u;
             const int T = ud.T, P = ud.P;
             const int64_t tok_off = ud.tok_off;
-            const int seed_base = ud.seed_base;
+            const int seed_base = ud.seed_base + c0;
             const int r = max(0, min(plan[u * 8 + CASK_PLAN_R], T - P));
-            const int m = max(0, min(plan[u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
+            const int m_all = max(0, min(plan[u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
+            const int m = MANY ? max(0, min(m_all - c0, chunk.width)) : m_all;
+            // MANY: is this the launch that finishes the unit's rows?
+            const bool last = !MANY || (m_all <= c0 + chunk.width && (m > 0 || c0 == 0));
             const int hi = T - r;
             const int a0 = P - (!SPLIT && sh.page_size ? P % sub_rows : 0);
             // shared buffers: the finishing group also computes the row norm, so it takes fewer seed columns
@@ -635,7 +667,7 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (pre) {
                     kd = kd_n; s_c = s_n; mi_c = mi_n;
                     if (SPLIT) nj_c = nj_n;
-                } else if (in_range) {
+                } else if (in_range && last) {
                     kd = kind[tok_off + i];
                     s_c = s[tok_off + i];
                     if (sh.mass_in) mi_c = sh.mass_in[tok_off + i];
@@ -643,7 +675,13 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 }
                 // the same fields of this group's next tile of the unit, in flight during this tile (a row's kind
                 // is read and written by the thread that owns the row only, so reading it early sees the same byte)
-                pre = t + n_bufs < nt;
+                pre = last && t + n_bufs < nt;
+                float2 carried = make_float2(-INFINITY, -INFINITY);
+                int carried_u = -1;
+                if (MANY && c0 > 0 && in_range) {
+                    carried = chunk.best[tok_off + i];
+                    carried_u = chunk.best_u[tok_off + i];
+                }
                 kd_n = (uint8_t)CASK_KIND_RECENT; s_n = 0.f; mi_n = 0.f;
                 if (pre) {
                     const int in_ = i + n_bufs * kTileRows;
@@ -660,6 +698,8 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (!SPLIT) {
                     ok = mbar_wait(&bar.k_full[st], (kit / kStages) & 1u, abort_flag);
                     if (!ok) break;
+                }
+                if (!SPLIT && last) {
                     const uint8_t* base = k_smem + st * kKStageBytes + my_row * 128;
                     if (!sh.chan_w) n2p = row_norm2<false, FULL>(base, lane, my_row, tail->w, n_kb);
                     else n2p = row_norm2<true, FULL>(base, lane, my_row, tail->w, n_kb);
@@ -675,8 +715,35 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 float best = -INFINITY, second = -INFINITY;
                 int best_u = -1;
                 if (!SPLIT && wpair) best_seed<1>(taddr, inv, 0, c_split, best, best_u, second);
-                else best_seed<0, SPLIT>(taddr, inv, 0, c_split, best, best_u, second);
-                const bool cand = in_range && best_u >= 0 && kd == CASK_KIND_DROPPED;
+                else best_seed<0, SPLIT || MANY>(taddr, inv, 0, c_split, best, best_u, second);
+                if (MANY) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar.d_empty[eg]);
+                    if (best_u >= 0) best_u += c0;
+                    second = fmaxf(fmaxf(second, carried.y), fminf(best, carried.x));
+                    if (!(best > carried.x)) { best = carried.x; best_u = carried_u; }       // (the first seed among equals)
+                    if (!last) {
+                        if (in_range && m > 0) {
+                            chunk.best[tok_off + i] = make_float2(best, second);
+                            chunk.best_u[tok_off + i] = best_u;
+                        }
+                        continue;
+                    }
+                }
+                bool cand = in_range && best_u >= 0 && kd == CASK_KIND_DROPPED;
+                if (MANY) {
+                    const float nj = sqrtf(n2), by = kClose * nj;
+                    const bool unsure = in_range && m_all > 0 && kd == CASK_KIND_DROPPED && !(best_u >= 0 && second < best - by && fabsf(best - tau * nj) > by);
+                    const unsigned ub = __ballot_sync(0xffffffffu, unsure);
+                    if (ub) {
+                        int at = 0;
+                        if (lane == 0) at = atomicAdd(chunk.n_close, __popc(ub));
+                        at = __shfl_sync(0xffffffffu, at, 0) + __popc(ub & ((1u << lane) - 1u));
+                        if (unsure) chunk.close[at] = (int)(tok_off + i);
+                    }
+                    cand = cand && !unsure;
+                }
                 uint32_t close[4] = {0u, 0u, 0u, 0u};            // SPLIT: the plain cosines decide between these seeds
                 const float least = best - kClose * nj_c;
                 const bool plain = SPLIT && cand && nj_c > 0.f && (second >= least || fabsf(best - tau * nj_c) <= kClose * nj_c);
@@ -698,8 +765,8 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         if (m < 32 * b + 32) close[b] &= (1u << (m - 32 * b)) - 1u;
                     }
                 }
-                tc_fence_before();
-                if (split == 2) {
+                if (!MANY) tc_fence_before();
+                if (!MANY && split == 2) {
                     // The other group's candidate has the larger seed indices, so it wins only when strictly
                     // better: the same outcome as one scan over all columns.  The buffer is released after this
                     // read, so the other group cannot start the buffer's next use (and overwrite its hand-over
@@ -712,8 +779,10 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         best_u = tail->x_idx[eg][use & 1u][my_row];
                     }
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bar.d_empty[eg]);
+                if (!MANY) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar.d_empty[eg]);
+                }
 
                 float sm_ = 0.f;
                 if (cand) {
@@ -727,9 +796,9 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (in_range) { const float a = s_c + eps; sc = sh.mass_in ? a + mi_c : a; }
                 const unsigned long long fx = cand ? mass_to_fx(sc) : 0ull;
                 if (joined) {
-                    const int bu = CASK_IDX(best_u, m, err);
+                    const int bu = CASK_IDX(best_u, m_all, err);
                     kind[tok_off + i] = CASK_KIND_MERGED;
-                    seed_of[tok_off + i] = srow[bu];
+                    seed_of[tok_off + i] = MANY ? seed_rows[ud.seed_base + bu] : srow[bu];
                     grp[tok_off + i] = bu;
                     atomicAdd(&mass_u[bu], fx);
                 }
@@ -766,6 +835,83 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     }
 }
 
+// MANY: the rows whose cosines with two seeds, or with one and tau, lie within what the sums of the tensor cores may be off.  A CTA a row, a
+// thread every 256th seed; the additions are those of assign_simt_kernel.  Bound by latency (list, unit, row, seeds in series), so
+// a seed's row is read 128 bytes at a time.  16 units of 15,276 rows, 380 seeds: 44 us with a warp a row, 15 so.
+constexpr int kCloseThreads = 256;
+__global__ void __launch_bounds__(kCloseThreads) assign_close_kernel(
+    const UnitDesc* __restrict__ desc, Shape sh, const __nv_bfloat16* __restrict__ K, const float* __restrict__ s, const int32_t* __restrict__ plan,
+    const int32_t* __restrict__ seed_rows, const __nv_bfloat16* __restrict__ seed_k, const float* __restrict__ seed_norm, uint8_t* __restrict__ kind,
+    int32_t* __restrict__ seed_of, float* __restrict__ sim, int32_t* __restrict__ grp, unsigned long long* __restrict__ mass_fx,
+    int32_t* __restrict__ njoin, int32_t* __restrict__ mem_row, int32_t* __restrict__ mem_seed, int max_m, float tau, float eps,
+    const int32_t* __restrict__ close, const int32_t* __restrict__ n_close) {
+    __shared__ alignas(16) float row[128];
+    __shared__ float best_w[kCloseThreads / 32];
+    __shared__ int best_uw[kCloseThreads / 32];
+    pdl_wait();
+    const int tid = threadIdx.x, lane = tid & 31, n = *n_close, d = sh.d;
+    for (int x = blockIdx.x; x < n; x += gridDim.x) {
+        const int at = close[x];
+        const int u = warp_find_unit(sh.n_units, at, [&](int v) { return (int)desc[v].tok_off; });
+        const UnitDesc& ud = desc[u];
+        const int i = at - (int)ud.tok_off, m = max(0, min(plan[u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
+        __syncthreads();
+        if (tid < d) row[tid] = __bfloat162float(K[row_elem_off(sh, ud, ud.k_off, i) + tid]);
+        __syncthreads();
+        float best = -INFINITY;
+        int best_u = -1;
+        for (int j = tid; j < m; j += kCloseThreads) {
+            const uint4* seed = reinterpret_cast<const uint4*>(seed_k + (size_t)(ud.seed_base + j) * d);
+            const float nu = seed_norm[ud.seed_base + j];
+            float acc = 0.f, n2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+            for (int c = 0; c < d / 8; ++c) {
+                const uint4 v = seed[c];
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    const float r0 = row[8 * c + 2 * y], r1 = row[8 * c + 2 * y + 1];
+                    n2[(2 * y) & 3] = fmaf(r0, r0, n2[(2 * y) & 3]);
+                    n2[(2 * y + 1) & 3] = fmaf(r1, r1, n2[(2 * y + 1) & 3]);
+                    acc = fmaf(r0, __uint_as_float(w[y] << 16), acc);
+                    acc = fmaf(r1, __uint_as_float(w[y] & 0xFFFF0000u), acc);
+                }
+            }
+            const float nj = sqrtf((n2[0] + n2[1]) + (n2[2] + n2[3]));
+            const float v = nj > 0.f && nu > 0.f ? acc / (nj * nu) : 0.f;
+            if (v > best) { best = v; best_u = j; }
+        }
+        auto fold = [&](int width) {           // the greatest, the first seed among equals
+            for (int off = width / 2; off >= 1; off >>= 1) {
+                const float ob = __shfl_xor_sync(0xffffffffu, best, off);
+                const int ou = __shfl_xor_sync(0xffffffffu, best_u, off);
+                if (ou >= 0 && (ob > best || (ob == best && ou < best_u) || best_u < 0)) { best = ob; best_u = ou; }
+            }
+        };
+        fold(32);
+        if (lane == 0) { best_w[tid >> 5] = best; best_uw[tid >> 5] = best_u; }
+        __syncthreads();
+        if (tid >= 32) continue;
+        best = best_w[lane & (kCloseThreads / 32 - 1)];
+        best_u = best_uw[lane & (kCloseThreads / 32 - 1)];
+        fold(kCloseThreads / 32);
+        if (lane != 0) continue;
+        if (sim) sim[at] = best;
+        const unsigned long long fx = mass_to_fx(row_mass(sh, s, eps, at));
+        const bool joined = best_u >= 0 && best >= tau;
+        atomicAdd(&mass_fx[(size_t)u * (max_m + 1) + (joined ? best_u : max_m)], fx);
+        if (!joined) continue;
+        kind[at] = CASK_KIND_MERGED;
+        seed_of[at] = seed_rows[ud.seed_base + CASK_IDX(best_u, m, sh.err)];
+        grp[at] = best_u;
+        const int p = atomicAdd(&njoin[u], 1);
+        if (mem_row && p < ud.T) {
+            mem_row[ud.tok_off + p] = i;
+            mem_seed[ud.tok_off + p] = best_u;
+        }
+    }
+}
+
 }  // namespace
 
 // Rows per TMA box of the key stream (see the scoring kernel): 128, one page piece, or 0 if unsupported.
@@ -776,10 +922,14 @@ int assign_tc_box_rows(const Shape& sh) {
     return 0;
 }
 
+bool assign_many(int dtype, bool weighted, int max_m, int64_t sum_T) {
+    return dtype == CASK_DTYPE_BF16 && !weighted && max_m > 256 && sum_T < (int64_t)1 << 31;
+}
+
 bool assign_tc_supported(const Launch& L) {
     const Shape& sh = L.sh;
     const int cols = L.max_m << (sh.chan_w ? 1 : 0);      // a weighted seed takes two accumulator columns
-    if (sh.d > 128 || cols > 256 || L.max_m < 1 || L.total_atiles < 1) return false;
+    if (sh.d > 128 || (cols > 256 && !assign_many(sh.dtype, sh.chan_w != nullptr, L.max_m, L.sum_T)) || L.max_m < 1 || L.total_atiles < 1) return false;
     if (sh.dtype == CASK_DTYPE_FP32) return !sh.chan_w && L.max_m <= 128 && 3 * L.sum_T < (int64_t)1 << 31;
     if (sh.page_size) return assign_tc_box_rows(sh) != 0 && sh.n_pages * sh.page_size < ((int64_t)1 << 31);
     int64_t max_row = 0;
@@ -811,17 +961,37 @@ cudaError_t launch_assign_tc(const Launch& L, const cask_params& prm, const floa
         return cudaErrorInvalidValue;
     // the seed table has 256 spare rows behind the last seed, so a full box never leaves the allocation
     const int wpair = sh.chan_w ? 1 : 0;
-    const int n_bufs = (L.max_m << wpair) <= 128 ? 4 : 2;      // accumulator buffers; four: seed boxes of 128 rows
+    const bool many = (L.max_m << wpair) > 256;
+    const int n_bufs = many || (L.max_m << wpair) <= 128 ? 4 : 2;      // accumulator buffers; four: seed boxes of 128 rows
     if (!encode_rows_bf16(tmap_encode_fn, &tmSeed, ws.seed_k, split ? 3 * ((uint64_t)sum_m + 256) : ((uint64_t)sum_m << wpair) + 256, sh.d, (uint64_t)sh.d * 2, n_bufs == 4 ? 128 : 256))
         return cudaErrorInvalidValue;
     const int grid = std::max(1, std::min(L.sms > 0 ? L.sms : 128, L.total_atiles));
-    auto kern = split ? (sh.d > 112 ? assign_tc_kernel<true, true> : assign_tc_kernel<false, true>) : sh.d > 112 ? assign_tc_kernel<true, false> : assign_tc_kernel<false, false>;
-    cudaError_t e = allow_smem(L, kSmemBitAssign + (sh.d > 112) + 2 * split, kern, kSmemBytesA);
+    const bool full = sh.d > 112;
+    auto kern = many ? (full ? assign_tc_kernel<true, false, true> : assign_tc_kernel<false, false, true>)
+                : split ? (full ? assign_tc_kernel<true, true, false> : assign_tc_kernel<false, true, false>)
+                        : (full ? assign_tc_kernel<true, false, false> : assign_tc_kernel<false, false, false>);
+    cudaError_t e = allow_smem(L, many ? kSmemBitAssignMany + full : kSmemBitAssign + full + 2 * split, kern, kSmemBytesA);
+    if (e != cudaSuccess) return e;
+    // chunks of equal width, a multiple of the contraction's 16 columns
+    const int n_chunks = many ? (L.max_m + 127) / 128 : 1;
+    Chunk chunk{0, many ? ((L.max_m + n_chunks - 1) / n_chunks + 15) / 16 * 16 : 0, (float2*)ws.row_best, ws.row_best_u, ws.close, ws.err + 4};
+    for (int k = 0; k < n_chunks; ++k, chunk.c0 += chunk.width) {
+        Timed t(L, KID_ASSIGN);
+        e = launch_dependent(L.stream, kern, grid, kThreadsA, kSmemBytesA, tmK, tmSeed, L.desc, sh, L.total_atiles, n_bufs, sub_rows,
+                             wpair, (int)sum_m + 256, split ? (const float*)L.k : nullptr, ws.k_norm, s, plan, ws.seed_rows, ws.seed_norm, kind, seed_of, sim, ws.grp,
+                             ws.mass_fx, ws.njoin, ws.slot_lists ? ws.mem_row : nullptr, ws.mem_slot, L.max_m, prm.tau, prm.eps, ws.err, chunk);
+        if (e != cudaSuccess) return e;
+    }
+    if (!many) return e;
+    // four CTAs an SM, which the shared memory that they ask for spreads over all of them (see spread_smem)
+    const int close_grid = 4 * (L.sms > 0 ? L.sms : 128);
+    size_t fixed = 0;
+    e = allow_smem(L, kSmemBitAssignMany + 2, assign_close_kernel, kMaxSpread, &fixed);
     if (e != cudaSuccess) return e;
     Timed t(L, KID_ASSIGN);
-    return launch_dependent(L.stream, kern, grid, kThreadsA, kSmemBytesA, tmK, tmSeed, L.desc, sh, L.total_atiles, n_bufs, sub_rows,
-                            wpair, (int)sum_m + 256, split ? (const float*)L.k : nullptr, ws.k_norm, s, plan, ws.seed_rows, ws.seed_norm, kind, seed_of, sim, ws.grp,
-                            ws.mass_fx, ws.njoin, ws.slot_lists ? ws.mem_row : nullptr, ws.mem_slot, L.max_m, prm.tau, prm.eps, ws.err);
+    return launch_dependent(L.stream, assign_close_kernel, close_grid, kCloseThreads, spread_smem(L, close_grid, fixed, 0), L.desc, sh, (const __nv_bfloat16*)L.k, s, plan,
+                            ws.seed_rows, (const __nv_bfloat16*)ws.seed_k, ws.seed_norm, kind, seed_of, sim, ws.grp, ws.mass_fx, ws.njoin,
+                            ws.slot_lists ? ws.mem_row : nullptr, ws.mem_slot, L.max_m, prm.tau, prm.eps, ws.close, ws.err + 4);
 }
 
 }  // namespace cask

@@ -122,7 +122,7 @@ inline cudaError_t allow_smem(const Launch& L, int bit, K kern, size_t bytes, si
     }
     return cudaSuccess;
 }
-constexpr int kSmemBitScore = 0, kSmemBitAssign = 28, kSmemBitConsolidate = 32, kSmemBitCopy = 40;   // first bit of each file's kernels
+constexpr int kSmemBitScore = 0, kSmemBitAssign = 28, kSmemBitConsolidate = 32, kSmemBitCopy = 40, kSmemBitAssignMany = 60;   // first bit of each file's kernels
 
 // Dynamic shared memory with which no more CTAs of a kernel share an SM than the grid needs (`need` bytes if that is more).
 // CTAs that start while the kernel before them leaves go to the SMs that are free first, as many as fit: 288 CTAs of which
@@ -205,6 +205,9 @@ struct Workspace {
     int32_t* grp;        // [sumT] seed slot (0..m) of a joined row, -1
     unsigned long long* mass_fx;  // [units*(max_m+1)] fixed-point group masses (+ lost mass)
     int32_t* njoin;      // [units]
+    float* row_best;     // assignment to more than 256 seeds (assign_many): [sumT, 2] greatest and second greatest value of a row so far,
+    int32_t* row_best_u; //   [sumT] the former's seed,
+    int32_t* close;      //   [sumT] rows that the plain cosines decide
     int32_t* mem_row;    // [sumT] rows of kind 4/5 in ascending order; slot lists: the rows that joined (njoin), in any order
     int32_t* mem_slot;   // [sumT] slot each of them feeds; slot lists: the number of their seed
     int32_t* n_mem;      // [units]; slot lists: kept rows, -1: this unit has no lists
@@ -213,7 +216,7 @@ struct Workspace {
     bool filled;         // the scoring call has written Launch::fill
     bool slot_lists;     // the selection of this call has listed the slots, and the assignment kernel lists the rows that join
     int32_t max_B;
-    int32_t* err;        // [1]
+    int32_t* err;        // [8] flags (0, 1), clocks of the scoring passes (2, 3), entries of `close` (4)
     float* stats_a;      // [units, d] query-statistics scorer: head-pooled mu * kappa per band (re, im)
     size_t bytes;
 };
@@ -268,6 +271,7 @@ cudaError_t launch_diagnostics(const Launch& L, const cask_params& prm, const fl
                                const cask_outputs& out);
 
 // Tensor-core assignment of scratch rows to seeds (cosine Gram + argmax), same outputs as the SIMT kernel.
+bool assign_many(int dtype, bool weighted, int max_m, int64_t sum_T);      // seeds in chunks (they need row_best and the like)
 bool assign_tc_supported(const Launch& L);      // fp32 caches: through their bf16 parts
 int assign_tc_box_rows(const Shape& sh);   // rows per TMA box of the key stream, 0 if the page size does not fit
 cudaError_t launch_assign_tc(const Launch& L, const cask_params& prm, const float* s, const int32_t* plan,

@@ -1,0 +1,95 @@
+"""More than 256 seeds a unit: the tensor-core assignment takes them in chunks, a launch each, and leaves the rows its sums cannot tell to a
+kernel with the SIMT kernel's sums.  The SIMT kernel, which served these shapes before, is the reference: the same scores and selections
+go in, and every row has to go where that kernel sends it."""
+import numpy as np
+import pytest
+
+from paper_2604_10900_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _compare(hb, page=0, change=None, **kw):
+    import gpu_harness as gh
+    import torch
+    tc, simt = (gh.GpuRun(hb, page_size=page, **kw) for _ in range(2))
+    if change:
+        for run in (tc, simt):
+            change(run)
+    slow = simt.cb.params(score_path=1, **kw)
+    outs = []
+    for run, prm in ((tc, tc.prm), (simt, slow)):
+        o, args = run.out, (run.ctx, run.batch)
+        ws = (run.ws, run.ws_bytes)
+        run.cb.cask_score(*args, run.prm, o["s"], o["lse"], *ws)
+        run.cb.cask_prefix_evict(*args, run.prm, o["s"], o["kind"], o["plan"], *ws)
+        run.cb.cask_select_core(*args, run.prm, o["s"], o["plan"], o["kind"], *ws)
+        run.cb.cask_consolidate_scratch(*args, prm, o["s"], o["plan"], o["kind"], o["seed_of"], o["weight"], o["sim"], o["unit_status"], o["lost_mass"], *ws)
+        torch.cuda.synchronize()
+        assert run.ctx.device_flags() == 0
+        outs.append({n: o[n].cpu().numpy() for n in ("s", "kind", "seed_of", "weight", "unit_status", "lost_mass", "sim", "plan")})
+    a, b = outs
+    for name in a:
+        if name == "sim":      # both are sums of 128 products of at most the norms' product: off by up to 128 roundings of 2^-24 each
+            assert np.abs(a["sim"] - b["sim"]).max() <= 2 * 128 * 2.0 ** -24
+        else:
+            assert np.array_equal(a[name].view(np.uint8), b[name].view(np.uint8)), name
+    if page == 0 and not change:
+        ev = gh.GpuRun(hb, **kw)
+        e = ev.event()
+        for name in ("kind", "seed_of", "lost_mass"):
+            assert np.array_equal(e[name].view(np.uint8), a[name].view(np.uint8)), name
+    return a
+
+
+def _batch(units=3, prefix=100, decode=1500, budget=800, reserve=700, head_dim=128, window=32):
+    return wl.make_batch(wl.WORKLOADS["reasoning8k_b384"].with_(layers=1, kv_heads=units, group=4, window=window, prefix=prefix, decode=decode,
+                                                                budget=budget, reserve=reserve, head_dim=head_dim))
+
+
+@pytest.mark.parametrize("m,kw,page", [
+    (257, dict(), 0),                                      # three chunks of 96, the last of 65
+    (288, dict(units=5), 16),                              # three whole chunks
+    (385, dict(decode=1283), 0),                           # four chunks, the last of 73; a ragged last tile
+    (700, dict(head_dim=64, decode=2001), 0),
+    (300, dict(head_dim=72, units=160, decode=700), 64),   # more units than multiprocessors
+    (1100, dict(units=2, decode=2600), 0),                 # more seeds than a selection's list holds
+    (284, dict(units=2, decode=17000, budget=652, reserve=600, window=32), 0),      # long units: listed slots and rows that join
+])
+def test_rows_go_where_the_simt_kernel_sends_them(m, kw, page):
+    kw = dict(kw)
+    if "budget" not in kw:     # room for r recent rows, m - 1 or m core rows and m seeds beside a prefix of 100 rows
+        kw.update(budget=100 + 32 + 2 * m, reserve=32 + 2 * m)
+    a = _compare(_batch(**kw), page)
+    assert (a["plan"][:, 5] == m).all(), a["plan"][:, 5]
+    assert (a["kind"] == 5).any() and (a["kind"] == 0).any()
+
+
+@pytest.mark.parametrize("tau", [-1.0, 0.3])
+def test_thresholds(tau):
+    _compare(_batch(), tau=tau)
+
+
+def test_units_of_few_and_many_seeds():
+    """Budgets from a handful of seeds to several chunks: a unit is finished by the launch with its last chunk and passed over by the rest."""
+    hb = _batch(units=12)
+    hb.B[:] = [800, 60, 400, 1100, 100, 800, 140, 700, 220, 1500, 70, 360]
+    hb.reserve[:] = np.maximum(hb.B - 100, 40)
+    a = _compare(hb)
+    assert a["plan"][:, 5].min() < 16 and a["plan"][:, 5].max() > 600
+
+
+def test_equal_and_empty_rows():
+    """Seeds equal to one another, rows equal to seeds, rows and seeds of zeros, rows with a number that is none: nothing is certain, and
+    the first seed among equals wins."""
+    hb = _batch(units=2, decode=900)
+    rng = np.random.default_rng(3)
+    T = int(hb.T[0])
+    k = hb.k.reshape(2, T, -1)
+    k[0, 100:] = k[0, 100 + rng.integers(0, 5, T - 100)]          # five distinct keys
+    k[1, rng.permutation(np.arange(100, T))[:300]] = 0
+
+    def nan_row(run):
+        run.dev["k"].view(2, T, -1)[1, 700] = float("nan")
+    _compare(hb)
+    _compare(hb, change=nan_row)
