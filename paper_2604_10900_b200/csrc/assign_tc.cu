@@ -6,8 +6,12 @@
 //
 // The contraction is small (2*128*m*128 flop per tile) next to the 32 KB of K it consumes, so the
 // kernel is bound by the K stream: a 4-stage TMA ring feeds one persistent CTA per SM.
+// What kept it from the stream's rate, 288 units of 33,280 rows with 64 and 96 seeds (508 and 586 us, 4.8 and 4.2 TB/s): one issuer took 1,730 clk a
+// tile, 850 of them blocked on the tensor pipe and the rest in two barrier probes one after the other, where two overlap them (452, 588); each group
+// walked through the other groups' tiles and added up the lost mass with ten shuffles a tile instead of a unit (410, 541); the seed of the
+// greatest cosine was looked for in every chunk (409, 477); waiting warps read the abort flag after every probe (382, 454: 6.4 and 5.4 TB/s).
 //   warp 0      TMA producer: seed matrix once per unit, K tiles through the ring
-//   warp 1      TMEM allocation, tcgen05.mma issue
+//   warps 1-2   tcgen05.mma issue, even and odd tiles (warp 1 also owns the TMEM allocation)
 //   warps 4-19  epilogue in groups of four warps (one per TMEM lane quadrant); group e takes the
 //               tiles e, e+G, e+2G, ... of the CTA and owns one accumulator buffer, so up to G
 //               tiles are in flight and the global-memory round trips of a tile (row kind, score,
@@ -60,7 +64,7 @@ struct __align__(8) ABarriers {
     uint64_t d_full[kMaxGroups], d_empty[kMaxGroups];
     uint64_t inv_ready[kMaxGroups];   // a group's table of inverse seed norms is written
     uint64_t x_full[2];      // shared buffers: the second group's best seed of a tile is in shared memory
-    uint64_t mma_drain;      // give-up path only: the contractions in flight have completed
+    uint64_t mma_drain[2];   // give-up path only: an issuer's contractions in flight have completed
 };
 
 struct ASmemTail {
@@ -158,51 +162,133 @@ __device__ __forceinline__ uint64_t row_norm2(const uint8_t* base, int lane, int
 
 // Best seed among the accumulator columns [c_lo, c_hi) of this thread's row: the greatest dot * 1/|k_seed|, the
 // first seed among equals.  PAIR = 1: a seed owns two adjacent columns (the hi and lo parts of its weighted key)
-// whose sum is its dot product.  A block of 32 columns costs a multiply and a maximum per seed; the position of
-// the maximum is looked for only in a block that beats everything before it.  SECOND: the second greatest value as well.
+// whose sum is its dot product.  Sixteen columns at a time, the next sixteen on their way meanwhile.  A chunk costs a multiply (packed in
+// pairs) and a maximum per seed; the position of the maximum is looked for only in a chunk that beats everything before it: first its half
+// of the chunk, then its place there, so that the chain of selections is half as long.  SECOND: the second greatest value as well.
+template <int PAIR>
+__device__ __forceinline__ void chunk_products(const float (&v)[16], uint32_t inv32, int cc, int c_hi, float (&p)[2][PAIR ? 4 : 8]) {
+    constexpr int kHalf = PAIR ? 4 : 8;          // seeds per half chunk
+    const int u0 = PAIR ? cc >> 1 : cc, u_hi = PAIR ? c_hi >> 1 : c_hi;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int x = 0; x < kHalf; x += 4) {
+            const int at = h * kHalf + x;        // (inverse norms 16 bytes at a time, shared-space)
+            const uint4 q = lds128(inv32 + (uint32_t)(u0 + at) * 4u);
+            const uint64_t n01 = pack2(__uint_as_float(q.x), __uint_as_float(q.y)), n23 = pack2(__uint_as_float(q.z), __uint_as_float(q.w));
+            if (PAIR) {
+                unpack2(mul2(pack2(v[2 * at] + v[2 * at + 1], v[2 * at + 2] + v[2 * at + 3]), n01), p[h][x], p[h][x + 1]);
+                unpack2(mul2(pack2(v[2 * at + 4] + v[2 * at + 5], v[2 * at + 6] + v[2 * at + 7]), n23), p[h][x + 2], p[h][x + 3]);
+            } else {
+                unpack2(mul2(pack2(v[at], v[at + 1]), n01), p[h][x], p[h][x + 1]);
+                unpack2(mul2(pack2(v[at + 2], v[at + 3]), n23), p[h][x + 2], p[h][x + 3]);
+            }
+        }
+    if (cc + 16 > c_hi) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int x = 0; x < kHalf; ++x)
+                if (u0 + h * kHalf + x >= u_hi) p[h][x] = -INFINITY;
+    }
+}
+
+template <int PAIR, bool SECOND>
+__device__ __forceinline__ void best_of_chunk(const float (&v)[16], uint32_t inv32, int cc, int c_hi, float& best, int& best_u, float& second) {
+    constexpr int kHalf = PAIR ? 4 : 8;
+    const int u0 = PAIR ? cc >> 1 : cc;
+    float p[2][kHalf];
+    chunk_products<PAIR>(v, inv32, cc, c_hi, p);
+    float m0 = -INFINITY, m1 = -INFINITY, b2 = -INFINITY;
+#pragma unroll
+    for (int x = 0; x < kHalf; ++x) {
+        if (SECOND) b2 = fmaxf(b2, fmaxf(fminf(m0, p[0][x]), fminf(m1, p[1][x])));
+        m0 = fmaxf(m0, p[0][x]);
+        m1 = fmaxf(m1, p[1][x]);
+    }
+    const float bm = fmaxf(m0, m1);
+    if (SECOND) second = fmaxf(fmaxf(second, b2), fmaxf(fminf(m0, m1), fminf(best, bm)));
+    if (bm > best) {
+        best = bm;
+        const bool low = m0 == bm;
+        int at = kHalf - 1;
+#pragma unroll
+        for (int x = kHalf - 2; x >= 0; --x) {
+            float w;
+            asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %3, 0;\n\tselp.f32 %0, %1, %2, q;\n\t}" : "=f"(w) : "f"(p[0][x]), "f"(p[1][x]), "r"((int)low));
+            if (w == bm) at = x;
+        }
+        best_u = u0 + at + (low ? 0 : kHalf);
+    }
+}
+
 template <int PAIR, bool SECOND = false>
 __device__ __forceinline__ void best_seed(uint32_t taddr, const float* inv, int c_lo, int c_hi, float& best, int& best_u, float& second) {
-    constexpr int kPer = PAIR ? 16 : 32;          // seeds per block of 32 columns
-    const uint32_t inv32 = smem_u32(inv);        // full blocks read the inverse norms 16 bytes at a time, shared-space
+    const uint32_t inv32 = smem_u32(inv);
+    const int last = max(c_lo, (c_hi - 1) & ~15);      // (every load is unconditional: past the last chunk it is that one again)
+    float a[16], b[16];
+    tc_ld16(taddr + c_lo, a);
+#pragma unroll 1
     for (int cc = c_lo; cc < c_hi; cc += 32) {
-        float v[32];
-        tc_ld32(taddr + cc, v);
-        tc_wait_ld_regs(v);
-        const int u0 = PAIR ? cc >> 1 : cc, u_hi = PAIR ? c_hi >> 1 : c_hi;
-        float bm = -INFINITY, b2 = -INFINITY;
-        auto take = [&](float x) {
-            if (SECOND) b2 = fmaxf(b2, fminf(bm, x));
-            bm = fmaxf(bm, x);
-        };
-        if (cc + 32 <= c_hi) {
-#pragma unroll
-            for (int x = 0; x < kPer; x += 4) {
-                const uint4 q = lds128(inv32 + (uint32_t)(u0 + x) * 4u);
-                const float nv[4] = {__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), __uint_as_float(q.w)};
-#pragma unroll
-                for (int y = 0; y < 4; ++y) {
-                    v[x + y] = (PAIR ? v[2 * (x + y)] + v[2 * (x + y) + 1] : v[x + y]) * nv[y];
-                    take(v[x + y]);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int x = 0; x < kPer; ++x) {
-                const float dot = PAIR ? v[2 * x] + v[2 * x + 1] : v[x];
-                v[x] = (u0 + x < u_hi) ? dot * inv[u0 + x] : -INFINITY;
-                take(v[x]);
-            }
-        }
-        if (SECOND) second = fmaxf(fmaxf(second, b2), fminf(best, bm));
-        if (bm > best) {
-            best = bm;
-            int at = kPer - 1;
-#pragma unroll
-            for (int x = kPer - 2; x >= 0; --x)
-                if (v[x] == bm) at = x;
-            best_u = u0 + at;
-        }
+        tc_wait_ld_regs(a);
+        tc_ld16(taddr + min(cc + 16, last), b);
+        best_of_chunk<PAIR, SECOND>(a, inv32, cc, c_hi, best, best_u, second);
+        tc_wait_ld_regs(b);
+        tc_ld16(taddr + min(cc + 32, last), a);
+        if (cc + 16 < c_hi) best_of_chunk<PAIR, SECOND>(b, inv32, cc + 16, c_hi, best, best_u, second);
     }
+    tc_wait_ld_regs(a);
+}
+
+// The value alone, and the chunk it is in; the seed of the rows that join (`ask`) afterwards.  Few rows do (tau is 0.9), and a search in
+// every chunk is two fifths of the instructions a tile takes.
+__device__ __forceinline__ void best_value(uint32_t taddr, const float* inv, int c_hi, float& best, int& best_chunk) {
+    const uint32_t inv32 = smem_u32(inv);
+    const int last = max(0, (c_hi - 1) & ~15);
+    auto look = [&](const float (&v)[16], int cc) __attribute__((always_inline)) {
+        float p[2][8];
+        chunk_products<0>(v, inv32, cc, c_hi, p);
+        float m0 = p[0][0], m1 = p[1][0];
+#pragma unroll
+        for (int x = 1; x < 7; x += 2) {
+            m0 = fmaxf(fmaxf(m0, p[0][x]), p[0][x + 1]);
+            m1 = fmaxf(fmaxf(m1, p[1][x]), p[1][x + 1]);
+        }
+        m0 = fmaxf(fmaxf(m0, m1), fmaxf(p[0][7], p[1][7]));
+        if (m0 > best) { best = m0; best_chunk = cc; }
+    };
+    float a[16], b[16];
+    tc_ld16(taddr, a);
+#pragma unroll 1
+    for (int cc = 0; cc < c_hi; cc += 32) {
+        tc_wait_ld_regs(a);
+        tc_ld16(taddr + min(cc + 16, last), b);
+        look(a, cc);
+        tc_wait_ld_regs(b);
+        tc_ld16(taddr + min(cc + 32, last), a);
+        if (cc + 16 < c_hi) look(b, cc + 16);
+    }
+    tc_wait_ld_regs(a);
+}
+__device__ __forceinline__ int find_seed(uint32_t taddr, const float* inv, int c_hi, bool ask, float best, int best_chunk) {
+    const uint32_t inv32 = smem_u32(inv);
+    int best_u = -1;
+    unsigned todo = __ballot_sync(0xffffffffu, ask);
+    while (todo) {                               // chunk by chunk, for all rows that have theirs there
+        const int cc = __shfl_sync(0xffffffffu, best_chunk, __ffs(todo) - 1);
+        float v[16], p[2][8];
+        tc_ld16(taddr + cc, v);
+        tc_wait_ld_regs(v);
+        chunk_products<0>(v, inv32, cc, c_hi, p);
+        int at = 15;
+#pragma unroll
+        for (int x = 14; x >= 0; --x)
+            if (p[x >> 3][x & 7] == best) at = x;
+        const bool here = ask && best_chunk == cc;
+        if (here) best_u = cc + at;
+        todo &= ~__ballot_sync(0xffffffffu, here);
+    }
+    return best_u;
 }
 
 // fp32 rows whose best cosine is within kClose of another seed's or of tau are decided by the sums assign_simt_kernel takes, one
@@ -335,7 +421,7 @@ __device__ __forceinline__ void produce_paged(const CUtensorMap* tmK, const CUte
         const Batch nxt = next_batch();
         if (cur.fresh) {
             const uint32_t sb = dual ? (ucount & 1u) : 0u, suse = dual ? (ucount >> 1) : ucount;
-            ok = mbar_wait(&bar.b_empty[sb], (suse & 1u) ^ 1u, abort_flag);
+            ok = mbar_wait<true>(&bar.b_empty[sb], (suse & 1u) ^ 1u, abort_flag);
             if (!ok) break;
             if (lane == 0) {
                 mbar_expect_tx(&bar.b_full[sb], n_kb * seed_region);
@@ -347,7 +433,7 @@ __device__ __forceinline__ void produce_paged(const CUtensorMap* tmK, const CUte
         }
         for (int t = 0; t < cur.n && ok; ++t, ++kit) {
             const int st = kit % kStages;
-            ok = mbar_wait(&bar.k_empty[st], ((kit / kStages) & 1u) ^ 1u, abort_flag);
+            ok = mbar_wait<true>(&bar.k_empty[st], ((kit / kStages) & 1u) ^ 1u, abort_flag);
             if (!ok) break;
             uint8_t* dst = k_smem + st * kKStageBytes + my_piece * sub_rows * 128;
             const int n_sub = min(pieces, (cur.T - cur.row0 - t * kTileRows + sub_rows - 1) >> piece_shift);
@@ -400,13 +486,14 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const uint32_t seed_region = dual ? 128u * 128u : kSeedRegionBytes;      // one 64-channel half of a seed buffer
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 2; ++i) { mbar_init(&bar.b_full[i], 1); mbar_init(&bar.b_empty[i], 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar.b_full[i], 1); mbar_init(&bar.b_empty[i], SPLIT || !dual ? 1 : 2); }
         for (int i = 0; i < kRegions; ++i) { mbar_init(&bar.k_full[i], 1); mbar_init(&bar.k_empty[i], SPLIT ? 1 : 1 + 4); }
         for (int i = 0; i < kMaxGroups; ++i) { mbar_init(&bar.d_full[i], 1); mbar_init(&bar.d_empty[i], 4 * split); }
         for (int i = 0; i < kMaxGroups; ++i) mbar_init(&bar.inv_ready[i], 128);
         mbar_init(&bar.x_full[0], 4);
         mbar_init(&bar.x_full[1], 4);
-        mbar_init(&bar.mma_drain, 1);
+        mbar_init(&bar.mma_drain[0], 1);
+        mbar_init(&bar.mma_drain[1], 1);
         tail->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -440,14 +527,14 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         // parts in the order of their use, l, m, h; part p of the keys starts p * sub_rows rows down the table
                         for (int r = 0; r < kRegions && ok; ++r) {
                             if ((r & 1) >= n_kb) continue;
-                            ok = mbar_wait(&bar.k_empty[r], (kit & 1u) ^ 1u, abort_flag);
+                            ok = mbar_wait<true>(&bar.k_empty[r], (kit & 1u) ^ 1u, abort_flag);
                             if (!ok) break;
                             mbar_expect_tx(&bar.k_full[r], kKRegionBytes);
                             tma_load_2d(k_smem + r * kKRegionBytes, &tmK, &bar.k_full[r], 64 * (r & 1),
                                         (2 - (r >> 1)) * sub_rows + krow0 + t * kTileRows);
                         }
                         if (t == 0 && ok) {
-                            ok = mbar_wait(&bar.b_empty[0], (ucount & 1u) ^ 1u, abort_flag);
+                            ok = mbar_wait<true>(&bar.b_empty[0], (ucount & 1u) ^ 1u, abort_flag);
                             if (!ok) break;
                             mbar_expect_tx(&bar.b_full[0], 3 * n_kb * kKRegionBytes);
                             for (int r = 0; r < kRegions; ++r)
@@ -461,7 +548,7 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     continue;
                 }
                 const uint32_t sb = dual ? (ucount & 1u) : 0u, suse = dual ? (ucount >> 1) : ucount;
-                ok = mbar_wait(&bar.b_empty[sb], (suse & 1u) ^ 1u, abort_flag);
+                ok = mbar_wait<true>(&bar.b_empty[sb], (suse & 1u) ^ 1u, abort_flag);
                 if (!ok) break;
                 mbar_expect_tx(&bar.b_full[sb], n_kb * seed_region);
                 uint8_t* bdst = b_smem + sb * 2 * seed_region;
@@ -472,7 +559,7 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 const int nt = wk.run();
                 for (int t = 0; t < nt && ok; ++t, ++kit) {
                     const int st = kit % kStages;
-                    ok = mbar_wait(&bar.k_empty[st], ((kit / kStages) & 1u) ^ 1u, abort_flag);
+                    ok = mbar_wait<true>(&bar.k_empty[st], ((kit / kStages) & 1u) ^ 1u, abort_flag);
                     if (!ok) break;
                     uint8_t* dst = k_smem + st * kKStageBytes;
                     mbar_expect_tx(&bar.k_full[st], n_kb * kKRegionBytes);
@@ -490,8 +577,8 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     for (uint32_t it = 0; it < 4096 && !mbar_try(&bar.k_full[j % kStages], (j / kStages) & 1u); ++it) {}
             }
         }
-    } else if (warp == 1) {
-        // ================= MMA issuer =================
+    } else if (warp == 1 || (!SPLIT && dual && warp == 2)) {        // (with two buffers a second issuer's contractions only delay the first one's)
+        // ================= MMA issuers: even and odd tiles =================
         if (lane == 0) {
             uint32_t kit = 0, ucount = 0;
             bool ok = true;
@@ -502,16 +589,16 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 const int m = MANY ? min(m_all - c0, chunk.width) : m_all;
                 const uint32_t idesc = umma_idesc(max(16, ((m << wpair) + 15) & ~15));
                 if constexpr (SPLIT) {
-                    ok = mbar_wait(&bar.b_full[0], ucount & 1u, abort_flag);
+                    ok = mbar_wait<true>(&bar.b_full[0], ucount & 1u, abort_flag);
                     if (!ok) break;
                     ++ucount;
                     const int nt = wk.run();
                     for (int t = 0; t < nt && ok; ++t, ++kit) {
                         const uint32_t buf = kit & buf_mask, use = kit >> buf_shift;
-                        ok = mbar_wait(&bar.d_empty[buf], (use & 1u) ^ 1u, abort_flag);
+                        ok = mbar_wait<true>(&bar.d_empty[buf], (use & 1u) ^ 1u, abort_flag);
 #pragma unroll
                         for (int kp = 0; kp < 3; ++kp) {
-                            for (int kb = 0; kb < n_kb && ok; ++kb) ok = mbar_wait(&bar.k_full[2 * kp + kb], kit & 1u, abort_flag);
+                            for (int kb = 0; kb < n_kb && ok; ++kb) ok = mbar_wait<true>(&bar.k_full[2 * kp + kb], kit & 1u, abort_flag);
                             if (!ok) break;
                             tc_fence_after();
 #pragma unroll
@@ -540,17 +627,18 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     continue;
                 }
                 const uint32_t sb = dual ? (ucount & 1u) : 0u, suse = dual ? (ucount >> 1) : ucount;
-                ok = mbar_wait(&bar.b_full[sb], suse & 1u, abort_flag);
+                ok = mbar_wait<true>(&bar.b_full[sb], suse & 1u, abort_flag);
                 if (!ok) break;
                 ++ucount;
                 const uint32_t bu_lo = b_lo + ((sb * 2 * seed_region) >> 4), half_lo = seed_region >> 4;
                 const int nt = wk.run();
                 for (int t = 0; t < nt && ok; ++t, ++kit) {
+                    if (dual && (kit & 1u) != (uint32_t)warp - 1u) continue;
                     const int st = kit % kStages;
                     const uint32_t buf = kit & buf_mask, use = kit >> buf_shift;
-                    ok = mbar_wait(&bar.k_full[st], (kit / kStages) & 1u, abort_flag);
+                    ok = mbar_wait<true>(&bar.k_full[st], (kit / kStages) & 1u, abort_flag);
                     if (!ok) break;
-                    ok = mbar_wait(&bar.d_empty[buf], (use & 1u) ^ 1u, abort_flag);
+                    ok = mbar_wait<true>(&bar.d_empty[buf], (use & 1u) ^ 1u, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t kst_lo = k_lo + st * (kKStageBytes >> 4);
@@ -572,8 +660,8 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             if (!ok) {
                 // contractions already issued may still be running: the TMEM they write is freed below, so give them
                 // a bounded wait (a commit completes when everything this thread issued before it has)
-                tc_commit(&bar.mma_drain);
-                for (uint32_t it = 0; it < 4096 && !mbar_try(&bar.mma_drain, 0u); ++it) {}
+                tc_commit(&bar.mma_drain[warp - 1]);
+                for (uint32_t it = 0; it < 4096 && !mbar_try(&bar.mma_drain[warp - 1], 0u); ++it) {}
             }
         }
     } else if (warp >= kEpiWarp0) {
@@ -626,20 +714,22 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     srow[c] = (c < m) ? seed_rows[seed_base + c] : 0;
                 }
                 mbar_arrive(&bar.inv_ready[ew >> 2]);
-                ok = mbar_wait(&bar.inv_ready[ew >> 2], ucount & 1u, abort_flag);
+                ok = mbar_wait<true>(&bar.inv_ready[ew >> 2], ucount & 1u, abort_flag);
                 if (!ok) break;
             }
             ++ucount;
             uint8_t kd_n = (uint8_t)CASK_KIND_RECENT;
             float s_n = 0.f, mi_n = 0.f, nj_n = 0.f;
             bool pre = false;
-            for (int t = 0; t < nt && ok; ++t, ++kit) {
-                if ((kit & buf_mask) != eg) continue;
-                const int st = kit % kStages;
-                const uint32_t use = kit >> buf_shift;
+            unsigned long long lost = 0ull;                  // masses of the thread's rows that join no group, and rows of the warp that do
+            int n_joined = 0;
+            for (int t = first; t < nt && ok; t += n_bufs) {
+                const uint32_t tile = kit + (uint32_t)t;
+                const int st = tile % kStages;
+                const uint32_t use = tile >> buf_shift;
                 if (half == 1) {
                     // second group of a shared buffer: best seed among the columns [c_split, m)
-                    ok = mbar_wait(&bar.d_full[eg], use & 1u, abort_flag);
+                    ok = mbar_wait<true>(&bar.d_full[eg], use & 1u, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     float best = -INFINITY, second = 0.f;
@@ -696,7 +786,7 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 // sixteen 16-byte pieces of the row gives the same set of elements)
                 uint64_t n2p = 0ull;
                 if (!SPLIT) {
-                    ok = mbar_wait(&bar.k_full[st], (kit / kStages) & 1u, abort_flag);
+                    ok = mbar_wait<true>(&bar.k_full[st], (tile / kStages) & 1u, abort_flag);
                     if (!ok) break;
                 }
                 if (!SPLIT && last) {
@@ -709,12 +799,17 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 n2 += n2b;
                 __syncwarp();
                 if (!SPLIT && lane == 0) mbar_arrive(&bar.k_empty[st]);
-                ok = mbar_wait(&bar.d_full[eg], use & 1u, abort_flag);
+                ok = mbar_wait<true>(&bar.d_full[eg], use & 1u, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 float best = -INFINITY, second = -INFINITY;
                 int best_u = -1;
-                if (!SPLIT && wpair) best_seed<1>(taddr, inv, 0, c_split, best, best_u, second);
+                // Few rows join where tau is high: their seeds are looked for afterwards.  (Below, with most rows joining, that is a second way
+                // through all chunks: 112 units of 8,448 rows, tau = 0.3, 65 to 72 us; searched in every chunk 66.)
+                const bool late = !SPLIT && !MANY && dual && !wpair && tau >= 0.5f;
+                int best_chunk = 0;
+                if (late) best_value(taddr, inv, mc, best, best_chunk);
+                else if (!SPLIT && wpair) best_seed<1>(taddr, inv, 0, c_split, best, best_u, second);
                 else best_seed<0, SPLIT || MANY>(taddr, inv, 0, c_split, best, best_u, second);
                 if (MANY) {
                     tc_fence_before();
@@ -731,7 +826,7 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         continue;
                     }
                 }
-                bool cand = in_range && best_u >= 0 && kd == CASK_KIND_DROPPED;
+                bool cand = in_range && (late ? best > -INFINITY : best_u >= 0) && kd == CASK_KIND_DROPPED;
                 if (MANY) {
                     const float nj = sqrtf(n2), by = kClose * nj;
                     const bool unsure = in_range && m_all > 0 && kd == CASK_KIND_DROPPED && !(best_u >= 0 && second < best - by && fabsf(best - tau * nj) > by);
@@ -765,13 +860,19 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         if (m < 32 * b + 32) close[b] &= (1u << (m - 32 * b)) - 1u;
                     }
                 }
+                float sm_ = 0.f;
+                if (late) {
+                    const float nj = sqrtf(n2);
+                    sm_ = cand && nj > 0.f ? best / nj : 0.f;
+                    best_u = find_seed(taddr, inv, mc, cand && sm_ >= tau, best, best_chunk);
+                }
                 if (!MANY) tc_fence_before();
                 if (!MANY && split == 2) {
                     // The other group's candidate has the larger seed indices, so it wins only when strictly
                     // better: the same outcome as one scan over all columns.  The buffer is released after this
                     // read, so the other group cannot start the buffer's next use (and overwrite its hand-over
                     // slot or run a barrier phase ahead) before it.
-                    ok = mbar_wait(&bar.x_full[eg], use & 1u, abort_flag);
+                    ok = mbar_wait<true>(&bar.x_full[eg], use & 1u, abort_flag);
                     if (!ok) break;
                     const float ov = tail->x_val[eg][use & 1u][my_row];
                     if (ov > best) {
@@ -784,10 +885,9 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     if (lane == 0) mbar_arrive(&bar.d_empty[eg]);
                 }
 
-                float sm_ = 0.f;
                 if (cand) {
                     const float nj = SPLIT ? nj_c : sqrtf(n2);              // best = <k_row, k_seed> / |k_seed| (0 for a zero seed)
-                    sm_ = nj > 0.f ? best / nj : 0.f;
+                    if (!late) sm_ = nj > 0.f ? best / nj : 0.f;
                     if (SPLIT && plain) best_u = plain_best(K, sh, ud, i, srow, seed_norm + seed_base, close, sm_);
                     if (sim) sim[tok_off + i] = sm_;
                 }
@@ -802,7 +902,7 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     grp[tok_off + i] = bu;
                     atomicAdd(&mass_u[bu], fx);
                 }
-                // Joiner count and lost mass go out once per warp: the fixed-point sums are exact, so
+                // Joiner count and lost mass go out once per warp and unit: the fixed-point sums are exact, so
                 // the grouping of the additions does not show in the result.
                 const unsigned jb = __ballot_sync(0xffffffffu, joined);
                 if (jb && mem_row) {                              // (few: the compaction takes them from this list)
@@ -814,14 +914,16 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         mem_seed[tok_off + at] = best_u;
                     }
                 }
-                unsigned long long lost = joined ? 0ull : fx;
-#pragma unroll
-                for (int off = 16; off >= 1; off >>= 1) lost += __shfl_xor_sync(0xffffffffu, lost, off);
-                if (lane == 0) {
-                    if (jb && !mem_row) atomicAdd(&njoin[u], __popc(jb));
-                    if (lost) atomicAdd(&mass_u[max_m], lost);
-                }
+                n_joined += __popc(jb);
+                if (!joined) lost += fx;
             }
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1) lost += __shfl_xor_sync(0xffffffffu, lost, off);
+            if (lane == 0) {
+                if (n_joined && !mem_row) atomicAdd(&njoin[u], n_joined);
+                if (lost) atomicAdd(&mass_u[max_m], lost);
+            }
+            kit += nt;
             wk.advance(nt);
         }
     }

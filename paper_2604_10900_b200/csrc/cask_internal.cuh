@@ -395,7 +395,7 @@ __device__ __forceinline__ uint32_t order_key(float x) {
 // fixed-point image of a mass a in [0, 2^20): 2^43 steps per unit
 constexpr double kMassScale = 8796093022208.0;   // 2^43
 __device__ __forceinline__ unsigned long long mass_to_fx(float a) {
-    return (unsigned long long)__double2ll_rn((double)a * kMassScale);
+    return (unsigned long long)__float2ll_rn(a * (float)kMassScale);      // (a power of two: the product is exact in fp32 too)
 }
 __device__ __forceinline__ float fx_to_mass(unsigned long long f) {
     return (float)((double)f / kMassScale);
