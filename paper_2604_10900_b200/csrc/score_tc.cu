@@ -396,10 +396,13 @@ __device__ __forceinline__ void load_query_block(const CUtensorMap* tmQ, uint64_
             tma_load_3d(dst + kb * region + x * 4096, tmQ, bar, kb * 64, row0 + ((32 * x + block_turn<PASS, NB>(b)) & 127), u);
 }
 
-// The TMA producer of a paged cache (one warp).  A lane owns a page piece of every tile: it looks its page up a tile ahead (the latency of the block table hides behind the tile before)
-// and issues its own boxes.  One lane doing that piece by piece took 5,600 clk a tile with pages of 16 rows, more than the
-// tile's exponentials (3,072 such units of 640 rows: passes 377 + 370 to 356 + 339 us).  The waits, and the order of copies, are
-// those of the contiguous producer in score_tc_kernel.
+// The TMA producer of a paged cache (one warp).  A lane owns a page piece of a tile and issues its boxes.  The block table is read for as many
+// tiles of a segment at once as the lanes have pieces, and one such batch ahead of its use: nothing touches a page number, not even to
+// check it, before its own tiles are issued, so the table's latency hides behind the batch before.  (One lane going through the pieces took
+// 5,600 clk a tile with pages of 16 rows; lanes that looked up and checked their pages a tile ahead waited for them every tile, 2,800 clk, more
+// than the tiles of 256 query rows and fewer take: 216 units of 6,600 rows, 64 query rows, pages of 16, passes 119 + 118 to 94 + 97 us (76 + 70 with
+// contiguous rows), event 388 to 340; with 256 query rows 466 to 410, head_dim 64 369 to 345; 512 rows even.)  The waits, and the order of copies, are those of the contiguous
+// producer in score_tc_kernel.
 template <int PASS, int NB, bool PLAIN>
 __device__ __forceinline__ void produce_paged(const CUtensorMap* tmK, const CUtensorMap* tmQ, const Shape& sh, TileWalk<!PLAIN> wk,
                                               int per, int block_rows, int sub_rows, int n_kb, uint8_t* q_smem, uint8_t* k_smem,
@@ -409,33 +412,51 @@ __device__ __forceinline__ void produce_paged(const CUtensorMap* tmK, const CUte
     auto& bar = tail->bar;
     volatile int* abort_flag = &tail->abort;
     const int lane = threadIdx.x & 31, n_blk = (per + block_rows - 1) / block_rows;
+    const int piece_shift = 31 - __clz(sub_rows), tile_shift = 7 - piece_shift;      // rows of a piece, pieces of a tile
+    const int my_tile = lane >> tile_shift, my_piece = lane & ((1 << tile_shift) - 1);
     uint32_t kit = 0, seg = 0;
     bool ok = true;
     TileWalk<!PLAIN> pf = wk;
-    int pf_t = 0, bt0 = -1, prow = 0;
-    auto look_up = [&]() {
-        const int row = pf.key_begin() + pf_t * kTileKeys + lane * sub_rows;
+    int pf_t = 0, bt0 = -1;
+    struct Batch { int n, page, in_page; };
+    auto next_batch = [&]() {
+        Batch b{0, 0, 0};
+        if (!pf.valid()) return b;
+        const int left = pf.seg_tiles() - pf_t, row = pf.key_begin() + (pf_t + my_tile) * kTileKeys + my_piece * sub_rows;
         if (bt0 < 0) bt0 = pf.desc[pf.u].bt0;
-        if (lane * sub_rows < kTileKeys && row < pf.T) prow = (int)paged_row(sh, bt0, row);
+        b.n = min(left, 32 >> tile_shift);
+        if (my_tile < b.n && row < pf.T) {
+            const int pg = row / sh.page_size;
+            b.page = sh.bt[bt0 + pg];
+            b.in_page = row - pg * sh.page_size;
+        }
+        pf_t += b.n;
+        if (b.n == left) { pf.next_segment(); pf_t = 0; bt0 = -1; }
+        return b;
     };
-    if (pf.valid()) look_up();
+    Batch cur = next_batch(), nxt = next_batch();
+    int at = 0;                                  // tile of the batch
     for (; wk.valid() && ok; wk.next_segment(), ++seg) {
         const int key_begin = wk.key_begin(), nt = wk.seg_tiles();
         for (int t = 0; t < nt && ok; ++t, ++kit) {
             const int st = kit % kStages;
             ok = mbar_wait<true>(&bar.k_empty[st], ((kit / kStages) & 1u) ^ 1u, abort_flag);
             if (!ok) break;
-            uint8_t* dst = k_smem + st * kKStageBytes;
+            uint8_t* dst = k_smem + st * kKStageBytes + my_piece * sub_rows * 128;
             // pieces past the end of the unit are not read (their accumulator rows / columns are masked by the epilogue)
-            const int n_sub = min(kTileKeys / sub_rows, (wk.T - key_begin - t * kTileKeys + sub_rows - 1) / sub_rows);
-            if (lane == 0) mbar_expect_tx(&bar.k_full[st], (uint32_t)n_sub * sub_rows * (128u * n_kb));
+            const int n_sub = min(kTileKeys >> piece_shift, (wk.T - key_begin - t * kTileKeys + sub_rows - 1) >> piece_shift);
+            if (lane == 0) mbar_expect_tx(&bar.k_full[st], (uint32_t)(n_sub << piece_shift) * (128u * n_kb));
             __syncwarp();
-            if (lane < n_sub) {
-                tma_load_2d(dst + lane * sub_rows * 128, tmK, &bar.k_full[st], 0, prow);
-                if (n_kb == 2) tma_load_2d(dst + kKRegionBytes + lane * sub_rows * 128, tmK, &bar.k_full[st], 64, prow);
+            if (my_tile == at && my_piece < n_sub) {
+                const int prow = (int)page_row(sh, cur.page, cur.in_page);
+                tma_load_2d(dst, tmK, &bar.k_full[st], 0, prow);
+                if (n_kb == 2) tma_load_2d(dst + kKRegionBytes, tmK, &bar.k_full[st], 64, prow);
             }
-            if (++pf_t >= pf.seg_tiles()) { pf.next_segment(); pf_t = 0; bt0 = -1; }
-            if (pf.valid()) look_up();
+            if (++at == cur.n) {
+                cur = nxt;
+                nxt = next_batch();
+                at = 0;
+            }
             for (int j = 0; t == 0 && j < NB && ok; ++j) {
                 ok = mbar_wait<true>(&bar.q_empty[j], (seg & 1u) ^ 1u, abort_flag);
                 if (!ok || lane != 0) continue;
