@@ -317,6 +317,7 @@ __device__ __forceinline__ void make_row_table(int u, int rg, int lo, int cnt, b
         return;
     }
     const size_t p0 = ((size_t)parts * (u * rgs.groups + rg) + lo) * part_step;
+#pragma unroll 1
     for (int r = idx; r < limit; r += n) {
         if (r >= rows) { rc[r] = -1.0e30f; continue; }
         const float *pm = part_m + p0 + r, *pl = part_l + p0 + r;
@@ -362,7 +363,7 @@ __device__ __forceinline__ void copy_table(const float* __restrict__ tables, int
     for (int r = idx; r < 512; r += n) rc[r] = r < rows ? src[r] : -1.0e30f;
 }
 
-constexpr int kRowThreads = 128;
+constexpr int kRowThreads = 512;
 __global__ void __launch_bounds__(kRowThreads) score_row_tables(const UnitDesc* __restrict__ desc, RowGroups rgs, int nb, int total_tiles,
                                                                 int grid, const float* __restrict__ part_m,
                                                                 const float* __restrict__ part_l, float* __restrict__ tables,
@@ -540,7 +541,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // pass's CTAs have come back: pdl_wait() waits first and releases afterwards.  With score_row_tables between the two, pass N itself is
     // over.  Nothing changes it while pass S runs.  (The fence drops what this SM's L1 may hold of an earlier call's; reading past the
     // L1 instead costs eight units of 640 rows 0.3 us of 49.6.)
-    if (PASS == 0 || !ahead) pdl_wait();
+    if (PASS == 0 && ahead) asm volatile("griddepcontrol.wait;" ::: "memory");        // (`ahead` there: the next kernel starts when this one has ended)
+    else if (PASS == 0 || !ahead) pdl_wait();
     else __threadfence();
 
     TileWalk<!PLAIN || SPLIT> wk;
@@ -1310,16 +1312,18 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     const int bit = kSmemBitScore + 2 * (NB >> 1) + 6 * PLAIN + 12 * SPLIT;
     cudaError_t e = lse_in ? cudaSuccess : allow_smem(L, bit, norm, smem);
     if (e == cudaSuccess) e = allow_smem(L, bit + 1, mass, smem);
+    const bool own_tables = !lse_in && sh.n_units * rg.groups > grid;       // the row tables by a kernel of their own
     if (e == cudaSuccess && !lse_in) {
         Timed t(L, KID_SCORE_NORM);
         e = launch_kernel(total < 256 * grid, L.stream, norm, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
-                             ws.part_l, nullptr, nullptr, nullptr, nullptr, 0, RowDefaults{}, 0, nullptr, ws.err);
+                             ws.part_l, nullptr, nullptr, nullptr, nullptr, 0, RowDefaults{}, own_tables, nullptr, ws.err);
     }
-    const bool own_tables = !lse_in && sh.n_units * rg.groups > grid;       // the row tables by a kernel of their own
     if (e == cudaSuccess && own_tables) {
         Timed t(L, KID_ROW_COMBINE);
-        // (never early: its CTAs would hold slots of the score pass that follows; 288 units of 640 rows 149.4 to 148.2 us)
-        e = launch_kernel(false, L.stream, score_row_tables, sh.n_units * rg.groups, kRowThreads, 0, L.desc, rg, NB, total, grid, ws.part_m,
+        // A row a thread (the rows rolled: the code runs once): with four rows a thread, 128 threads, 288 units of 640 rows 134.9 to 133.4 us,
+        // 300 of 4,000 548 to 542.  Launched dependent, but the normaliser pass does not release it, so that its CTAs hold no slots of
+        // that pass or of the next and it need not wait for an ordinary launch: 296 units of 640 143.6 to 142.4, 600 270 to 267.7.
+        e = launch_dependent(L.stream, score_row_tables, sh.n_units * rg.groups, kRowThreads, 0, L.desc, rg, NB, total, grid, ws.part_m,
                              ws.part_l, ws.rowm, lse_out);
     }
     if (e == cudaSuccess) {
