@@ -855,8 +855,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             // The code of the row tables once through on nothing while pass N still runs: fetching its instructions is most of what
             // the first table costs (one partial address for all, out of `scratch`, into the room of the key sums).  A unit of one tile
             // (the 1): one round over the partials, whatever the segment's own unit has.  The rounds of a unit that many CTAs share go on
-            // when pass N, short there, is long over: event of four units of 9,000 rows 79.4 us with them, 72.5 without.
-            if (!tables && wk.valid())
+            // when pass N, short there, is long over: event of four units of 9,000 rows 79.4 us with them, 72.5 without.  (ahead > 1: pass N
+            // leaves SMs free.  Else this CTA began when pass N's had left its SM, and there is little to wait for: those four units 71.2
+            // to 69.7, with head_dim 64 74.0 to 72.2, eight of 9,000 82.1 to 81.0; 112 of 8,448 even.)
+            if (!tables && wk.valid() && ahead > 1)
                 row_table(wk.u, 0, 1, wk.tile0, false, rgs, NB, total_tiles, gridDim.x, scratch, scratch, nullptr, nullptr,
                           &tail->red[0][0][0], etid, 32 * kEpiWarps, 0);
             pdl_wait();
@@ -1331,7 +1333,7 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
         const bool early = lse_in || total < 256 * grid;
         e = launch_kernel(early, L.stream, mass, grid, kThreadsTc, smem, tmK, tmQ, L.desc, sh, rg, scale2, total, sub_rows, ws.part_m,
                              ws.part_l, lse_in, lse_out, own_tables ? ws.rowm : nullptr, rg.groups > 1 ? ws.s_part : s, rg.groups > 1 ? L.sum_T : 0, L.fill,
-                             early && !lse_in, ws.roww, ws.err);
+                             early && !lse_in ? (grid < L.sms ? 2 : 1) : 0, ws.roww, ws.err);
         ws.filled = L.fill.kind != nullptr;
         if (e == cudaSuccess && rg.groups > 1) {
             const int per = kFoldThreads * kFoldKeys;
