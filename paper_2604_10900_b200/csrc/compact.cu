@@ -483,11 +483,23 @@ struct RowSource {
     int u;
 };
 
+template <int N> struct alignas(4 * N) Words { uint32_t w[N]; };
+// Channel x of them (whole words, so that a row can be left out without its registers going to memory).
+template <typename T, int N>
+__device__ __forceinline__ float channel(const Words<N>& p, int x) {
+    if (sizeof(T) == 4) return __uint_as_float(p.w[x < N ? x : 0]);
+    const uint32_t w = p.w[(x >> 1) < N ? x >> 1 : 0];
+    return __uint_as_float(x & 1 ? w & 0xFFFF0000u : w << 16);
+}
+
 // Two kinds of work, handed out to the warps of a unit's CTAs one after the other:
 //   * the slots that others joined, `per_item` of them at a time: their members' rows are added up (ascending row order, fp32, rounded
 //     once) and written out.  A lane looks one member up (page, score, carried mass, group mass) and the rows are loaded kRows at
-//     a time whatever slots they feed.  (Eight rows spill, and the bf16 kernels are slower with them.)  They come first: a
-//     group is a chain of memory latencies, three and one more per four members.
+//     a time whatever slots they feed: eight where a lane's piece of a row is one word, else four (eight of two words spill, and cost eight
+//     units of 33,280 rows 2 us).  Where the rows lie and what they count goes through shared memory: by shuffles, six a row, a member took
+//     0.24 us of a group's time, now 0.15 (128 units of 4,608 rows at head_dim 64, kernel alone 31.2 to 27.5; 8 of 9,000 29.1 to 24.1; 240 of
+//     1,024 whose other rows all join 69.4 to 64.6).  They come first: a group is a chain of memory latencies, three and one more per
+//     kRows members.
 //   * batches of consecutive slots: bulk copies of the rows of the other ones into the warp's staging buffer, then bulk stores, two
 //     for a batch without merged slots, because consecutive slots are contiguous in the output; two buffers, so the copies of a
 //     batch run under the stores of the one before.
@@ -512,8 +524,9 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
                                              Busy busy) {
     using namespace tc;
     constexpr int kPer = CH > 0 ? CH : 8;
-    constexpr int kRows = 4;                     // member rows in flight
+    constexpr int kRows = CH > 0 && CH * sizeof(T) <= 4 ? 8 : 4;           // member rows in flight
     struct alignas((CH > 0 ? CH : 1) * sizeof(T)) Vec { T x[CH > 0 ? CH : 1]; };
+    using Piece = Words<(CH > 0 ? CH * sizeof(T) / 4 : 1)>;      // a lane's channels of a row
     const Shape& sh = in.sh;
     const UnitDesc& ud = in.ud;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, u = in.u, d = sh.d;
@@ -522,6 +535,11 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
     const int sb = min(32, (int)(STAGE / 2 / row_bytes));                  // slots per batch
     volatile int* abort_flag = abort_word;
     uint8_t* my = staging + w * 2 * STAGE;
+    // (a warp's merged slots come before its batches of rows to copy: the staging area is free until then)
+    int64_t* at_k = reinterpret_cast<int64_t*>(my);
+    int64_t* at_v = at_k + 32;
+    float2* counts = reinterpret_cast<float2*>(at_v + 32);
+    static_assert(2 * STAGE >= 24 * 32, "one member a lane");
     const int nb = (nk + sb - 1) / sb, n_items = (n_busy + per_item - 1) / per_item;
     uint32_t it = 0;
     bool ok = true;
@@ -595,27 +613,35 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
                 const float ae = row_mass(sh, in.s, in.eps, o + row);
                 const float mg = __shfl_sync(0xffffffffu, mg_t, sl);
                 const float we = in.fw.s ? ae / mg : in.weight[o + row];
+                __syncwarp();
+                at_k[lane] = ko;
+                at_v[lane] = vo;
+                counts[lane] = make_float2(we, ae);
+                __syncwarp();
                 for (int c0 = 0; c0 < n; c0 += kRows) {
-                    Vec kr[kRows], vr[kRows];
+                    Piece kr[kRows], vr[kRows];
                     if (CH > 0) {
 #pragma unroll
                         for (int q = 0; q < kRows; ++q) {
-                            kr[q] = reinterpret_cast<const Vec*>(in.K + __shfl_sync(0xffffffffu, ko, c0 + q))[lane];
-                            vr[q] = reinterpret_cast<const Vec*>(in.V + __shfl_sync(0xffffffffu, vo, c0 + q))[lane];
+                            kr[q] = vr[q] = Piece{};
+                            if (c0 + q < n) {
+                                kr[q] = reinterpret_cast<const Piece*>(in.K + at_k[c0 + q])[lane];
+                                vr[q] = reinterpret_cast<const Piece*>(in.V + at_v[c0 + q])[lane];
+                            }
                         }
                     }
 #pragma unroll
                     for (int q = 0; q < kRows; ++q) {
                         if (c0 + q >= n) break;
-                        const float wi = __shfl_sync(0xffffffffu, we, c0 + q);
-                        msum += __shfl_sync(0xffffffffu, ae, c0 + q);
-                        const int64_t kq = CH > 0 ? 0 : __shfl_sync(0xffffffffu, ko, c0 + q);
-                        const int64_t vq = CH > 0 ? 0 : __shfl_sync(0xffffffffu, vo, c0 + q);
+                        const float wi = counts[c0 + q].x;
+                        msum += counts[c0 + q].y;
+                        const int64_t kq = CH > 0 ? 0 : at_k[c0 + q];
+                        const int64_t vq = CH > 0 ? 0 : at_v[c0 + q];
 #pragma unroll
                         for (int x = 0; x < kPer; ++x) {
                             if (CH > 0) {
-                                ak[x] = fmaf(wi, Elem<T>::ld(&kr[q].x[CH > 0 ? x : 0]), ak[x]);
-                                av[x] = fmaf(wi, Elem<T>::ld(&vr[q].x[CH > 0 ? x : 0]), av[x]);
+                                ak[x] = fmaf(wi, channel<T>(kr[q], x), ak[x]);
+                                av[x] = fmaf(wi, channel<T>(vr[q], x), av[x]);
                             } else if (lane + 32 * x < d) {
                                 ak[x] = fmaf(wi, Elem<T>::ld(in.K + kq + lane + 32 * x), ak[x]);
                                 av[x] = fmaf(wi, Elem<T>::ld(in.V + vq + lane + 32 * x), av[x]);
@@ -641,6 +667,7 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
         const int n_copied = __popc(__ballot_sync(0xffffffffu, copied));
         // the stores that read this buffer two batches ago must have read it (every lane has groups of its own)
         asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        if (it == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // (the members' places are written over)
         if (lane == 0) mbar_expect_tx(&bars[w][st], (uint32_t)n_copied * 2u * row_bytes);
         __syncwarp();
         if (copied) {
