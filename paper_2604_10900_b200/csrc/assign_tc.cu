@@ -826,10 +826,11 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         continue;
                     }
                 }
+                if (MANY && n2 == 0.f && m_all > 0) { best = 0.f; best_u = 0; }        // a row of zeros: cosine 0 with every seed, nothing to tell apart
                 bool cand = in_range && (late ? best > -INFINITY : best_u >= 0) && kd == CASK_KIND_DROPPED;
                 if (MANY) {
                     const float nj = sqrtf(n2), by = kClose * nj;
-                    const bool unsure = in_range && m_all > 0 && kd == CASK_KIND_DROPPED && !(best_u >= 0 && second < best - by && fabsf(best - tau * nj) > by);
+                    const bool unsure = in_range && m_all > 0 && n2 != 0.f && kd == CASK_KIND_DROPPED && !(best_u >= 0 && second < best - by && fabsf(best - tau * nj) > by);
                     const unsigned ub = __ballot_sync(0xffffffffu, unsure);
                     if (ub) {
                         int at = 0;
@@ -940,64 +941,123 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // MANY: the rows whose cosines with two seeds, or with one and tau, lie within what the sums of the tensor cores may be off.  A CTA a row, a
 // thread every 256th seed; the additions are those of assign_simt_kernel.  Bound by latency (list, unit, row, seeds in series), so
 // a seed's row is read 128 bytes at a time.  16 units of 15,276 rows, 380 seeds: 44 us with a warp a row, 15 so.
-constexpr int kCloseThreads = 256;
-__global__ void __launch_bounds__(kCloseThreads) assign_close_kernel(
+// Caches whose rows repeat list nearly all of them; a seed's row then is read once for eight (kCloseRows) rows of a unit, which stand
+// side by side in the list.  240 units of 3,000 rows drawn from 64 keys each (event): 18.7 ms a row at a time, 5.7 so (SIMT kernel 5.1); four of
+// 9,000 2,252 and 714 us (524).  Rows of zeros, whose cosine is 0 without a sum, are not listed: half of the rows 17.1 to 0.68 ms.
+constexpr int kCloseThreads = 256, kCloseRows = 8, kClosePitch = 132;      // (pitch: 16-byte pieces, and no conflicts where four threads take a row)
+struct CloseSmem {
+    alignas(16) float row[kCloseRows][kClosePitch];
+    float norm[kCloseRows];
+    float best[kCloseRows][kCloseThreads / 32];
+    int best_u[kCloseRows][kCloseThreads / 32];
+};
+
+// Greatest cosine (the first seed among equals) of the R rows in shared memory, to best[.][0] and best_u[.][0].
+template <int R>
+__device__ __forceinline__ void close_best(CloseSmem& sm, const __nv_bfloat16* __restrict__ seed_k, const float* __restrict__ seed_norm, int seed_base, int m, int d) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (R > 1) {
+        if (tid < 4 * R) {
+            float n2 = 0.f;
+            for (int c = tid & 3; c < d; c += 4) n2 = fmaf(sm.row[tid >> 2][c], sm.row[tid >> 2][c], n2);
+            n2 += __shfl_xor_sync(0xffffffffu, n2, 1);
+            n2 += __shfl_xor_sync(0xffffffffu, n2, 2);
+            if ((tid & 3) == 0) sm.norm[tid >> 2] = sqrtf(n2);
+        }
+        __syncthreads();
+    }
+    float best[R];
+    int best_u[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) { best[r] = -INFINITY; best_u[r] = -1; }
+    for (int j = tid; j < m; j += kCloseThreads) {
+        const uint4* seed = reinterpret_cast<const uint4*>(seed_k + (size_t)(seed_base + j) * d);
+        const float nu = seed_norm[seed_base + j];
+        float acc[R], n2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = 0.f;
+#pragma unroll(R == 1 ? 8 : 2)
+        for (int c = 0; c < d / 8; ++c) {
+            const uint4 v = seed[c];
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float4 r0 = *reinterpret_cast<const float4*>(&sm.row[r][8 * c]), r1 = *reinterpret_cast<const float4*>(&sm.row[r][8 * c + 4]);
+                const float x[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+#pragma unroll
+                for (int y = 0; y < 8; ++y) {
+                    if (R == 1) n2[y & 3] = fmaf(x[y], x[y], n2[y & 3]);
+                    acc[r] = fmaf(x[y], __uint_as_float(y & 1 ? w[y >> 1] & 0xFFFF0000u : w[y >> 1] << 16), acc[r]);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float nj = R == 1 ? sqrtf((n2[0] + n2[1]) + (n2[2] + n2[3])) : sm.norm[r];
+            const float v = nj > 0.f && nu > 0.f ? acc[r] / (nj * nu) : 0.f;
+            if (v > best[r]) { best[r] = v; best_u[r] = j; }
+        }
+    }
+    auto fold = [&](float& b, int& bu, int width) {
+        for (int off = width / 2; off >= 1; off >>= 1) {
+            const float ob = __shfl_xor_sync(0xffffffffu, b, off);
+            const int ou = __shfl_xor_sync(0xffffffffu, bu, off);
+            if (ou >= 0 && (ob > b || (ob == b && ou < bu) || bu < 0)) { b = ob; bu = ou; }
+        }
+    };
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        fold(best[r], best_u[r], 32);
+        if (lane == 0) { sm.best[r][tid >> 5] = best[r]; sm.best_u[r][tid >> 5] = best_u[r]; }
+    }
+    __syncthreads();
+    if (tid >= 32) return;
+#pragma unroll 1
+    for (int r = 0; r < R; ++r) {
+        float b = sm.best[r][lane & (kCloseThreads / 32 - 1)];
+        int bu = sm.best_u[r][lane & (kCloseThreads / 32 - 1)];
+        fold(b, bu, kCloseThreads / 32);
+        if (lane == 0) { sm.best[r][0] = b; sm.best_u[r][0] = bu; }
+    }
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(kCloseThreads, 4) assign_close_kernel(
     const UnitDesc* __restrict__ desc, Shape sh, const __nv_bfloat16* __restrict__ K, const float* __restrict__ s, const int32_t* __restrict__ plan,
     const int32_t* __restrict__ seed_rows, const __nv_bfloat16* __restrict__ seed_k, const float* __restrict__ seed_norm, uint8_t* __restrict__ kind,
     int32_t* __restrict__ seed_of, float* __restrict__ sim, int32_t* __restrict__ grp, unsigned long long* __restrict__ mass_fx,
     int32_t* __restrict__ njoin, int32_t* __restrict__ mem_row, int32_t* __restrict__ mem_seed, int max_m, float tau, float eps,
     const int32_t* __restrict__ close, const int32_t* __restrict__ n_close) {
-    __shared__ alignas(16) float row[128];
-    __shared__ float best_w[kCloseThreads / 32];
-    __shared__ int best_uw[kCloseThreads / 32];
+    __shared__ CloseSmem sm;
     pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, n = *n_close, d = sh.d;
-    for (int x = blockIdx.x; x < n; x += gridDim.x) {
-        const int at = close[x];
-        const int u = warp_find_unit(sh.n_units, at, [&](int v) { return (int)desc[v].tok_off; });
-        const UnitDesc& ud = desc[u];
-        const int i = at - (int)ud.tok_off, m = max(0, min(plan[u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
-        __syncthreads();
-        if (tid < d) row[tid] = __bfloat162float(K[row_elem_off(sh, ud, ud.k_off, i) + tid]);
-        __syncthreads();
-        float best = -INFINITY;
-        int best_u = -1;
-        for (int j = tid; j < m; j += kCloseThreads) {
-            const uint4* seed = reinterpret_cast<const uint4*>(seed_k + (size_t)(ud.seed_base + j) * d);
-            const float nu = seed_norm[ud.seed_base + j];
-            float acc = 0.f, n2[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-            for (int c = 0; c < d / 8; ++c) {
-                const uint4 v = seed[c];
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int y = 0; y < 4; ++y) {
-                    const float r0 = row[8 * c + 2 * y], r1 = row[8 * c + 2 * y + 1];
-                    n2[(2 * y) & 3] = fmaf(r0, r0, n2[(2 * y) & 3]);
-                    n2[(2 * y + 1) & 3] = fmaf(r1, r1, n2[(2 * y + 1) & 3]);
-                    acc = fmaf(r0, __uint_as_float(w[y] << 16), acc);
-                    acc = fmaf(r1, __uint_as_float(w[y] & 0xFFFF0000u), acc);
-                }
-            }
-            const float nj = sqrtf((n2[0] + n2[1]) + (n2[2] + n2[3]));
-            const float v = nj > 0.f && nu > 0.f ? acc / (nj * nu) : 0.f;
-            if (v > best) { best = v; best_u = j; }
+    const int step = n > kCloseRows * (int)gridDim.x ? kCloseRows : 1;
+    int run = 0;
+    for (int x0 = blockIdx.x * step, x = x0; x0 < n; x += run) {
+        const int end = min(n, x0 + step);
+        if (x >= end) {
+            x0 += gridDim.x * step;
+            x = x0;
+            run = 0;
+            continue;
         }
-        auto fold = [&](int width) {           // the greatest, the first seed among equals
-            for (int off = width / 2; off >= 1; off >>= 1) {
-                const float ob = __shfl_xor_sync(0xffffffffu, best, off);
-                const int ou = __shfl_xor_sync(0xffffffffu, best_u, off);
-                if (ou >= 0 && (ob > best || (ob == best && ou < best_u) || best_u < 0)) { best = ob; best_u = ou; }
-            }
-        };
-        fold(32);
-        if (lane == 0) { best_w[tid >> 5] = best; best_uw[tid >> 5] = best_u; }
+        // the rows of the first one's unit
+        const int listed = close[min(x + (lane & (kCloseRows - 1)), end - 1)];
+        const int u = warp_find_unit(sh.n_units, __shfl_sync(0xffffffffu, listed, 0), [&](int v) { return (int)desc[v].tok_off; });
+        const UnitDesc& ud = desc[u];
+        const int tok_off = (int)ud.tok_off, T = ud.T, m = max(0, min(plan[u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
+        run = __ffs(~__ballot_sync(0xffffffffu, lane < kCloseRows && x + lane < end && listed >= tok_off && listed < tok_off + T)) - 1;
         __syncthreads();
-        if (tid >= 32) continue;
-        best = best_w[lane & (kCloseThreads / 32 - 1)];
-        best_u = best_uw[lane & (kCloseThreads / 32 - 1)];
-        fold(kCloseThreads / 32);
-        if (lane != 0) continue;
+        for (int e = tid; e < (run > 1 ? kCloseRows : 1) * 128; e += kCloseThreads) {
+            const int r = e >> 7, c = e & 127;
+            if (c < d) sm.row[r][c] = r < run ? __bfloat162float(K[row_elem_off(sh, ud, ud.k_off, close[x + r] - tok_off) + c]) : 0.f;
+        }
+        __syncthreads();
+        if (run > 1) close_best<kCloseRows>(sm, seed_k, seed_norm, ud.seed_base, m, d);
+        else close_best<1>(sm, seed_k, seed_norm, ud.seed_base, m, d);
+        if (tid >= run) continue;
+        const float best = sm.best[tid][0];
+        const int best_u = sm.best_u[tid][0], at = close[x + tid], i = at - tok_off;
         if (sim) sim[at] = best;
         const unsigned long long fx = mass_to_fx(row_mass(sh, s, eps, at));
         const bool joined = best_u >= 0 && best >= tau;
@@ -1007,9 +1067,9 @@ __global__ void __launch_bounds__(kCloseThreads) assign_close_kernel(
         seed_of[at] = seed_rows[ud.seed_base + CASK_IDX(best_u, m, sh.err)];
         grp[at] = best_u;
         const int p = atomicAdd(&njoin[u], 1);
-        if (mem_row && p < ud.T) {
-            mem_row[ud.tok_off + p] = i;
-            mem_seed[ud.tok_off + p] = best_u;
+        if (mem_row && p < T) {
+            mem_row[tok_off + p] = i;
+            mem_seed[tok_off + p] = best_u;
         }
     }
 }
