@@ -90,6 +90,8 @@ struct Chunk {
     int32_t *close, *n_close;        // [sumT], [1] rows left to assign_close_kernel
 };
 
+constexpr uint8_t kKindClose = 0x80;     // MANY: kind of a listed row until assign_close_kernel has decided it
+
 // Walks this CTA's contiguous range of scratch tiles, unit by unit.
 struct TileWalk {
     const UnitDesc* desc;
@@ -836,7 +838,10 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                         int at = 0;
                         if (lane == 0) at = atomicAdd(chunk.n_close, __popc(ub));
                         at = __shfl_sync(0xffffffffu, at, 0) + __popc(ub & ((1u << lane) - 1u));
-                        if (unsure) chunk.close[at] = (int)(tok_off + i);
+                        if (unsure) {
+                            chunk.close[at] = (int)(tok_off + i);
+                            kind[tok_off + i] = kKindClose;
+                        }
                     }
                     cand = cand && !unsure;
                 }
@@ -941,9 +946,11 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // MANY: the rows whose cosines with two seeds, or with one and tau, lie within what the sums of the tensor cores may be off.  A CTA a row, a
 // thread every 256th seed; the additions are those of assign_simt_kernel.  Bound by latency (list, unit, row, seeds in series), so
 // a seed's row is read 128 bytes at a time.  16 units of 15,276 rows, 380 seeds: 44 us with a warp a row, 15 so.
-// Caches whose rows repeat list nearly all of them; a seed's row then is read once for eight (kCloseRows) rows of a unit, which stand
-// side by side in the list.  240 units of 3,000 rows drawn from 64 keys each (event): 18.7 ms a row at a time, 5.7 so (SIMT kernel 5.1); four of
-// 9,000 2,252 and 714 us (524).  Rows of zeros, whose cosine is 0 without a sum, are not listed: half of the rows 17.1 to 0.68 ms.
+// Caches whose rows repeat list many of them.  A seed's row then is read once for eight (kCloseRows) rows of a unit, which stand side by side
+// in the list, and if more than half of all rows are listed they are taken tile by tile.  Rows drawn from 64 keys (event), 240 units of 3,000
+// 18.7 ms a row at a time, 5.7 eight, 5.6 by tiles (SIMT kernel 5.05); four of 9,000 2,252, 714 and 545 us (523); 104 of 27,043 from 100 keys
+// 21.4 ms eight, 12.3 by tiles (11.3).  Below half the eight are no slower than the tiles.  Rows of zeros, whose cosine is 0 without a
+// sum, are not listed: half of the rows 17.1 to 0.68 ms.
 constexpr int kCloseThreads = 256, kCloseRows = 8, kClosePitch = 132;      // (pitch: 16-byte pieces, and no conflicts where four threads take a row)
 struct CloseSmem {
     alignas(16) float row[kCloseRows][kClosePitch];
@@ -951,8 +958,19 @@ struct CloseSmem {
     float best[kCloseRows][kCloseThreads / 32];
     int best_u[kCloseRows][kCloseThreads / 32];
 };
+constexpr int kCloseTile = 64, kClosePart = 64;      // rows and seeds of a tile; channels of it in shared memory at a time
+struct CloseTile {
+    float row[kCloseTile][kClosePart + 1], seed[kCloseTile][kClosePart + 1], norm[kCloseTile];
+};
 
 // Greatest cosine (the first seed among equals) of the R rows in shared memory, to best[.][0] and best_u[.][0].
+__device__ __forceinline__ void close_fold(float& b, int& bu, int width) {
+    for (int off = width / 2; off >= 1; off >>= 1) {
+        const float ob = __shfl_xor_sync(0xffffffffu, b, off);
+        const int ou = __shfl_xor_sync(0xffffffffu, bu, off);
+        if (ou >= 0 && (ob > b || (ob == b && ou < bu) || bu < 0)) { b = ob; bu = ou; }
+    }
+}
 template <int R>
 __device__ __forceinline__ void close_best(CloseSmem& sm, const __nv_bfloat16* __restrict__ seed_k, const float* __restrict__ seed_norm, int seed_base, int m, int d) {
     const int tid = threadIdx.x, lane = tid & 31;
@@ -998,16 +1016,9 @@ __device__ __forceinline__ void close_best(CloseSmem& sm, const __nv_bfloat16* _
             if (v > best[r]) { best[r] = v; best_u[r] = j; }
         }
     }
-    auto fold = [&](float& b, int& bu, int width) {
-        for (int off = width / 2; off >= 1; off >>= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, b, off);
-            const int ou = __shfl_xor_sync(0xffffffffu, bu, off);
-            if (ou >= 0 && (ob > b || (ob == b && ou < bu) || bu < 0)) { b = ob; bu = ou; }
-        }
-    };
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        fold(best[r], best_u[r], 32);
+        close_fold(best[r], best_u[r], 32);
         if (lane == 0) { sm.best[r][tid >> 5] = best[r]; sm.best_u[r][tid >> 5] = best_u[r]; }
     }
     __syncthreads();
@@ -1016,7 +1027,7 @@ __device__ __forceinline__ void close_best(CloseSmem& sm, const __nv_bfloat16* _
     for (int r = 0; r < R; ++r) {
         float b = sm.best[r][lane & (kCloseThreads / 32 - 1)];
         int bu = sm.best_u[r][lane & (kCloseThreads / 32 - 1)];
-        fold(b, bu, kCloseThreads / 32);
+        close_fold(b, bu, kCloseThreads / 32);
         if (lane == 0) { sm.best[r][0] = b; sm.best_u[r][0] = bu; }
     }
     __syncwarp();
@@ -1027,10 +1038,100 @@ __global__ void __launch_bounds__(kCloseThreads, 4) assign_close_kernel(
     const int32_t* __restrict__ seed_rows, const __nv_bfloat16* __restrict__ seed_k, const float* __restrict__ seed_norm, uint8_t* __restrict__ kind,
     int32_t* __restrict__ seed_of, float* __restrict__ sim, int32_t* __restrict__ grp, unsigned long long* __restrict__ mass_fx,
     int32_t* __restrict__ njoin, int32_t* __restrict__ mem_row, int32_t* __restrict__ mem_seed, int max_m, float tau, float eps,
-    const int32_t* __restrict__ close, const int32_t* __restrict__ n_close) {
-    __shared__ CloseSmem sm;
+    const int32_t* __restrict__ close, const int32_t* __restrict__ n_close, int total_tiles, int sub_rows) {
+    __shared__ union { CloseSmem list; CloseTile tile; } both;
+    CloseSmem& sm = both.list;
     pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, n = *n_close, d = sh.d;
+    auto finish = [&](const UnitDesc& ud, int u, int m, int i, float best, int best_u) {
+        const int64_t at = ud.tok_off + i;
+        if (sim) sim[at] = best;
+        const unsigned long long fx = mass_to_fx(row_mass(sh, s, eps, at));
+        const bool joined = best_u >= 0 && best >= tau;
+        atomicAdd(&mass_fx[(size_t)u * (max_m + 1) + (joined ? best_u : max_m)], fx);
+        kind[at] = joined ? CASK_KIND_MERGED : CASK_KIND_DROPPED;
+        if (!joined) return;
+        seed_of[at] = seed_rows[ud.seed_base + CASK_IDX(best_u, m, sh.err)];
+        grp[at] = best_u;
+        const int p = atomicAdd(&njoin[u], 1);
+        if (mem_row && p < ud.T) {
+            mem_row[ud.tok_off + p] = i;
+            mem_seed[ud.tok_off + p] = best_u;
+        }
+    };
+    if (n > total_tiles * (kTileRows / 2)) {
+        // more than half of all rows: tile by tile, as assign_simt_kernel goes
+        CloseTile& sm = both.tile;
+        const int ty = tid / 16, tx = tid % 16;
+        for (int w = blockIdx.x; w < total_tiles * (kTileRows / kCloseTile); w += gridDim.x) {
+            const int g = w / (kTileRows / kCloseTile);
+            const int u = warp_find_unit(sh.n_units, g, [&](int v) { return desc[v].atile0; });
+            const UnitDesc& ud = desc[u];
+            const int P = ud.P, m = max(0, min(plan[u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M])), hi = ud.T - max(0, min(plan[u * 8 + CASK_PLAN_R], ud.T - P));
+            const int lo = P - (sh.page_size ? P % sub_rows : 0) + (g - ud.atile0) * kTileRows + w % (kTileRows / kCloseTile) * kCloseTile;
+            auto listed = [&](int r) { return lo + r >= P && lo + r < hi && kind[ud.tok_off + lo + r] == kKindClose; };
+            if (!__syncthreads_or(tid < kCloseTile && listed(tid))) continue;
+            auto clamped = [&](int r) { return row_elem_off(sh, ud, ud.k_off, max(0, min(lo + r, ud.T - 1))); };
+            {
+                const __nv_bfloat16* k = K + clamped(tid / 4);
+                float n2 = 0.f;
+                for (int c = tid & 3; c < d; c += 4) n2 = fmaf(__bfloat162float(k[c]), __bfloat162float(k[c]), n2);
+                n2 += __shfl_xor_sync(0xffffffffu, n2, 1);
+                n2 += __shfl_xor_sync(0xffffffffu, n2, 2);
+                if ((tid & 3) == 0) sm.norm[tid / 4] = sqrtf(n2);
+            }
+            float best[4];
+            int best_u[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) { best[a] = -INFINITY; best_u[a] = -1; }
+            for (int u0 = 0; u0 < m; u0 += kCloseTile) {
+                float acc[4][4] = {};
+                for (int c0 = 0; c0 < d; c0 += kClosePart) {
+                    const int vecs = min(kClosePart, d - c0) / 8;
+                    __syncthreads();
+                    for (int e = tid; e < 2 * kCloseTile * vecs; e += kCloseThreads) {
+                        const int r = e / vecs % kCloseTile, c = e % vecs * 8;
+                        const bool of_row = e < kCloseTile * vecs;
+                        const uint4 v = *reinterpret_cast<const uint4*>((of_row ? K + clamped(r) : seed_k + (size_t)(ud.seed_base + min(u0 + r, m - 1)) * d) + c0 + c);
+                        const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+                        float* to = (of_row ? sm.row[r] : sm.seed[r]) + c;
+#pragma unroll
+                        for (int y = 0; y < 8; ++y) to[y] = __uint_as_float(y & 1 ? x[y >> 1] & 0xFFFF0000u : x[y >> 1] << 16);
+                    }
+                    __syncthreads();
+#pragma unroll 4
+                    for (int c = 0; c < 8 * vecs; ++c) {
+                        float sa[4], rb[4];
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) { sa[a] = sm.row[ty + 16 * a][c]; rb[a] = sm.seed[tx + 16 * a][c]; }
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(sa[a], rb[b], acc[a][b]);
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const int j = u0 + tx + 16 * b;
+                    if (j >= m) continue;
+                    const float nu = seed_norm[ud.seed_base + j];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        const float nj = sm.norm[ty + 16 * a];
+                        const float v = nj > 0.f && nu > 0.f ? acc[a][b] / (nj * nu) : 0.f;
+                        if (v > best[a]) { best[a] = v; best_u[a] = j; }
+                    }
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                close_fold(best[a], best_u[a], 16);
+                if (tx == 0 && listed(ty + 16 * a)) finish(ud, u, m, lo + ty + 16 * a, best[a], best_u[a]);
+            }
+            __syncthreads();
+        }
+        return;
+    }
     const int step = n > kCloseRows * (int)gridDim.x ? kCloseRows : 1;
     int run = 0;
     for (int x0 = blockIdx.x * step, x = x0; x0 < n; x += run) {
@@ -1055,22 +1156,7 @@ __global__ void __launch_bounds__(kCloseThreads, 4) assign_close_kernel(
         __syncthreads();
         if (run > 1) close_best<kCloseRows>(sm, seed_k, seed_norm, ud.seed_base, m, d);
         else close_best<1>(sm, seed_k, seed_norm, ud.seed_base, m, d);
-        if (tid >= run) continue;
-        const float best = sm.best[tid][0];
-        const int best_u = sm.best_u[tid][0], at = close[x + tid], i = at - tok_off;
-        if (sim) sim[at] = best;
-        const unsigned long long fx = mass_to_fx(row_mass(sh, s, eps, at));
-        const bool joined = best_u >= 0 && best >= tau;
-        atomicAdd(&mass_fx[(size_t)u * (max_m + 1) + (joined ? best_u : max_m)], fx);
-        if (!joined) continue;
-        kind[at] = CASK_KIND_MERGED;
-        seed_of[at] = seed_rows[ud.seed_base + CASK_IDX(best_u, m, sh.err)];
-        grp[at] = best_u;
-        const int p = atomicAdd(&njoin[u], 1);
-        if (mem_row && p < T) {
-            mem_row[tok_off + p] = i;
-            mem_seed[tok_off + p] = best_u;
-        }
+        if (tid < run) finish(ud, u, m, close[x + tid] - tok_off, sm.best[tid][0], sm.best_u[tid][0]);
     }
 }
 
@@ -1153,7 +1239,7 @@ cudaError_t launch_assign_tc(const Launch& L, const cask_params& prm, const floa
     Timed t(L, KID_ASSIGN);
     return launch_dependent(L.stream, assign_close_kernel, close_grid, kCloseThreads, spread_smem(L, close_grid, fixed, 0), L.desc, sh, (const __nv_bfloat16*)L.k, s, plan,
                             ws.seed_rows, (const __nv_bfloat16*)ws.seed_k, ws.seed_norm, kind, seed_of, sim, ws.grp, ws.mass_fx, ws.njoin,
-                            ws.slot_lists ? ws.mem_row : nullptr, ws.mem_slot, L.max_m, prm.tau, prm.eps, ws.close, ws.err + 4);
+                            ws.slot_lists ? ws.mem_row : nullptr, ws.mem_slot, L.max_m, prm.tau, prm.eps, ws.close, ws.err + 4, L.total_atiles, sub_rows);
 }
 
 }  // namespace cask

@@ -95,14 +95,21 @@ def test_equal_and_empty_rows():
     _compare(hb, change=nan_row)
 
 
-@pytest.mark.parametrize("units,head_dim,distinct", [(12, 128, 40), (160, 128, 300), (24, 72, 1000)])
-def test_more_uncertain_rows_than_there_are_blocks(units, head_dim, distinct):
-    """Nearly every row repeats: several rows of a unit are decided at a time, in runs that end where the list goes on with another unit."""
-    hb = _batch(units=units, head_dim=head_dim, decode=1500 if units < 100 else 900, budget=800 if units < 100 else 700, reserve=700 if units < 100 else 650)
+@pytest.mark.parametrize("units,head_dim,distinct,decode,budget,page", [
+    (12, 128, 40, 1500, 800, 0),         # runs of rows from the list
+    (160, 128, 300, 900, 700, 0),
+    (24, 72, 1000, 1500, 800, 0),
+    (12, 128, 40, 3000, 750, 0),         # more than half of all rows: tile by tile
+    (5, 80, 30, 3011, 750, 64),
+])
+def test_more_uncertain_rows_than_there_are_blocks(units, head_dim, distinct, decode, budget, page):
+    """Nearly every row repeats: several rows of a unit are decided at a time, in runs that end where the list goes on with another unit, or
+    whole tiles."""
+    hb = _batch(units=units, head_dim=head_dim, decode=decode, budget=budget, reserve=budget - 50 if decode < 1000 else 700)
     T = int(hb.T[0])
     k = hb.k.reshape(units, T, -1)
     rng = np.random.default_rng(units)
     for u in range(units):
         k[u, 100:] = k[u, 100 + rng.integers(0, distinct, T - 100)]
-    a = _compare(hb)
+    a = _compare(hb, page)
     assert a["plan"][:, 5].min() > 256
