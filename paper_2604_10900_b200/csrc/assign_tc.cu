@@ -963,7 +963,7 @@ struct CloseTile {
     float row[kCloseTile][kClosePart + 1], seed[kCloseTile][kClosePart + 1], norm[kCloseTile];
 };
 
-// Greatest cosine (the first seed among equals) of the R rows in shared memory, to best[.][0] and best_u[.][0].
+// The greatest of `width` lanes, the first seed among equals.
 __device__ __forceinline__ void close_fold(float& b, int& bu, int width) {
     for (int off = width / 2; off >= 1; off >>= 1) {
         const float ob = __shfl_xor_sync(0xffffffffu, b, off);
@@ -971,6 +971,7 @@ __device__ __forceinline__ void close_fold(float& b, int& bu, int width) {
         if (ou >= 0 && (ob > b || (ob == b && ou < bu) || bu < 0)) { b = ob; bu = ou; }
     }
 }
+// Greatest cosine (the first seed among equals) of the R rows in shared memory, to best[.][0] and best_u[.][0].
 template <int R>
 __device__ __forceinline__ void close_best(CloseSmem& sm, const __nv_bfloat16* __restrict__ seed_k, const float* __restrict__ seed_norm, int seed_base, int m, int d) {
     const int tid = threadIdx.x, lane = tid & 31;
