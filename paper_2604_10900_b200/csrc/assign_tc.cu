@@ -773,6 +773,11 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (MANY && c0 > 0 && in_range) {
                     carried = chunk.best[tok_off + i];
                     carried_u = chunk.best_u[tok_off + i];
+                    // (a launch that gave up a wait has written nothing here: what the workspace held before it is no seed)
+                    if ((unsigned)carried_u >= (unsigned)c0) {
+                        carried = make_float2(-INFINITY, -INFINITY);
+                        carried_u = -1;
+                    }
                 }
                 kd_n = (uint8_t)CASK_KIND_RECENT; s_n = 0.f; mi_n = 0.f;
                 if (pre) {

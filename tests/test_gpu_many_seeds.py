@@ -19,6 +19,7 @@ def _compare(hb, page=0, change=None, **kw):
     slow = simt.cb.params(score_path=1, **kw)
     outs = []
     for run, prm in ((tc, tc.prm), (simt, slow)):
+        run.ws.fill_(0x7f)      # what a workspace held before is no value, seed or row of this call
         o, args = run.out, (run.ctx, run.batch)
         ws = (run.ws, run.ws_bytes)
         run.cb.cask_score(*args, run.prm, o["s"], o["lse"], *ws)
