@@ -1149,20 +1149,22 @@ __global__ void __launch_bounds__(kCloseThreads, 4) assign_close_kernel(
             continue;
         }
         // the rows of the first one's unit
-        const int listed = close[min(x + (lane & (kCloseRows - 1)), end - 1)];
+        const UnitDesc& last_unit = desc[sh.n_units - 1];
+        const int listed = CASK_IDX(close[min(x + (lane & (kCloseRows - 1)), end - 1)], (int)last_unit.tok_off + last_unit.T, sh.err);
         const int u = warp_find_unit(sh.n_units, __shfl_sync(0xffffffffu, listed, 0), [&](int v) { return (int)desc[v].tok_off; });
         const UnitDesc& ud = desc[u];
         const int tok_off = (int)ud.tok_off, T = ud.T, m = max(0, min(plan[u * 8 + CASK_PLAN_M], ud.plan[CASK_PLAN_M]));
-        run = __ffs(~__ballot_sync(0xffffffffu, lane < kCloseRows && x + lane < end && listed >= tok_off && listed < tok_off + T)) - 1;
+        // (one at least, so that the loop goes on whatever the list holds)
+        run = max(1, __ffs(~__ballot_sync(0xffffffffu, lane < kCloseRows && x + lane < end && listed >= tok_off && listed < tok_off + T)) - 1);
         __syncthreads();
         for (int e = tid; e < (run > 1 ? kCloseRows : 1) * 128; e += kCloseThreads) {
             const int r = e >> 7, c = e & 127;
-            if (c < d) sm.row[r][c] = r < run ? __bfloat162float(K[row_elem_off(sh, ud, ud.k_off, close[x + r] - tok_off) + c]) : 0.f;
+            if (c < d) sm.row[r][c] = r < run ? __bfloat162float(K[row_elem_off(sh, ud, ud.k_off, CASK_IDX(close[x + r] - tok_off, T, sh.err)) + c]) : 0.f;
         }
         __syncthreads();
         if (run > 1) close_best<kCloseRows>(sm, seed_k, seed_norm, ud.seed_base, m, d);
         else close_best<1>(sm, seed_k, seed_norm, ud.seed_base, m, d);
-        if (tid < run) finish(ud, u, m, close[x + tid] - tok_off, sm.best[tid][0], sm.best_u[tid][0]);
+        if (tid < run) finish(ud, u, m, CASK_IDX(close[x + tid] - tok_off, T, sh.err), sm.best[tid][0], sm.best_u[tid][0]);
     }
 }
 

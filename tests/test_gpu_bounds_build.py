@@ -35,6 +35,11 @@ def _cases():
     yield "bf16_tensor_path", r8k.with_(layers=1, kv_heads=2, decode=1024 + 19), {}
     yield "bf16_paged", r8k.with_(layers=1, kv_heads=2, decode=900), dict(page_size=16)
     yield "bf16_many_seeds", wl.WORKLOADS["reasoning32k_b1024"].with_(layers=1, kv_heads=1, decode=3000), {}
+    many = r8k.with_(layers=1, group=4, window=32, prefix=100, budget=800, reserve=700)      # 334 seeds a unit
+    yield "more_than_256_seeds", many.with_(kv_heads=2, decode=1500), {}
+    yield "more_than_256_seeds_paged", many.with_(kv_heads=2, decode=5000), dict(page_size=16)
+    yield "rows_of_few_keys", many.with_(kv_heads=12, decode=1500), dict(distinct=40)
+    yield "most_rows_of_few_keys", many.with_(kv_heads=12, decode=3000), dict(distinct=40)
     yield "slot_lists", r8k.with_(layers=1, kv_heads=3, decode=5000, budget=200, reserve=120), {}
     yield "slot_lists_given_up", r8k.with_(layers=1, kv_heads=2, decode=5000, budget=200, reserve=120), dict(tau=-1.0, page_size=64)
     yield "thousands_of_members", r8k.with_(layers=1, kv_heads=2, decode=3000), dict(tau=-1.0)
@@ -64,6 +69,11 @@ def test_every_index_check_stays_silent_and_the_results_are_the_ordinary_builds(
     try:
         for name, w, kw in _cases():
             hb = wl.make_batch(w)
+            distinct = kw.pop("distinct", 0)                 # every unit's decode rows drawn from so many of its keys
+            if distinct:
+                k, rng = hb.k.reshape(hb.n_units, int(hb.T[0]), -1), np.random.default_rng(distinct)
+                for u in range(hb.n_units):
+                    k[u, w.prefix:] = k[u, w.prefix + rng.integers(0, distinct, w.decode)]
             cb.use_library(None)
             g0, b0, f0 = _event(hb, kw)
             cb.use_library(cbuild.LIB_BOUNDS)
@@ -75,4 +85,4 @@ def test_every_index_check_stays_silent_and_the_results_are_the_ordinary_builds(
             ran += 1
     finally:
         cb.use_library(None)
-    assert ran >= 19
+    assert ran >= 23
