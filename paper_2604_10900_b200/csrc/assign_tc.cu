@@ -22,7 +22,7 @@
 //
 // More than 256 seeds (MANY): their columns are taken in chunks of at most 128, a launch each, with four buffers.  A row's greatest and second
 // greatest value and the former's seed go from launch to launch through the workspace; the launch with a unit's last chunk finishes its
-// rows.  Rows that the sums of the tensor cores cannot tell (see kClose) are listed, and assign_close_kernel decides them by the sums of
+// rows.  Rows that the sums of the tensor cores cannot tell (see kCloseSeeds) are listed, and assign_close_kernel decides them by the sums of
 // assign_simt_kernel, which served these shapes before: a row goes where that kernel sends it.  Chunks of 128 and four buffers, not of
 // 256 and two: a pass of the former takes half of one of the latter (0.44 and 0.87 ms for 9.6 M rows).  Event of 16 units of 15,276 rows
 // (380 seeds) 1,283 to 250 us, 104 of 27,043 (270) 11,242 to 1,377, 4 of 9,000 (860) 517 to 204, 8 of 1,024 (434) 155 to 88, one of
@@ -294,10 +294,17 @@ __device__ __forceinline__ int find_seed(uint32_t taddr, const float* inv, int c
 }
 
 // fp32 rows whose best cosine is within kClose of another seed's or of tau are decided by the sums assign_simt_kernel takes, one
-// multiply-add after the other in the order of the channels.  A cosine of the two kernels differs by up to 1.2e-6 (768,000 of them;
-// a sum of 128 products is off by 7.6e-6 if all its roundings go one way), so two seeds 7.6e-6 apart come out in the same order
-// either way.  Without this, one event of 16 units of 8,448 rows in eight sent a row to another seed.
+// multiply-add after the other in the order of the channels.  A margin, not a bound: the two kernels' cosines differ by up to 1.2e-6 (768,000
+// of them), so two seeds 7.6e-6 apart come out in the same order either way unless the keys are made for it (see kCloseSeeds).  Without
+// this, one event of 16 units of 8,448 rows in eight sent a row to another seed.
 constexpr float kClose = 1.f / 131072.f;
+// bf16 rows, MANY.  The plain sum of 128 products rounds 127 times by at most 2^-24 of the norms' product: 7.6e-6.  The tensor cores' sum lacks
+// at most 4.8e-6: a product is cut at 2^-25 of the greatest magnitude of its step (keys of one great channel and 120 equal small ones show it,
+// product by product), a step's sum at 2^-23.  Between the kernels two cosines may so move by 2.5e-5 against one another and one
+// by 1.25e-5 against tau, where the row's norm adds 1e-6.  The greatest difference of one cosine over twelve kinds of keys, 168,000 rows each
+// (normal, channels of 8 and 800 times the rest, log-normal, all positive, near one another), is 3.3e-6, but keys can be made of which a margin of
+// 7.6e-6 sends a row elsewhere.
+constexpr float kCloseSeeds = 3.5f / 131072.f, kCloseTau = 2.f / 131072.f;
 
 // Of the seeds marked in `close` the one of greatest plain cosine, the first among equals; its cosine in sm.  Four seeds at a time.  The
 // loops stay rolled: the code runs once or twice a CTA, and fetching its instructions takes longer than they do.
@@ -836,8 +843,10 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (MANY && n2 == 0.f && m_all > 0) { best = 0.f; best_u = 0; }        // a row of zeros: cosine 0 with every seed, nothing to tell apart
                 bool cand = in_range && (late ? best > -INFINITY : best_u >= 0) && kd == CASK_KIND_DROPPED;
                 if (MANY) {
-                    const float nj = sqrtf(n2), by = kClose * nj;
-                    const bool unsure = in_range && m_all > 0 && n2 != 0.f && kd == CASK_KIND_DROPPED && !(best_u >= 0 && second < best - by && fabsf(best - tau * nj) > by);
+                    // (a row that certainly stays below tau goes to no seed, whichever is the nearest)
+                    const float nj = sqrtf(n2), at_tau = tau * nj, by = kCloseTau * nj;
+                    const bool unsure = in_range && m_all > 0 && n2 != 0.f && kd == CASK_KIND_DROPPED &&
+                                        !(best_u >= 0 && (best < at_tau - by || (best > at_tau + by && second < best - kCloseSeeds * nj)));
                     const unsigned ub = __ballot_sync(0xffffffffu, unsure);
                     if (ub) {
                         int at = 0;

@@ -9,7 +9,7 @@ from paper_2604_10900_b200 import workloads as wl
 pytestmark = pytest.mark.gpu
 
 
-def _compare(hb, page=0, change=None, **kw):
+def _compare(hb, page=0, change=None, scores=None, **kw):
     import gpu_harness as gh
     import torch
     tc, simt = (gh.GpuRun(hb, page_size=page, **kw) for _ in range(2))
@@ -23,6 +23,8 @@ def _compare(hb, page=0, change=None, **kw):
         o, args = run.out, (run.ctx, run.batch)
         ws = (run.ws, run.ws_bytes)
         run.cb.cask_score(*args, run.prm, o["s"], o["lse"], *ws)
+        if scores is not None:
+            o["s"].copy_(torch.from_numpy(scores))
         run.cb.cask_prefix_evict(*args, run.prm, o["s"], o["kind"], o["plan"], *ws)
         run.cb.cask_select_core(*args, run.prm, o["s"], o["plan"], o["kind"], *ws)
         run.cb.cask_consolidate_scratch(*args, prm, o["s"], o["plan"], o["kind"], o["seed_of"], o["weight"], o["sim"], o["unit_status"], o["lost_mass"], *ws)
@@ -35,7 +37,7 @@ def _compare(hb, page=0, change=None, **kw):
             assert np.abs(a["sim"] - b["sim"]).max() <= 2 * 128 * 2.0 ** -24
         else:
             assert np.array_equal(a[name].view(np.uint8), b[name].view(np.uint8)), name
-    if page == 0 and not change:
+    if page == 0 and not change and scores is None:
         ev = gh.GpuRun(hb, **kw)
         e = ev.event()
         for name in ("kind", "seed_of", "lost_mass"):
@@ -114,3 +116,23 @@ def test_more_uncertain_rows_than_there_are_blocks(units, head_dim, distinct, de
         k[u, 100:] = k[u, 100 + rng.integers(0, distinct, T - 100)]
     a = _compare(hb, page)
     assert a["plan"][:, 5].min() > 256
+
+
+def test_near_seeds_whose_plain_sums_round_apart():
+    """A row of cosines 1.28e-5 apart with two seeds, the products with one rounded up at every addition of the plain sum and those with the
+    other lost: the plain sums order the seeds the other way round than the cosines, by 1.4e-6."""
+    hb = _batch(units=2)
+    T, eps = int(hb.T[0]), 2.0 ** -12
+
+    def key(x, rest):
+        v = np.zeros(128, np.float32)
+        v[0], v[1:121], v[121:] = 1, x, rest
+        u = v.view(np.uint32)
+        return ((u + 0x7FFF + ((u >> 16) & 1)) >> 16).astype(np.uint16)
+    row, rounded, lost = key(eps, 0), key(eps * (1 + 2.0 ** -7), (1.28e-5 / 3.5) ** 0.5), key(eps * (1 - 2.0 ** -8), 0)
+    k = hb.k.reshape(2, T, -1)
+    k[:, 900:1300] = row
+    k[0, 500], k[0, 600] = rounded, lost            # among the seeds, decode rows 334 to 667 in the order of the scores
+    k[1, 500], k[1, 600] = lost, rounded
+    a = _compare(hb, scores=np.tile(np.linspace(1, 0.1, T, dtype=np.float32), 2))
+    assert (a["seed_of"].reshape(2, T)[0, 900:1300] == 500).all() and (a["seed_of"].reshape(2, T)[1, 900:1300] == 600).all()
