@@ -498,7 +498,9 @@ __device__ __forceinline__ float channel(const Words<N>& p, int x) {
 //     a time whatever slots they feed: eight where a lane's piece of a row is one word, else four (eight of two words spill, and cost eight
 //     units of 33,280 rows 2 us).  Where the rows lie and what they count goes through shared memory: by shuffles, six a row, a member took
 //     0.24 us of a group's time, now 0.15 (128 units of 4,608 rows at head_dim 64, kernel alone 31.2 to 27.5; 8 of 9,000 29.1 to 24.1; 240 of
-//     1,024 whose other rows all join 69.4 to 64.6).  They come first: a group is a chain of memory latencies, three and one more per
+//     1,024 whose other rows all join 69.4 to 64.6).  But by shuffles for the other head dims (CH == 0), whose loads follow each row's place:
+//     100 units of 5,000 rows at head_dim 96, kernel alone 55.6 to 68.7 through shared memory, 361 to 462 where all other rows join;
+//     8 at 80 27.1 to 29.3.  They come first: a group is a chain of memory latencies, three and one more per
 //     kRows members.
 //   * batches of consecutive slots: bulk copies of the rows of the other ones into the warp's staging buffer, then bulk stores, two
 //     for a batch without merged slots, because consecutive slots are contiguous in the output; two buffers, so the copies of a
@@ -613,11 +615,13 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
                 const float ae = row_mass(sh, in.s, in.eps, o + row);
                 const float mg = __shfl_sync(0xffffffffu, mg_t, sl);
                 const float we = in.fw.s ? ae / mg : in.weight[o + row];
-                __syncwarp();
-                at_k[lane] = ko;
-                at_v[lane] = vo;
-                counts[lane] = make_float2(we, ae);
-                __syncwarp();
+                if (CH > 0) {
+                    __syncwarp();
+                    at_k[lane] = ko;
+                    at_v[lane] = vo;
+                    counts[lane] = make_float2(we, ae);
+                    __syncwarp();
+                }
                 for (int c0 = 0; c0 < n; c0 += kRows) {
                     Piece kr[kRows], vr[kRows];
                     if (CH > 0) {
@@ -633,10 +637,10 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
 #pragma unroll
                     for (int q = 0; q < kRows; ++q) {
                         if (c0 + q >= n) break;
-                        const float wi = counts[c0 + q].x;
-                        msum += counts[c0 + q].y;
-                        const int64_t kq = CH > 0 ? 0 : at_k[c0 + q];
-                        const int64_t vq = CH > 0 ? 0 : at_v[c0 + q];
+                        const float wi = CH > 0 ? counts[c0 + q].x : __shfl_sync(0xffffffffu, we, c0 + q);
+                        msum += CH > 0 ? counts[c0 + q].y : __shfl_sync(0xffffffffu, ae, c0 + q);
+                        const int64_t kq = CH > 0 ? 0 : __shfl_sync(0xffffffffu, ko, c0 + q);
+                        const int64_t vq = CH > 0 ? 0 : __shfl_sync(0xffffffffu, vo, c0 + q);
 #pragma unroll
                         for (int x = 0; x < kPer; ++x) {
                             if (CH > 0) {
@@ -667,7 +671,7 @@ __device__ __forceinline__ void copy_batches(const RowSource<T>& in, int nk, int
         const int n_copied = __popc(__ballot_sync(0xffffffffu, copied));
         // the stores that read this buffer two batches ago must have read it (every lane has groups of its own)
         asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-        if (it == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // (the members' places are written over)
+        if (CH > 0 && it == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // (the members' places are written over)
         if (lane == 0) mbar_expect_tx(&bars[w][st], (uint32_t)n_copied * 2u * row_bytes);
         __syncwarp();
         if (copied) {
