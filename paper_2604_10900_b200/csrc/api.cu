@@ -247,9 +247,10 @@ cudaError_t descriptor_staging(cask_ctx* ctx, size_t n) {
 }
 
 // Validates, builds and uploads the per-unit descriptors, resolves the launch record.  `stage`: pinned room for them that
-// the caller keeps alive until the upload has been read (the slices of a host batch); NULL = the context's own staging.
+// the caller keeps alive until the upload has been read (the slices of a host batch); NULL = the context's own staging.  `scores`: the
+// scoring passes follow.
 int prepare(cask_ctx* ctx, const cask_batch* b, const cask_params* p, void* ws, size_t ws_bytes, Launch& L,
-            Workspace& W, UnitDesc* stage = nullptr) {
+            Workspace& W, UnitDesc* stage = nullptr, bool scores = false) {
     if (!ctx) return CASK_ERR_NULL;
     int rc = check_batch(b, p);
     if (rc != CASK_OK) return rc;
@@ -297,7 +298,8 @@ int prepare(cask_ctx* ctx, const cask_batch* b, const cask_params* p, void* ws, 
     if (own_stage) {
         bool reads_staging = false;
         e = upload_descriptors(ctx->stream, stage, b->n_units, W.desc, W.err,
-                               !b->lse_in || !given_score_long(b->dtype, b->head_dim, b->group * b->window, tile0, ctx->sms), &reads_staging);
+                               !(scores && b->lse_in && b->dtype == CASK_DTYPE_BF16 &&
+                                 given_score_long(b->dtype, b->head_dim, b->group * b->window, tile0, ctx->sms)), &reads_staging);
         if (e == cudaSuccess && reads_staging) {
             e = cudaEventRecord(ctx->staged, ctx->stream);
             ctx->staged_pending = e == cudaSuccess;
@@ -523,7 +525,7 @@ int cask_score(cask_ctx* ctx, const cask_batch* b, const cask_params* p, float* 
     if (!s) return CASK_ERR_NULL;
     Launch L{};
     Workspace W{};
-    int rc = prepare(ctx, b, p, ws, ws_bytes, L, W);
+    int rc = prepare(ctx, b, p, ws, ws_bytes, L, W, nullptr, true);
     if (rc != CASK_OK || b->n_units == 0) return rc;
     return run_score(ctx, L, b, p, s, lse_out, W);
 }
@@ -639,7 +641,7 @@ int cask_compress_event(cask_ctx* ctx, const cask_batch* b, const cask_params* p
         return CASK_ERR_NULL;
     Launch L{};
     Workspace W{};
-    rc = prepare(ctx, b, p, ws, ws_bytes, L, W);
+    rc = prepare(ctx, b, p, ws, ws_bytes, L, W, nullptr, true);
     if (rc != CASK_OK || b->n_units == 0) return rc;
     rc = event_decide(ctx, L, W, b, p, out);
     if (rc != CASK_OK) return rc;

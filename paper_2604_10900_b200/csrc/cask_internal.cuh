@@ -222,7 +222,8 @@ struct Workspace {
 };
 
 // ---- kernels (defined in the .cu files) --------------------------------------
-// Descriptors into the workspace, flag words cleared (upload.cu).  release: the kernel that follows may start beside this one.
+// Descriptors into the workspace, flag words cleared (upload.cu).  release: the kernel that follows may start beside this one (all but a
+// long score pass with given normalisers, see launch_passes).
 // *reads_staging: the kernel still reads `staged` (page-locked).
 cudaError_t upload_descriptors(cudaStream_t stream, const UnitDesc* staged, int n, UnitDesc* dst, int32_t* err, bool release, bool* reads_staging);
 cudaError_t launch_score_simt(const Launch& L, const float* lse_in, float* s, float* lse_out,

@@ -1305,6 +1305,9 @@ cudaError_t launch_passes(const Launch& L, const RowGroups& rg, const CUtensorMa
     // kernel (units of 8,448 rows, 512 query rows).  Longer passes (given_score_long) are launched the same way, but that kernel does not
     // release them, so that they start when it and the last CTAs of the call before are gone, without the 4 us of an ordinary launch:
     // eight units of 33,280 rows 159.9 to 157.2 us (168 beside those CTAs), 288 of 2,000 201.8 to 198.2, 112 of 4,608 121.6 to 119.1.
+    // fp32: the kernel before is split_rows_kernel, which releases the pass however long.  With an ordinary launch and so (event): 16 units
+    // of 8,448 rows (512 query rows) 197 and 190 us, 12 with 1,024 rows 218 and 212; 24 of them, or 40 with 512 rows, within the 3 % that the
+    // runs differ by.  Not released by that kernel: the same.
     // Behind the normaliser pass it has its first keys, queries and contractions done and its code fetched by the end of that pass
     // (`ahead`): events of 8 units of 640 rows 54.0 to 49.9 us (0.3 tiles a CTA), two fp32 ones of 1,024 52.1 to 50.0, 128 of 4,608 at
     // head_dim 64 (31 tiles) 182 to 176; 24 to 60 tiles 0.5 to 2.5 % (100 units of 11,366 rows 485.7 to 479.4), 90 to 200 up to 1.5, 250 and
