@@ -960,11 +960,14 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // MANY: the rows whose cosines with two seeds, or with one and tau, lie within what the sums of the tensor cores may be off.  A CTA a row, a
 // thread every 256th seed; the additions are those of assign_simt_kernel.  Bound by latency (list, unit, row, seeds in series), so
 // a seed's row is read 128 bytes at a time.  16 units of 15,276 rows, 380 seeds: 44 us with a warp a row, 15 so.
-// Caches whose rows repeat list many of them.  A seed's row then is read once for eight (kCloseRows) rows of a unit, which stand side by side
-// in the list, and if more than half of all rows are listed they are taken tile by tile.  Rows drawn from 64 keys (event), 240 units of 3,000
-// 18.7 ms a row at a time, 5.7 eight, 5.6 by tiles (SIMT kernel 5.05); four of 9,000 2,252, 714 and 545 us (523); 104 of 27,043 from 100 keys
-// 21.4 ms eight, 12.3 by tiles (11.3).  Below half the eight are no slower than the tiles.  Rows of zeros, whose cosine is 0 without a
-// sum, are not listed: half of the rows 17.1 to 0.68 ms.
+// Caches whose rows repeat list many of them where tau lets them join: a copy of a seed is as near to a row as the seed.  A seed's row then is read
+// once for eight (kCloseRows) rows of a unit, which stand side by side in the list, and if more than a quarter of all rows are listed
+// they are taken tile by tile, four rows by four seeds a thread and 16 bytes of each from shared memory at a time, in parts of at most 80 channels.
+// Kernels of the assignment in us, element by element in parts of 64 and so, in brackets the SIMT kernel that these shapes had before: 104 units of
+// 27,000 rows drawn from 64 keys (tau -1, 270 seeds) 12,850 and 10,640 (12,020), 240 of 3,000 (0.3, 750) 5,630 and 5,160 (5,790), four of
+// 9,000 615 and 529 (539), 104 of 7,000 at head_dim 72 2,100 and 1,745 (1,776), at 96 2,630 and 2,210 (2,270).  The line: with a third to a half of
+// the rows listed, eight at a time and by tiles, 104 of 7,000 at head_dim 72 2,310 and 1,790; with a sixth 104 of 27,000 7,910 and 10,560.  Rows of
+// zeros, whose cosine is 0 without a sum, are not listed: half of the rows 17.1 to 0.68 ms.
 constexpr int kCloseThreads = 256, kCloseRows = 8, kClosePitch = 132;      // (pitch: 16-byte pieces, and no conflicts where four threads take a row)
 struct CloseSmem {
     alignas(16) float row[kCloseRows][kClosePitch];
@@ -972,9 +975,9 @@ struct CloseSmem {
     float best[kCloseRows][kCloseThreads / 32];
     int best_u[kCloseRows][kCloseThreads / 32];
 };
-constexpr int kCloseTile = 64, kClosePart = 64;      // rows and seeds of a tile; channels of it in shared memory at a time
+constexpr int kCloseTile = 64, kClosePart = 80;      // rows and seeds of a tile; channels of it in shared memory at a time
 struct CloseTile {
-    float row[kCloseTile][kClosePart + 1], seed[kCloseTile][kClosePart + 1], norm[kCloseTile];
+    float row[kCloseTile][kClosePart + 4], seed[kCloseTile][kClosePart + 4], norm[kCloseTile];      // (16-byte pieces without conflicts)
 };
 
 // The greatest of `width` lanes, the first seed among equals.
@@ -1074,10 +1077,10 @@ __global__ void __launch_bounds__(kCloseThreads, 4) assign_close_kernel(
             mem_seed[ud.tok_off + p] = best_u;
         }
     };
-    if (n > total_tiles * (kTileRows / 2)) {
-        // more than half of all rows: tile by tile, as assign_simt_kernel goes
+    if (n > total_tiles * (kTileRows / 4)) {
+        // more than a quarter of all rows: tile by tile, as assign_simt_kernel goes
         CloseTile& sm = both.tile;
-        const int ty = tid / 16, tx = tid % 16;
+        const int ty = tid / 16, tx = tid % 16, n_parts = (d + kClosePart - 1) / kClosePart, part = (d / 8 + n_parts - 1) / n_parts * 8;
         for (int w = blockIdx.x; w < total_tiles * (kTileRows / kCloseTile); w += gridDim.x) {
             const int g = w / (kTileRows / kCloseTile);
             const int u = warp_find_unit(sh.n_units, g, [&](int v) { return desc[v].atile0; });
@@ -1101,28 +1104,29 @@ __global__ void __launch_bounds__(kCloseThreads, 4) assign_close_kernel(
             for (int a = 0; a < 4; ++a) { best[a] = -INFINITY; best_u[a] = -1; }
             for (int u0 = 0; u0 < m; u0 += kCloseTile) {
                 float acc[4][4] = {};
-                for (int c0 = 0; c0 < d; c0 += kClosePart) {
-                    const int vecs = min(kClosePart, d - c0) / 8;
+                for (int c0 = 0; c0 < d; c0 += part) {
+                    const int vecs = min(part, d - c0) / 8;
                     __syncthreads();
                     for (int e = tid; e < 2 * kCloseTile * vecs; e += kCloseThreads) {
                         const int r = e / vecs % kCloseTile, c = e % vecs * 8;
                         const bool of_row = e < kCloseTile * vecs;
                         const uint4 v = *reinterpret_cast<const uint4*>((of_row ? K + clamped(r) : seed_k + (size_t)(ud.seed_base + min(u0 + r, m - 1)) * d) + c0 + c);
-                        const uint32_t x[4] = {v.x, v.y, v.z, v.w};
-                        float* to = (of_row ? sm.row[r] : sm.seed[r]) + c;
-#pragma unroll
-                        for (int y = 0; y < 8; ++y) to[y] = __uint_as_float(y & 1 ? x[y >> 1] & 0xFFFF0000u : x[y >> 1] << 16);
+                        float4* to = reinterpret_cast<float4*>((of_row ? sm.row[r] : sm.seed[r]) + c);
+                        to[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
+                        to[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u), __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xFFFF0000u));
                     }
                     __syncthreads();
-#pragma unroll 4
-                    for (int c = 0; c < 8 * vecs; ++c) {
-                        float sa[4], rb[4];
+#pragma unroll 1
+                    for (int c = 0; c < 8 * vecs; c += 4) {
+                        float4 x[4];
 #pragma unroll
-                        for (int a = 0; a < 4; ++a) { sa[a] = sm.row[ty + 16 * a][c]; rb[a] = sm.seed[tx + 16 * a][c]; }
+                        for (int a = 0; a < 4; ++a) x[a] = *reinterpret_cast<const float4*>(&sm.row[ty + 16 * a][c]);
 #pragma unroll
-                        for (int a = 0; a < 4; ++a)
+                        for (int b = 0; b < 4; ++b) {
+                            const float4 y = *reinterpret_cast<const float4*>(&sm.seed[tx + 16 * b][c]);
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(sa[a], rb[b], acc[a][b]);
+                            for (int a = 0; a < 4; ++a) acc[a][b] = fmaf(x[a].w, y.w, fmaf(x[a].z, y.z, fmaf(x[a].y, y.y, fmaf(x[a].x, y.x, acc[a][b]))));
+                        }
                     }
                 }
 #pragma unroll

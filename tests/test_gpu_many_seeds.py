@@ -136,3 +136,22 @@ def test_near_seeds_whose_plain_sums_round_apart():
     k[1, 500], k[1, 600] = lost, rounded
     a = _compare(hb, scores=np.tile(np.linspace(1, 0.1, T, dtype=np.float32), 2))
     assert (a["seed_of"].reshape(2, T)[0, 900:1300] == 500).all() and (a["seed_of"].reshape(2, T)[1, 900:1300] == 600).all()
+
+
+@pytest.mark.parametrize("units,head_dim,distinct,decode,page", [
+    (12, 128, 40, 3000, 0),          # 64 channels at a time
+    (5, 72, 30, 3011, 64),           # all 72 at a time; a ragged last tile
+    (4, 80, 60, 2000, 0),
+    (3, 120, 25, 1283, 16),          # 64 and 56
+    (3, 8, 20, 1283, 0),             # one piece of a row
+])
+def test_caches_that_repeat_and_a_threshold_that_every_row_passes(units, head_dim, distinct, decode, page):
+    """At tau = -1 every row is as near to a seed as to its copies, so more than a quarter of all rows are listed and go tile by tile."""
+    hb = _batch(units=units, head_dim=head_dim, decode=decode, budget=750)
+    T = int(hb.T[0])
+    k = hb.k.reshape(units, T, -1)
+    rng = np.random.default_rng(units)
+    for u in range(units):
+        k[u, 100:] = k[u, 100 + rng.integers(0, distinct, T - 100)]
+    a = _compare(hb, page, tau=-1.0)
+    assert a["plan"][:, 5].min() > 256 and (a["kind"] == 5).mean() > 0.25
