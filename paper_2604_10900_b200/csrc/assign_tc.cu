@@ -958,8 +958,10 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 }
 
 // MANY: the rows whose cosines with two seeds, or with one and tau, lie within what the sums of the tensor cores may be off.  A CTA a row, a
-// thread every 256th seed; the additions are those of assign_simt_kernel.  Bound by latency (list, unit, row, seeds in series), so
-// a seed's row is read 128 bytes at a time.  16 units of 15,276 rows, 380 seeds: 44 us with a warp a row, 15 so.
+// thread every 256th seed; the additions are those of assign_simt_kernel.  Bound by latency: list, unit, row and seeds in series, and half of
+// the time goes to the fetch of code that runs once, so a seed's row is read 64 bytes at a time (128, twice the code: event of 240
+// units of 3,000 rows with 1,071 of them listed 847 us, so 835; 4 of 9,000, 51 listed, 233 and 227; 8 of 1,024, two listed, 78.9
+// and 78.2).  16 units of 15,276 rows, 380 seeds: 44 us with a warp a row, 15 so.
 // Caches whose rows repeat list many of them where tau lets them join: a copy of a seed is as near to a row as the seed.  A seed's row then is read
 // once for eight (kCloseRows) rows of a unit, which stand side by side in the list, and if more than a quarter of all rows are listed
 // they are taken tile by tile, four rows by four seeds a thread and 16 bytes of each from shared memory at a time, in parts of at most 80 channels.
@@ -1012,7 +1014,7 @@ __device__ __forceinline__ void close_best(CloseSmem& sm, const __nv_bfloat16* _
         float acc[R], n2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int r = 0; r < R; ++r) acc[r] = 0.f;
-#pragma unroll(R == 1 ? 8 : 2)
+#pragma unroll(R == 1 ? 4 : 2)
         for (int c = 0; c < d / 8; ++c) {
             const uint4 v = seed[c];
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
