@@ -155,3 +155,47 @@ def test_caches_that_repeat_and_a_threshold_that_every_row_passes(units, head_di
         k[u, 100:] = k[u, 100 + rng.integers(0, distinct, T - 100)]
     a = _compare(hb, page, tau=-1.0)
     assert a["plan"][:, 5].min() > 256 and (a["kind"] == 5).mean() > 0.25
+
+
+@pytest.mark.parametrize("head_dim,page,kw,tau", [
+    (128, 0, dict(), 0.9),                                             # 334 seeds, three chunks
+    (64, 16, dict(decode=2001, budget=900), 0.3),                      # most rows join
+    (128, 0, dict(decode=6000, budget=652, reserve=600), 0.9),         # longer units: listed slots and rows that join
+])
+def test_events_with_carried_masses_against_the_oracle(head_dim, page, kw, tau):
+    """The whole event, compacted rows and all, and the chunks' launches: this is not the SIMT kernel's path."""
+    import gpu_harness as gh
+    hb = _batch(units=2, head_dim=head_dim, **kw)
+    hb.mass_in = np.random.default_rng(head_dim).uniform(0, 2e-3, int(hb.tok_off[-1])).astype(np.float32)
+    run = gh.GpuRun(hb, page_size=page, tau=tau)
+    run.ctx.profile_enable(True)
+    g = run.event()
+    m = int(g["plan"][:, 5].max())
+    assert m > 256 and run.ctx.profile_read()["assign"]["launches"] == -(-m // 128) + 1 and run.ctx.device_flags() == 0
+    st = gh.compare_event(hb, g, gh.run_oracle(hb, tau=tau), tau=tau)
+    assert st["merged_elems"] > 0 and (g["kind"] == 5).any()
+
+
+@pytest.mark.parametrize("distinct", [0, 40])
+def test_a_host_resident_cache_gives_the_device_events_bytes(distinct):
+    """The list of close rows is emptied by another route there; with rows that repeat it is long, in both of two calls."""
+    import gpu_harness as gh
+    import torch
+    hb = _batch(units=3)
+    if distinct:
+        k, rng = hb.k.reshape(3, int(hb.T[0]), -1), np.random.default_rng(distinct)
+        for u in range(3):
+            k[u, 100:] = k[u, 100 + rng.integers(0, distinct, 1500)]
+    w, run = hb.wl, gh.GpuRun(hb, tau=0.3)
+    run.event()
+    cb = run.cb
+    batch, keep = cb.make_batch(hb.k, hb.v, hb.q, hb.T, hb.P, hb.B, hb.reserve, hb.tok_off, w.head_dim, w.group, w.window, w.dtype)
+    nbytes = cb.cask_host_event_device_bytes(batch, run.prm, run.Bmax)
+    dev = torch.full((nbytes,), 0x7f, dtype=torch.uint8, device="cuda:0")
+    want = {name: t.cpu().view(torch.uint8).numpy() for name, t in run.out.items()}
+    ho = {name: np.zeros(t.cpu().view(torch.uint8).shape, np.uint8) for name, t in run.out.items()}
+    for _ in range(2):
+        cb.cask_compress_event_host(run.ctx, batch, run.prm, cb.make_outputs(ho, run.Bmax), dev, nbytes)
+    assert run.ctx.device_flags() == 0 and (run.out["n_out"].cpu().numpy() == hb.B).all()
+    for name in want:
+        assert np.array_equal(ho[name], want[name]), name

@@ -26,3 +26,19 @@ def test_first_seed_among_equals(m, head_dim, page, units, tau):
     a = _compare(hb, page, tau=tau)
     assert (a["plan"][:, 5] == m).all()
     assert m < 15 or ((a["kind"] == 5).any() and (a["kind"] == 0).any())
+
+
+@pytest.mark.parametrize("m", [96, 200])
+def test_the_reference_is_another_kernel(m):
+    """The two sum 128 products in another order, so that some cosine differs: what is compared above is not one kernel with itself."""
+    import gpu_harness as gh
+    hb = wl.make_batch(wl.WORKLOADS["reasoning8k_b384"].with_(layers=1, kv_heads=3, group=4, window=32, prefix=50, decode=1200, budget=82 + 2 * m, reserve=32 + 2 * m))
+    run = gh.GpuRun(hb)
+    o, args, ws, sims = run.out, (run.ctx, run.batch), (run.ws, run.ws_bytes), []
+    run.cb.cask_score(*args, run.prm, o["s"], o["lse"], *ws)
+    for prm in (run.prm, run.cb.params(score_path=1)):
+        run.cb.cask_prefix_evict(*args, run.prm, o["s"], o["kind"], o["plan"], *ws)
+        run.cb.cask_select_core(*args, run.prm, o["s"], o["plan"], o["kind"], *ws)
+        run.cb.cask_consolidate_scratch(*args, prm, o["s"], o["plan"], o["kind"], o["seed_of"], o["weight"], o["sim"], o["unit_status"], o["lost_mass"], *ws)
+        sims.append(o["sim"].cpu().numpy())
+    assert (o["plan"][:, 5] == m).all() and (sims[0] != sims[1]).any() and np.abs(sims[0] - sims[1]).max() <= 2 * 128 * 2.0 ** -24
