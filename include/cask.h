@@ -166,7 +166,9 @@ typedef struct {
     float* lost_mass;      /* [n_units] sum of a_j over scratch rows that joined nobody       */
     float* s;              /* optional [sumT] scores                                          */
     float* lse;            /* optional [n_units, g, W] natural-log normalisers used           */
-    float* sim;            /* optional [sumT] best cosine similarity of non-seed scratch rows, -2 elsewhere */
+    float* sim;            /* optional [sumT] best cosine similarity of non-seed scratch rows, -2 elsewhere; summed by the
+                              tensor cores or in fp32 by the rows' and seeds' channels in turn, whichever decided the row:
+                              the two are at most 1.5e-5 apart */
     /* optional mass diagnostics of Sec. 2.6, [n_units] each: share of the mass of the B best rows of the
        cache that the protected core (recent + core rows) holds, and that the output slots carry */
     float* rho_core;

@@ -24,9 +24,9 @@
 // greatest value and the former's seed go from launch to launch through the workspace; the launch with a unit's last chunk finishes its
 // rows.  Rows that the sums of the tensor cores cannot tell (see kCloseSeeds) are listed, and assign_close_kernel decides them by the sums of
 // assign_simt_kernel, which served these shapes before: a row goes where that kernel sends it.  Chunks of 128 and four buffers, not of
-// 256 and two: a pass of the former takes half of one of the latter (0.44 and 0.87 ms for 9.6 M rows).  Event of 16 units of 15,276 rows
-// (380 seeds) 1,283 to 250 us, 104 of 27,043 (270) 11,242 to 1,377, 4 of 9,000 (860) 517 to 204, 8 of 1,024 (434) 155 to 88, one of
-// 3,000 (1,386) 251 to 145.
+// 256 and two: a pass of the former takes half of one of the latter (0.44 and 0.87 ms for 9.6 M rows).  Event (512 query rows) of 16 units of
+// 15,276 rows (380 seeds) 1,248 to 250 us, 104 of 27,043 (270) 10,980 to 1,337, 240 of 3,000 (576) 4,829 to 748, 4 of 9,000 (860) 517 to
+// 195, 8 of 1,024 (434) 141 to 75, one of 3,000 (1,386) 303 to 166.
 //
 // fp32 caches (SPLIT): the contraction takes the bf16 parts of the rows and the seeds (split.cu) in six products as the scoring
 // passes do (score_tc.cu), one tile of six 16 KB regions at a time, m <= 128; the row norms come from the split.  What that sum
@@ -818,8 +818,11 @@ assign_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 tc_fence_after();
                 float best = -INFINITY, second = -INFINITY;
                 int best_u = -1;
-                // Few rows join where tau is high: their seeds are looked for afterwards.  (Below, with most rows joining, that is a second way
-                // through all chunks: 112 units of 8,448 rows, tau = 0.3, 65 to 72 us; searched in every chunk 66.)
+                // Few rows join where tau is high: their seeds are looked for afterwards.  Where most join, that is a second way through all chunks:
+                // kernel of 112 units of 8,448 rows of which all join 73 us, searched in every chunk 67; 240 of 2,256 43.5 and 41.5.  How many join
+                // depends on the cache as well, but every way to go by that costs more where few do than it gives back: 288 units of 33,280 rows
+                // with 96 and 64 seeds 424 and 392 us by tau alone, by the joiners of the warp's tile before 442 and 414 (the flag in a register, in
+                // shared memory 462 and 417), by those of the unit so far 455 and 408.
                 const bool late = !SPLIT && !MANY && dual && !wpair && tau >= 0.5f;
                 int best_chunk = 0;
                 if (late) best_value(taddr, inv, mc, best, best_chunk);
