@@ -35,11 +35,6 @@ def _cases():
     yield "bf16_tensor_path", r8k.with_(layers=1, kv_heads=2, decode=1024 + 19), {}
     yield "bf16_paged", r8k.with_(layers=1, kv_heads=2, decode=900), dict(page_size=16)
     yield "bf16_many_seeds", wl.WORKLOADS["reasoning32k_b1024"].with_(layers=1, kv_heads=1, decode=3000), {}
-    many = r8k.with_(layers=1, group=4, window=32, prefix=100, budget=800, reserve=700)      # 334 seeds a unit
-    yield "more_than_256_seeds", many.with_(kv_heads=2, decode=1500), {}
-    yield "more_than_256_seeds_paged", many.with_(kv_heads=2, decode=5000), dict(page_size=16)
-    yield "rows_of_few_keys", many.with_(kv_heads=12, decode=1500), dict(distinct=40)
-    yield "most_rows_of_few_keys", many.with_(kv_heads=12, decode=3000), dict(distinct=40)
     yield "slot_lists", r8k.with_(layers=1, kv_heads=3, decode=5000, budget=200, reserve=120), {}
     yield "slot_lists_given_up", r8k.with_(layers=1, kv_heads=2, decode=5000, budget=200, reserve=120), dict(tau=-1.0, page_size=64)
     yield "thousands_of_members", r8k.with_(layers=1, kv_heads=2, decode=3000), dict(tau=-1.0)
@@ -69,11 +64,6 @@ def test_every_index_check_stays_silent_and_the_results_are_the_ordinary_builds(
     try:
         for name, w, kw in _cases():
             hb = wl.make_batch(w)
-            distinct = kw.pop("distinct", 0)                 # every unit's decode rows drawn from so many of its keys
-            if distinct:
-                k, rng = hb.k.reshape(hb.n_units, int(hb.T[0]), -1), np.random.default_rng(distinct)
-                for u in range(hb.n_units):
-                    k[u, w.prefix:] = k[u, w.prefix + rng.integers(0, distinct, w.decode)]
             cb.use_library(None)
             g0, b0, f0 = _event(hb, kw)
             cb.use_library(cbuild.LIB_BOUNDS)
@@ -85,4 +75,35 @@ def test_every_index_check_stays_silent_and_the_results_are_the_ordinary_builds(
             ran += 1
     finally:
         cb.use_library(None)
-    assert ran >= 23
+    assert ran >= 19
+
+
+def _many_seeds():
+    many = wl.WORKLOADS["reasoning8k_b384"].with_(layers=1, group=4, window=32, prefix=100, budget=800, reserve=700)      # 334 seeds a unit
+    yield many.with_(kv_heads=2, decode=1500), 0, {}
+    yield many.with_(kv_heads=2, decode=5000), 0, dict(page_size=16)
+    yield many.with_(kv_heads=12, decode=1500), 40, dict(tau=0.3)          # rows that repeat, from the list
+    yield many.with_(kv_heads=12, decode=3000), 40, dict(tau=-1.0)         # tile by tile
+
+
+def test_index_checks_of_more_than_256_seeds():
+    from paper_2604_10900_b200 import binding as cb
+    cbuild.build_lib()
+    cbuild.build_lib(bounds=True)
+    try:
+        for w, distinct, kw in _many_seeds():
+            hb = wl.make_batch(w)
+            if distinct:                                     # every unit's decode rows drawn from so many of its keys
+                k, rng = hb.k.reshape(hb.n_units, int(hb.T[0]), -1), np.random.default_rng(distinct)
+                for u in range(hb.n_units):
+                    k[u, w.prefix:] = k[u, w.prefix + rng.integers(0, distinct, w.decode)]
+            cb.use_library(None)
+            g0, b0, f0 = _event(hb, kw)
+            cb.use_library(cbuild.LIB_BOUNDS)
+            g1, b1, f1 = _event(hb, kw)
+            assert f0 == 0 and f1 == 0 and g0["plan"][:, 5].min() > 256, (w.decode, kw, f0, f1)
+            assert not (g1["unit_status"] & (cb.ST_BOUNDS | cb.ST_TIMEOUT)).any()
+            for k in b0:
+                assert np.array_equal(b0[k], b1[k]), (w.decode, kw, k)
+    finally:
+        cb.use_library(None)

@@ -9,7 +9,7 @@ from paper_2604_10900_b200 import workloads as wl
 pytestmark = pytest.mark.gpu
 
 
-def _compare(hb, page=0, change=None, scores=None, **kw):
+def _compare(hb, page=0, change=None, **kw):
     import gpu_harness as gh
     import torch
     tc, simt = (gh.GpuRun(hb, page_size=page, **kw) for _ in range(2))
@@ -19,12 +19,9 @@ def _compare(hb, page=0, change=None, scores=None, **kw):
     slow = simt.cb.params(score_path=1, **kw)
     outs = []
     for run, prm in ((tc, tc.prm), (simt, slow)):
-        run.ws.fill_(0x7f)      # what a workspace held before is no value, seed or row of this call
         o, args = run.out, (run.ctx, run.batch)
         ws = (run.ws, run.ws_bytes)
         run.cb.cask_score(*args, run.prm, o["s"], o["lse"], *ws)
-        if scores is not None:
-            o["s"].copy_(torch.from_numpy(scores))
         run.cb.cask_prefix_evict(*args, run.prm, o["s"], o["kind"], o["plan"], *ws)
         run.cb.cask_select_core(*args, run.prm, o["s"], o["plan"], o["kind"], *ws)
         run.cb.cask_consolidate_scratch(*args, prm, o["s"], o["plan"], o["kind"], o["seed_of"], o["weight"], o["sim"], o["unit_status"], o["lost_mass"], *ws)
@@ -37,7 +34,7 @@ def _compare(hb, page=0, change=None, scores=None, **kw):
             assert np.abs(a["sim"] - b["sim"]).max() <= 2 * 128 * 2.0 ** -24
         else:
             assert np.array_equal(a[name].view(np.uint8), b[name].view(np.uint8)), name
-    if page == 0 and not change and scores is None:
+    if page == 0 and not change:
         ev = gh.GpuRun(hb, **kw)
         e = ev.event()
         for name in ("kind", "seed_of", "lost_mass"):
@@ -118,7 +115,16 @@ def test_more_uncertain_rows_than_there_are_blocks(units, head_dim, distinct, de
     assert a["plan"][:, 5].min() > 256
 
 
-def test_near_seeds_whose_plain_sums_round_apart():
+def _no_seeds(run):
+    run.ws.fill_(0x7f)      # what a workspace held before is no value, seed or row of this call
+
+
+@pytest.mark.parametrize("kw,page", [(dict(), 0), (dict(budget=1400, reserve=1300), 16), (dict(units=160, decode=900, budget=700, reserve=650, head_dim=64), 0)])
+def test_a_workspace_full_of_numbers_that_are_no_seeds(kw, page):
+    _compare(_batch(**kw), page, change=_no_seeds)
+
+
+def test_near_seeds_whose_plain_sums_round_apart(monkeypatch):
     """A row of cosines 1.28e-5 apart with two seeds, the products with one rounded up at every addition of the plain sum and those with the
     other lost: the plain sums order the seeds the other way round than the cosines, by 1.4e-6."""
     hb = _batch(units=2)
@@ -134,7 +140,11 @@ def test_near_seeds_whose_plain_sums_round_apart():
     k[:, 900:1300] = row
     k[0, 500], k[0, 600] = rounded, lost            # among the seeds, decode rows 334 to 667 in the order of the scores
     k[1, 500], k[1, 600] = lost, rounded
-    a = _compare(hb, scores=np.tile(np.linspace(1, 0.1, T, dtype=np.float32), 2))
+    import torch
+    from paper_2604_10900_b200 import binding as cb
+    scores = torch.from_numpy(np.tile(np.linspace(1, 0.1, T, dtype=np.float32), 2))
+    monkeypatch.setattr(cb, "cask_score", lambda ctx, batch, prm, s, *rest: s.copy_(scores))
+    a = _compare(hb, change=_no_seeds)
     assert (a["seed_of"].reshape(2, T)[0, 900:1300] == 500).all() and (a["seed_of"].reshape(2, T)[1, 900:1300] == 600).all()
 
 
